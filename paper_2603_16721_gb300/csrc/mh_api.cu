@@ -249,9 +249,10 @@ struct mh_handle {
     u32 *dCounts = nullptr;               // frontier sizes, one per depth, then work-distribution counters
     Rec *dF[kMaxH] = {};               // frontier of depth l at index l
     u32 cap[kMaxH] = {};
-    unsigned char *dSide[kMaxH] = {};     // per record slot of depth l: sig, lb, lc (incremental rounds)
-    u32 *dGK = nullptr;                   // per gene: uncovered tumors carrying it (incremental rounds)
-    u64 *dCov = nullptr;                  // tumors covered by the last round's winner
+    unsigned char *dSide[kMaxH] = {};     // per record slot of depth l: lb, ub, lc (solve by levels)
+    unsigned char *dLevel = nullptr;      // solve by levels: Level, picks, cover arrays
+    Member *dMem = nullptr;               // its members, two buffers of mcap
+    u32 mcap = 0;
     int *hState = nullptr;                // pinned: state + frontier counts
     void *hRes = nullptr;                 // pinned: a solve's results on their way back
     size_t hRes_bytes = 0;
@@ -275,8 +276,8 @@ struct mh_handle {
             dfree(dF[l], stream);
             dfree(dSide[l], stream);
         }
-        dfree(dGK, stream);
-        dfree(dCov, stream);
+        dfree(dLevel, stream);
+        dfree(dMem, stream);
         pinned_state_put(hState);
         pinned_res_put(hRes, hRes_bytes);
     }
@@ -472,6 +473,32 @@ int ensure_frontier(mh_handle *H, int l, u64 n, bool exact = false)
     return MH_OK;
 }
 
+// Device bytes of a solve by levels: Level, the picks, covsel and cr.
+size_t level_bytes(int Nt)
+{
+    const size_t nt1 = (size_t)std::max(Nt, 1);
+    return 256 + nt1 * (sizeof(Key) + sizeof(int) + sizeof(u16));
+}
+
+// Room for n members of a level (at least 8192 of them, or MH_FRONTIER_MIN_RECORDS).
+int ensure_members(mh_handle *H, u64 n)
+{
+    if (n <= H->mcap) return MH_OK;
+    u64 least = 1u << 13;
+    const char *mn = getenv("MH_FRONTIER_MIN_RECORDS");
+    if (mn && *mn && atoll(mn) > 0) least = (u64)atoll(mn);
+    const u64 want = std::max<u64>(n + n / 4, least);
+    if (want > 0x7fffffffull) return fail(MH_ENOMEM, "a level of %llu members", (unsigned long long)n);
+    dfree(H->dMem, H->stream);
+    H->dMem = nullptr;
+    H->device_bytes -= (int64_t)(2 * sizeof(Member) * (size_t)H->mcap);
+    H->mcap = 0;
+    const int rc = dalloc(&H->dMem, 2 * (size_t)want, &H->device_bytes, H->dev, H->stream);
+    if (rc) return rc;
+    H->mcap = (u32)want;
+    return MH_OK;
+}
+
 // After an overflow: grows every depth whose busiest shard outgrew its region.
 int grow_overflowed(mh_handle *H, int h, const u32 *hc)
 {
@@ -504,9 +531,9 @@ int ensure_workspace(mh_handle *H, int h)
         (rc = need(&H->dWork, (size_t)kWorkCount + 2)) || (rc = need(&H->dCounts, (size_t)kCountSets * kCountWords)) ||
         (rc = need(&H->dCand, (size_t)kCandidates)) || (rc = need(&H->dChamp, nt1)) ||
         (rc = need(&H->dChampOk, nt1)) || (rc = need(&H->dSsum, nt1 * 2 * kMaxH)) ||
-        (rc = need(&H->dGK, (size_t)H->G)) || (rc = need(&H->dCov, (size_t)H->c.WTp + 2 * (kMaxH + 1))) ||
-        (rc = need(&H->dSync, (size_t)1)))
+        (rc = need(&H->dLevel, level_bytes(H->Nt))) || (rc = need(&H->dSync, (size_t)1)))
         return rc;
+    if ((rc = ensure_members(H, 1))) return rc;
     if (!H->hState) {
         H->pgrid = H->coop ? persistent_grid(H->num_sms, true) : 0;
         if (!(H->hState = pinned_state_get())) return fail(MH_ENOMEM, "pinned host allocation failed");
@@ -628,9 +655,15 @@ int prepare_solve(mh_handle *H, const mh_solve_opts *opts, Solve *s, int *max_ro
     s->champ = paper ? H->dChamp : nullptr;
     s->champ_ok = paper ? H->dChampOk : nullptr;
     s->ssum = paper ? H->dSsum : nullptr;
-    s->gk = H->dGK;
-    s->cov = H->dCov;
-    s->run = H->dCov + H->c.WTp;
+    {
+        const size_t nt1 = (size_t)std::max(H->Nt, 1);
+        s->lev = (Level *)H->dLevel;
+        s->sel = (Key *)(H->dLevel + 256);
+        s->covsel = (int *)(H->dLevel + 256 + nt1 * sizeof(Key));
+        s->cr = (u16 *)(H->dLevel + 256 + nt1 * (sizeof(Key) + sizeof(int)));
+        s->mem = H->dMem;
+        s->mcap = H->mcap;
+    }
     s->cut = H->dCut;
     s->shard = 0;
     s->nshards = 1;
@@ -642,6 +675,22 @@ int prepare_solve(mh_handle *H, const mh_solve_opts *opts, Solve *s, int *max_ro
     return MH_OK;
 }
 
+// After a level outgrew the member buffers: larger ones (the largest count seen sets the
+// size), and the level's count starts over.
+int grow_members(mh_handle *H, Solve *s, cudaStream_t st)
+{
+    Level lev;
+    MH_CUDA(cudaMemcpyAsync(&lev, s->lev, sizeof lev, cudaMemcpyDeviceToHost, st));
+    MH_CUDA(cudaStreamSynchronize(st));
+    const int rc = ensure_members(H, *std::max_element(lev.mcnt, lev.mcnt + 4));
+    if (rc) return rc;
+    s->mem = H->dMem;
+    s->mcap = H->mcap;
+    MH_CUDA(cudaMemsetAsync(s->lev->mcnt, 0, sizeof lev.mcnt, st));
+    MH_CUDA(cudaMemsetAsync(s->state + 3, 0, sizeof(int), st));
+    return MH_OK;
+}
+
 Frontiers frontiers_of(const mh_handle *H)
 {
     Frontiers f;
@@ -649,11 +698,11 @@ Frontiers frontiers_of(const mh_handle *H)
     for (int l = 0; l < kMaxH; ++l) {
         f.F[l] = H->dF[l];
         f.cap[l] = H->cap[l];
-        // side arrays of the slots: lb (Key), then sig and lc (u64)
+        // side arrays of the slots: lb (Key), then ub and lc (u64)
         const size_t n = (size_t)H->cap[l] * kShards;
         unsigned char *side = H->dSide[l];
         f.lb[l] = side ? (Key *)side : nullptr;
-        f.sig[l] = side ? (u64 *)(side + n * sizeof(Key)) : nullptr;
+        f.ub[l] = side ? (u64 *)(side + n * sizeof(Key)) : nullptr;
         f.lc[l] = side ? (u64 *)(side + n * (sizeof(Key) + sizeof(u64))) : nullptr;
     }
     return f;
@@ -919,6 +968,13 @@ MH_API int mh_solve_ex(mh_handle *H, const mh_solve_opts *opts, mh_result **out)
                 destroy_events();
                 return fail(MH_ETIMEOUT, "a grid barrier of the persistent solve timed out in round %d", rounds_done);
             }
+            if (hs[3] == kOverMembers) {  // the level is searched again
+                if ((rc = grow_members(H, &s, st))) {
+                    destroy_events();
+                    return rc;
+                }
+                continue;
+            }
             if (hs[3]) {  // the frontier counters of the overflowed round (its parity's set)
                 MH_CUDA(cudaMemcpy(H->hState + kStateWords, counts + (size_t)(rounds_done & 1) * kCountWords,
                                    sizeof(u32) * kCountWords, cudaMemcpyDeviceToHost));
@@ -1089,7 +1145,7 @@ std::string batch_signature(mh_handle *const *hs, const mh_solve_opts *opts, int
     }
     std::sort(parts.begin(), parts.end());
     std::ostringstream o;
-    o << "grid" << grid;
+    o << "levels,grid" << grid;  // (the schedules' times differ from those of solves round by round)
     for (auto &p : parts) o << "," << p;
     return o.str();
 }
@@ -1331,7 +1387,10 @@ int run_batch(mh_handle *const *hs, const mh_solve_opts *opts, int n, const std:
             mh_handle *H = hs[i];
             MH_CUDA(cudaMemcpy(H->hState, H->dState, sizeof(int) * kStateWords, cudaMemcpyDeviceToHost));
             if (H->hState[2]) return fail(MH_ETIMEOUT, "a team barrier of the batched solve timed out");
-            if (H->hState[3]) {
+            if (H->hState[3] == kOverMembers) {
+                const int rc = grow_members(H, &ss[i], st);
+                if (rc) return rc;
+            } else if (H->hState[3]) {
                 const int r = H->hState[4];
                 MH_CUDA(cudaMemcpy(H->hState + kStateWords, H->dCounts + (size_t)(r & 1) * kCountWords,
                                    sizeof(u32) * kCountWords, cudaMemcpyDeviceToHost));
@@ -1396,9 +1455,14 @@ int run_in_turn(mh_handle *const *hs, const mh_solve_opts *opts, int n, double *
         if (H->hState[2]) return fail(MH_ETIMEOUT, "a grid barrier of the batched solve timed out");
         if (H->hState[3]) {  // overflowed: grown and solved again from the start
             const int r = H->hState[4];
-            MH_CUDA(cudaMemcpy(H->hState + kStateWords, H->dCounts + (size_t)(r & 1) * kCountWords,
-                               sizeof(u32) * kCountWords, cudaMemcpyDeviceToHost));
-            int rc = grow_overflowed(H, opts[i].h, (const u32 *)(H->hState + kStateWords));
+            int rc = MH_OK;
+            if (H->hState[3] == kOverMembers) {
+                rc = grow_members(H, &ss[i], st);
+            } else {
+                MH_CUDA(cudaMemcpy(H->hState + kStateWords, H->dCounts + (size_t)(r & 1) * kCountWords,
+                                   sizeof(u32) * kCountWords, cudaMemcpyDeviceToHost));
+                rc = grow_overflowed(H, opts[i].h, (const u32 *)(H->hState + kStateWords));
+            }
             if (rc) return rc;
             MH_CUDA(cudaMemsetAsync(H->dCounts, 0, sizeof(u32) * kCountSets * kCountWords, st));
             std::vector<double> w(1, 1.0);
@@ -1797,7 +1861,13 @@ struct mh_server {
                 continue;
             }
             if (st8[2]) rc = fail(MH_ETIMEOUT, "a team barrier of the served solve timed out");
-            if (rc == MH_OK && st8[3]) {
+            if (rc == MH_OK && st8[3] == kOverMembers) {
+                rc = grow_members(H, &r->s, st);
+                if (rc == MH_OK) {
+                    keep.push_back(r);
+                    continue;
+                }
+            } else if (rc == MH_OK && st8[3]) {
                 std::vector<u32> hc(kCountWords);
                 cudaMemcpy(hc.data(), H->dCounts + (size_t)(st8[4] & 1) * kCountWords, sizeof(u32) * kCountWords,
                            cudaMemcpyDeviceToHost);

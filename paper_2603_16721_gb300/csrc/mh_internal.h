@@ -107,6 +107,26 @@ struct StoreBuild {
     u64 *GS;
 };
 
+// A combination of the level being resolved: its tuple (as in Key), the k uncovered
+// tumors it covers, listed when few (else its rows give them).
+constexpr int kMemIds = 18;
+struct __align__(16) Member {
+    u64 t0, t1, t2;
+    u16 k;
+    u16 ids[kMemIds];
+    u16 pad;
+};
+static_assert(sizeof(Member) == 64, "members are 64 bytes, read as four 16-byte words");
+
+// Step i of a solve by levels finds its level (score + 1) in lmax[i & 3] and counts its
+// members in mcnt[i & 3]; step i - 2 clears the entries.
+struct Level {
+    u64 lmax[4];
+    u32 mcnt[4];
+};
+// Solve::state word 3: what outgrew its memory.
+constexpr int kOverFrontier = 1, kOverMembers = 2;
+
 // Per-solve device state.
 struct Solve {
     int h;
@@ -137,11 +157,16 @@ struct Solve {
     // correction from the nodes shared by two or more uncovered tumors (see
     // mh_kernels.cu).  nullptr: the counters are counted node by node.
     u64 *ssum;
-    // Incremental rounds: gk[g] = uncovered tumors carrying gene g (G entries);
-    // cov = the tumors the previous round's winner covered (WTp words).
-    u32 *gk;
-    u64 *cov;
-    u64 *run;  // 2 (kMaxH + 1) words: running totals of the counter corrections (see mh_kernels.cu)
+    // Solve by score levels (see mh_levels.cuh; the others leave them nullptr): the
+    // levels' maxima and member counts, two buffers of mcap members, the picks (Nt
+    // entries: score + 1, tuple, TP in the low bits of t2), per tumor the pick that
+    // covers it (-1: none) and the round it is covered in.
+    Level *lev;
+    Member *mem;
+    u32 mcap;
+    Key *sel;
+    int *covsel;
+    u16 *cr;
     u64 *cut;  // score-bound mode: per round, per depth, the prefixes cut by the bound (nullptr: none)
     // Split search (one kernel per phase only): this solve searches the depth-1
     // genes g (search order) with g % nshards == shard; xbest[0] receives the
@@ -170,19 +195,18 @@ enum {
 };
 
 // Frontier buffers (depth l at index l): kShards regions of cap[l] records each.
-// Incremental rounds keep, per record slot of every depth: sig = the OR of
-// 1 << (s & 63) over the record's tumor samples (0: no longer shared by two
-// uncovered tumors, ~0: samples not listed), and for the leaf parents (depth h-1)
-// lb = the best key among the record's leaves with TP >= 2 and lc = the sum of
-// TP - 1 over them.  nullptr where not allocated.
+// A solve by levels keeps for every leaf parent i (depth h-1, by record index): ub = a
+// bound on the score + 1 of its leaves with TP >= 2 (0: none), and over all tumors lb =
+// the best key among those leaves and lc = the sum of TP - 1 over them.  nullptr where
+// not allocated.
 struct Frontiers {
     Rec *F[kMaxH];
     u32 cap[kMaxH];
-    u64 *sig[kMaxH];
+    u64 *ub[kMaxH];
     Key *lb[kMaxH];
     u64 *lc[kMaxH];
 };
-// Device bytes of one frontier record slot with its incremental-round data.
+// Device bytes of one frontier record slot with its per-record data.
 constexpr size_t kSlotBytes = sizeof(Rec) + 2 * sizeof(u64) + sizeof(Key);
 
 // Grid-wide barrier state of the persistent solve (zeroed before each launch):

@@ -51,11 +51,10 @@ __device__ __forceinline__ Team grid_team() { return Team{(int)blockIdx.x, (int)
 // threshold in s.best_hint.  Persistent solve: depth-1 nodes built from the gene
 // rows and the block's copy of U (Ush), bests stored into the round's slot array,
 // the round's threshold word, diagnostics by round parity.
-// fm: counters by per-sample sums and incremental rounds (see "Counting by
-// per-sample sums" and "Incremental rounds" below): only nodes shared by two or
-// more uncovered tumors are built and searched; build: the expansion builds the
-// kept frontiers of round 0 and adds no counters (the evaluation that follows
-// counts every kept node).
+// fm: the solve by score levels (see "Counting by per-sample sums" below and
+// mh_levels.cuh): only nodes shared by two or more tumors are built; build: the
+// expansion builds the kept frontiers and adds no counters (they follow from the kept
+// nodes after the last level).
 struct RoundIO {
     const u64 *Ush;
     Key *slots;
@@ -256,7 +255,7 @@ __device__ __forceinline__ u16 sat16(int v) { return (u16)(v < 0xffff ? v : 0xff
 
 // Round state (Solve::state): a kernel of a round does nothing once the solve is
 // done or a frontier of the round has overflowed.
-enum { kStK = 0, kStDone = 1, kStError = 2, kStOverflow = 3, kStRound = 4, kStMaxRounds = 5, kStYield = 6 };
+enum { kStK = 0, kStDone = 1, kStError = 2, kStOverflow = 3, kStRound = 4, kStMaxRounds = 5, kStYield = 6, kStStep = 7 };
 
 __device__ __forceinline__ bool halted(const Solve &s) { return s.state[kStDone] | s.state[kStOverflow]; }
 
@@ -475,9 +474,8 @@ struct Batch {
     u64 ns[kMaxWords];              // child masks and their (record, word) of one item per lane
     int cx[33];                     // expansion: exclusive prefix sum of the lanes' child counts
     u16 po[kBatch][kMaxH - 1];      // leaves: ascending original indices of each record's prefix
-    Key rb[kBatch];                 // incremental rounds: per leaf parent, its best leaf (TP >= 2)
-    u64 rc[kBatch];                 //   and the sum of TP - 1 over those leaves (rb[j].s holds
-                                    //   the packed best while a listed record's items merge)
+    u64 pb[kBatch];                 // solve by levels: per leaf parent, its best leaf with TP >= 2
+    u64 rc[kBatch];                 //   (packed) and the sum of TP - 1 over those leaves
 };
 
 // Depth-1 node of gene g (search order) built from its rows and U: y_1 = U & x_g,
@@ -1834,46 +1832,12 @@ __device__ __noinline__ void phase_sample_sums(const Cohort &c, const Solve &s, 
     }
 }
 
-// tot[0 .. 2h) = the per-sample sums over all tumors.
-__device__ void block_sample_totals(const Cohort &c, const Solve &s, u64 *tot)
-{
-    const int h2 = 2 * s.h, lane = threadIdx.x & 31;
-    if (threadIdx.x < 2 * kMaxH) tot[threadIdx.x] = 0;
-    __syncthreads();
-    for (int k = 0; k < h2; ++k) {
-        u64 v = 0;
-        for (int smp = threadIdx.x; smp < c.Nt; smp += blockDim.x)
-            v += __ldcg(s.ssum + (size_t)smp * h2 + k);
-        v = warp_sum_u64(v);
-        if (lane == 0 && v) atomicAdd(&tot[k], v);
-    }
-    __syncthreads();
-}
-
 // ---------------------------------------------------------------------------
-// Incremental rounds.  U only shrinks from one round to the next, so the nodes
-// that two or more uncovered tumors share in a later round are among those of
-// round 0, and a node's tumor intersection -- its size, its children's TP and its
-// leaves' scores -- changes only if it holds a tumor that the previous winner
-// covered.  With counting by per-sample sums, round 0 builds the shared
-// ("multi-sample") nodes of every depth below the leaves and keeps them for the
-// whole solve, and evaluates every leaf parent once, caching its best leaf key
-// among its leaves with TP >= 2 and the sum of TP - 1 over them.  A later round
-// scans the kept nodes, brings up to date only those holding a newly covered
-// tumor (re-evaluating the leaf parents among them), reads everything else from
-// the caches, and ends after one grid barrier.  The argmax and every counter are
-// those of a full search of the round.
+// Kept nodes.  The solve by score levels (mh_levels.cuh) builds the nodes that two or
+// more tumors share, of every depth below the leaves, once per solve into the frontiers
+// and evaluates every leaf parent once.
 
 __device__ __forceinline__ bool in_mask(const u64 *m, int smp) { return (m[smp >> 6] >> (smp & 63)) & 1ull; }
-
-// Signature of a record's tumor samples: OR of 1 << (s & 63) (~0 when not listed).
-__device__ __forceinline__ u64 sample_sig(const Rec &r)
-{
-    if (is_dense(r.ky, r.kn)) return ~0ull;
-    u64 g = 0;
-    for (int q = 0; q < (int)r.ky; ++q) g |= 1ull << (r.ids[q] & 63);
-    return g;
-}
 
 // Slot (shard * cap + offset) of record i of a sharded frontier (soff from front_open).
 __device__ __forceinline__ u32 front_slot(u32 cap_s, const int *soff, u32 i)
@@ -1884,89 +1848,6 @@ __device__ __forceinline__ u32 front_slot(u32 cap_s, const int *soff, u32 i)
         if ((u32)soff[mid] <= i) lo = mid; else hi = mid - 1;
     }
     return (u32)lo * cap_s + (i - (u32)soff[lo]);
-}
-
-// Uncovered tumors carrying gene g: its static record's listed tumors in U, or
-// the popcount of its row and U.
-__device__ __forceinline__ u32 gene_uncovered(const Cohort &c, const u64 *Ush, int g)
-{
-    const Rec &sr = c.GR[g];
-    const int ky = (int)__ldg(&sr.ky);
-    if (ky <= kListT) {
-        u32 k = 0;
-        for (int q = 0; q < ky; ++q) k += (u32)in_mask(Ush, (int)__ldg(&sr.ids[q]));
-        return k;
-    }
-    const u64 *trow = c.T + (size_t)g * c.WTp;
-    u32 k = 0;
-    for (int w = 0; w < c.Wt; ++w) k += (u32)__popcll(__ldg(trow + w) & Ush[w]);
-    return k;
-}
-
-// Brings a kept record of depth L up to date with U; returns true if its tumor
-// intersection changed (always with force).  Listed samples: the covered ones are
-// dropped.  Unlisted: the intersection is recounted from the rows, and listed
-// once it is small enough.
-__device__ bool refresh_record(const Cohort &c, const u64 *Ush, const u64 *Csh, int L, Rec &r, bool force)
-{
-    if (!is_dense(r.ky, r.kn)) {
-        int k = 0;
-        for (int q = 0; q < (int)r.ky; ++q) {
-            const int smp = r.ids[q];
-            if (in_mask(Ush, smp)) r.ids[k++] = (u16)smp;
-        }
-        const bool changed = k != (int)r.ky;
-        r.ky = (u16)k;
-        return changed || force;
-    }
-    const u64 *rows[kMaxH - 1];
-#pragma unroll
-    for (int i = 0; i < kMaxH - 1; ++i) rows[i] = i < L ? c.T + (size_t)prefix_gene(r.p, i) * c.WTp : nullptr;
-    if (!force) {
-        // unchanged unless the prefix rows meet a covered tumor (few words of Csh are non-zero)
-        bool hit = false;
-        for (int w = 0; w < c.Wt && !hit; ++w) {
-            u64 y = Csh[w];
-            if (!y) continue;
-#pragma unroll
-            for (int i = 0; i < kMaxH - 1; ++i)
-                if (i < L) y &= __ldg(rows[i] + w);
-            hit = y != 0;
-        }
-        if (!hit) return false;
-    }
-    // recount over U, four words (and their rows) in flight at a time
-    int ky = 0;
-    for (int w0 = 0; w0 < c.Wt; w0 += 4) {
-        u64 y[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) y[k] = w0 + k < c.Wt ? Ush[w0 + k] : 0ull;
-#pragma unroll
-        for (int i = 0; i < kMaxH - 1; ++i) {
-            if (i >= L) break;
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (w0 + k < c.Wt) y[k] &= __ldg(rows[i] + w0 + k);
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) ky += __popcll(y[k]);
-    }
-    r.ky = sat16(ky);
-    if (!is_dense(ky, r.kn)) {
-        int k = 0;
-        for (int w = 0; w < c.Wt; ++w) {
-            u64 y = Ush[w];
-            for (int i = 0; i < L && y; ++i) y &= __ldg(c.T + (size_t)prefix_gene(r.p, i) * c.WTp + w);
-            for (; y; y &= y - 1) r.ids[k++] = (u16)(w * 64 + __ffsll((long long)y) - 1);
-        }
-        k = kListT;
-        for (int w = 0; w < c.Wn; ++w) {
-            u64 n = ~0ull;
-            for (int i = 0; i < L; ++i) n &= __ldg(c.N + (size_t)prefix_gene(r.p, i) * c.WNp + w);
-            for (; n; n &= n - 1) r.ids[k++] = (u16)(w * 64 + __ffsll((long long)n) - 1);
-        }
-    }
-    return true;
 }
 
 // One (record j, column word wi) item of a leaf parent: the record's tumor
@@ -2029,30 +1910,6 @@ __device__ __forceinline__ void leaf_item_eval(const Cohort &c, const Solve &s, 
     }
 }
 
-// Original indices of a kept record's prefix genes, ascending, in the record's
-// spare bytes (prefixes of up to kPadGenes genes).
-constexpr int kPadGenes = 6;
-__device__ __forceinline__ u16 *pad_po(Rec &r) { return reinterpret_cast<u16 *>(r.pad); }
-// The ascending original indices of a leaf parent's L prefix genes.
-__device__ __forceinline__ void record_po(const Cohort &c, Rec &r, int L, int *po)
-{
-#pragma unroll
-    for (int q = 0; q < kMaxH - 1; ++q) po[q] = 0;
-    if (L <= kPadGenes) {
-        for (int q = 0; q < L; ++q) po[q] = pad_po(r)[q];
-        return;
-    }
-    for (int q = 0; q < L; ++q) {
-        const int v = c.orig[prefix_gene(r.p, q)];
-        int k = q - 1;
-        while (k >= 0 && po[k] > v) {
-            po[k + 1] = po[k];
-            --k;
-        }
-        po[k + 1] = v;
-    }
-}
-
 // Merges the per-lane keys of one item step into the records' best keys: items of
 // a step sit on the lanes in record order, so a segmented warp maximum leaves each
 // record's best on its first lane, which merges it into rb.
@@ -2071,47 +1928,38 @@ __device__ __forceinline__ void merge_item_keys(Batch &b, int jr, u64 p, u64 cor
     const int jp = __shfl_up_sync(kFull, jr, 1);
     if (jr >= 0 && (lane == 0 || jp != jr)) {
         b.rc[jr] += corr;
-        if (p > b.rb[jr].s) b.rb[jr].s = p;
+        if (p > b.pb[jr]) b.pb[jr] = p;
     }
     __syncwarp();
 }
 
-// Evaluates the leaf parents b.r[j] (depth L = h - 1) of the lanes with `live`:
-// b.rb[j] = the best key among the record's leaves with TP >= 2 (empty if none),
-// b.rc[j] = the sum of TP - 1 over them.  TP = 1 leaves are left to the
-// champions.  The (record, column word) items are spread over the lanes as in the
-// leaf phase; unlisted records take the row path, the whole warp per record.
+// Evaluates the listed leaf parents b.r[j] (depth L = h - 1) of the lanes with `live`:
+// b.pb[j] = the best among the record's leaves with TP >= 2 (packed; 0 if none), b.rc[j] =
+// the sum of TP - 1 over them, b.po[j] = the prefix's ascending original indices.  TP = 1
+// leaves are left to the champions.  The (record, column word) items are spread over the
+// lanes as in the leaf phase.
 __device__ void leaf_parents_eval(const Cohort &c, const Solve &s, Batch &b, bool live, int L, int lane)
 {
-    int lo = 1, hi = 0, ky = 0, kn = 0;
-    b.rb[lane] = key_empty();
+    int lo = 1, hi = 0;
+    b.pb[lane] = 0;
     b.rc[lane] = 0;
     if (live) {
         Rec &r = b.r[lane];
         lo = prefix_gene(r.p, L - 1) + 1;
         hi = c.G - 1;
-        ky = r.ky;
-        kn = r.kn;
-        if (L <= kPadGenes) {  // ascending original indices of the prefix (leaf keys)
-            for (int q = 0; q < L; ++q) b.po[lane][q] = pad_po(r)[q];
-        } else {
-            for (int q = 0; q < L; ++q) {
-                const u16 v = c.orig[prefix_gene(r.p, q)];
-                int k = q - 1;
-                while (k >= 0 && b.po[lane][k] > v) {
-                    b.po[lane][k + 1] = b.po[lane][k];
-                    --k;
-                }
-                b.po[lane][k + 1] = v;
+        for (int q = 0; q < L; ++q) {
+            const u16 v = c.orig[prefix_gene(r.p, q)];
+            int k = q - 1;
+            while (k >= 0 && b.po[lane][k] > v) {
+                b.po[lane][k + 1] = b.po[lane][k];
+                --k;
             }
+            b.po[lane][k + 1] = v;
         }
     }
     b.lo[lane] = lo;
     b.hi[lane] = hi;
-    const bool any = live && hi >= lo;
-    const bool dense = any && is_dense(ky, kn);
-    unsigned dmask = __ballot_sync(kFull, dense);
-    const int nw = (any && !dense) ? (hi >> 6) - (lo >> 6) + 1 : 0;
+    const int nw = live && hi >= lo ? (hi >> 6) - (lo >> 6) + 1 : 0;
     const int incl = warp_incl_scan(nw, lane);
     b.off[lane] = incl - nw;
     if (lane == 31) b.off[kBatch] = incl;
@@ -2129,57 +1977,9 @@ __device__ void leaf_parents_eval(const Cohort &c, const Solve &s, Batch &b, boo
         }
         merge_item_keys(b, valid ? j : -1, ib, corr, lane);
     }
-    if (live && !dense && b.rb[lane].s != 0) {  // the packed best of each listed record as its key
-        int po[kMaxH - 1];
-#pragma unroll
-        for (int q = 0; q < kMaxH - 1; ++q) po[q] = q < L ? b.po[lane][q] : 0;
-        b.rb[lane] = unpack_leaf(b.rb[lane].s, po, L);
-    }
-    __syncwarp();
-    // unlisted records: the whole warp, one leaf gene per lane, on the rows
-    while (dmask) {
-        const int jd = __ffs(dmask) - 1;
-        dmask &= dmask - 1;
-        const Prefix p = b.r[jd].p;
-        const int dlo = b.lo[jd], dhi = b.hi[jd];
-        unsigned by, bn;
-        dense_setup(c, s, p, L, b, by, bn, lane);
-        int po[kMaxH - 1];
-#pragma unroll
-        for (int q = 0; q < kMaxH - 1; ++q) po[q] = q < L ? b.po[jd][q] : 0;
-        Key best = key_empty();
-        u64 corr = 0;
-        for (int g = dlo + lane; g <= dhi; g += 32) {
-            const u64 *trow = c.T + (size_t)g * c.WTp;
-            int tp = 0;
-            for (unsigned bits = by; bits; bits &= bits - 1) {
-                const int w = __ffs(bits) - 1;
-                tp += __popcll(b.ys[w] & trow[w]);
-            }
-            if (tp < 2) continue;
-            corr += (u64)(tp - 1);
-            const u64 *nrow = c.N + (size_t)g * c.WNp;
-            int fp = 0;
-            for (unsigned bits = bn; bits; bits &= bits - 1) {
-                const int w = __ffs(bits) - 1;
-                fp += __popcll(b.ns[w] & nrow[w]);
-            }
-            const u64 s1 = s.a_num * (u64)tp + s.a_den * (u64)(c.Nn - fp) + 1;
-            if (s1 < best.s) continue;
-            const Key k = leaf_key(s1, po, L, c.orig[g]);
-            if (key_better(k, best)) best = k;
-        }
-        best = warp_max_key(best);
-        corr = warp_sum_u64(corr);
-        if (lane == 0) {
-            b.rb[jd] = best;
-            b.rc[jd] = corr;
-        }
-        __syncwarp();
-    }
 }
 
-// Round 0 of an incremental solve with h = 2: the depth-1 nodes that two or more
+// Build of a solve by levels with h = 2: the depth-1 nodes that two or more
 // uncovered tumors share (the leaf parents) into the depth-1 frontier.  Every
 // thread of the block must call it.
 __device__ void phase_build1(const Cohort &c, const Solve &s, const Frontiers &f, u32 *counts, Batch &b,
@@ -2201,573 +2001,7 @@ __device__ void phase_build1(const Cohort &c, const Solve &s, const Frontiers &f
     }
 }
 
-// One incremental round, or with force the evaluation that follows round 0's
-// build, by every block of the team.  Depth 1: in round 0 the block counts its
-// share of the genes; later, each gene of a tumor covered since the previous
-// round loses one uncovered tumor.  Kept records: the block scans its share of
-// every depth (record i to block i mod B, then to warp (i / B) mod W, so that
-// records appended together spread out), brings up to date those holding a
-// covered tumor (their signature meets the covered tumors'), re-evaluates the leaf
-// parents among them, and takes the others' best keys from the caches.  After
-// round 0 each warp keeps its live records in an on-chip list (built once they
-// fit) and reads from L2 only the records a covered tumor touches; changed leaf
-// parents are evaluated by the whole block through a queue of tasks.  What it
-// adds to the round's counter slots are CHANGES of the running totals (in round
-// 0, the corrections themselves), which the end of the round accumulates: depth
-// 1's surviving count; (k - 1)(hi(2) - g) over the genes shared by k >= 2
-// uncovered tumors; for a kept node of depth l >= 2 with k >= 2 tumors, k - 1 to
-// depth l and (k - 1)(hi(l+1) - last) to depth l + 1; the leaf parents' sums of
-// TP - 1 to depth h; and the per-sample sums of the tumors the last winner
-// covered.  The block's best key (leaf caches, and the champions of its uncovered
-// tumors, which stand for the TP = 1 leaves) goes to its slot.  Every thread of
-// the block must call it; returns false (for every thread) if round 0 overflowed
-// a frontier.
-constexpr int kScanIlp = 4;  // records whose signature and cached score a lane loads at once
-// changed leaf parents a block spreads over its warps per round (one-block-per-SM
-// builds; the smaller blocks keep their shared memory for occupancy)
-constexpr int kEvalQueue = 64;
-// soffs / nrec / tab_ok: the kept frontiers' shard offsets and sizes, read once per
-// launch (after round 0's build) into the block's shared memory.
-struct FrontTab {
-    int soff[kMaxH][kShards + 1];
-    long long n[kMaxH];
-    int ok;
-    // per warp: its list of live kept records (built in a round after round 0, when
-    // they fit) and, per depth, where the depth's entries start and how many there are
-    signed char lok[kMaxWarpsPerBlock];
-    short lbase[kMaxWarpsPerBlock][kMaxH];
-    short lcnt[kMaxWarpsPerBlock][kMaxH];
-};
-// Entries of a warp's list of live kept records (one-block-per-SM builds).  After
-// round 0 a record that no longer holds two uncovered tumors can never hold them
-// again (U only shrinks): DelCols has emptied it for good, and the list drops it.
-// The list keeps each live record's slot, sample signature and cached best score
-// on chip, so a round reads only the records that a covered tumor touches.
-constexpr int kList = 160;
-template <int kLWarps>
-struct LiveLists {
-    u32 slot[kLWarps][kList];
-    u64 sig[kLWarps][kList];
-    u64 ls[kLWarps][kList];
-    u16 dq[kLWarps][kList];  // a round's touched entries, by position
-};
-template <int kQueue, int kLWarps>
-__device__ bool phase_update(const Cohort &c, const Solve &s, int round, const Frontiers &f, const u32 *counts,
-                             Batch &b, const Team &t, const RoundIO &io, const u64 *Csh, bool force, FrontTab &ft)
-{
-    __shared__ u64 acc[kAccN];
-    __shared__ int overflow;
-    __shared__ int qn;  // the block's queue of changed leaf parents
-    __shared__ Rec qrec[kQueue > 0 ? kQueue : 1];
-    __shared__ u32 qslot[kQueue > 0 ? kQueue : 1];
-    __shared__ u64 qlco[kQueue > 0 ? kQueue : 1];
-    __shared__ short qidx[kQueue > 0 ? kQueue : 1];  // list entry of a queued record (-1: none)
-    __shared__ signed char qwarp[kQueue > 0 ? kQueue : 1];
-    __shared__ int qlo[kQueue > 0 ? kQueue : 1], qtasks[kQueue > 0 ? kQueue : 1];  // first leaf gene, tasks
-    __shared__ u64 qbest[kQueue > 0 ? kQueue : 1];
-    __shared__ u32 qcorr[kQueue > 0 ? kQueue : 1];  // a record's sum of TP - 1 stays below 2^27
-    // a queued leaf parent's first leaf gene and tasks of 32 column words (set when it is queued)
-    auto queue_tasks = [&](int q, const Rec &r, int L) {
-        const int lo = prefix_gene(r.p, L - 1) + 1;
-        qlo[q] = lo;
-        qtasks[q] = (((c.G - 1) >> 6) - (lo >> 6) + 1 + 31) >> 5;
-        qbest[q] = 0;
-        qcorr[q] = 0;
-    };
-    __shared__ LiveLists<(kLWarps > 0 ? kLWarps : 1)> lv;
-    const long long t0 = clock64();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int h = s.h;
-    const u64 *Ush = io.Ush;
-    const int qcap = kQueue < 32 * nwarps ? kQueue : 32 * nwarps;
-    // each tumor's offset into the per-sample gene lists, on chip (one-block-per-SM builds)
-    __shared__ u32 so_sh[kLWarps > 0 ? kMaxWords * 64 + 1 : 1];
-    // the changes of the depths' corrections: per warp, summed over the warps at the
-    // end (one-block-per-SM builds), else block-wide in acc
-    __shared__ u64 wdeep[kLWarps > 0 ? kLWarps : 1][2 * kMaxH + 2];
-    u64 *deep = acc + kAccDeep;
-    if (kLWarps > 0)
-        for (int i = lane; i < 2 * kMaxH + 2; i += 32) wdeep[warp][i] = 0;
-    auto deep_add = [&](int i, u64 v) {
-        if (kLWarps > 0) wdeep[warp][i] += v;
-        else acc_add(deep, i, v);
-    };
-    if (threadIdx.x == 0) {
-        overflow = 0;
-        qn = 0;
-    }
-    if (kLWarps > 0 && (force || !ft.ok))  // once per launch, published by acc_begin's barrier
-        for (int i = (int)threadIdx.x; i <= c.Nt; i += (int)blockDim.x) so_sh[i] = __ldg(c.SO + i);
-    acc_begin(acc);
-    u64 csig = 0;
-    for (int w = 0; w < c.Wt; ++w) csig |= Csh[w];
-    Key best = key_empty();
-    // After round 0 the block's last warp takes the champions and depth 1 while the
-    // others scan the kept records, so that their chains of loads overlap; the lead
-    // block (rank 0), which ends the round with more work than the others, scans no
-    // records then.
-    const int gwarp = nwarps - 1;
-    const bool side = force || warp == gwarp;
-    const int sstride = force ? (int)blockDim.x : 32, sbase = force ? (int)threadIdx.x : lane;
-    for (int smp = t.rank * sstride + sbase; side && smp < c.Nt; smp += t.size * sstride) {
-        if (!in_mask(Ush, smp)) continue;
-        Key k;  // the four words in one round trip
-        k.s = __ldcg(&s.champ[smp].s);
-        k.t0 = __ldcg(&s.champ[smp].t0);
-        k.t1 = __ldcg(&s.champ[smp].t1);
-        k.t2 = __ldcg(&s.champ[smp].t2);
-        if (k.s != 0 && key_better(k, best)) best = k;
-    }
-    // the lead's idle warps: the previous round's longest warps join the diagnostics
-    if (t.rank == 0 && !side) {
-        if (warp == 0 && lane < 2 && round > 0) {
-            const int mx = (((round - 1) & 1) ? kWorkWarpMaxOdd : kWorkWarpMax) + lane;
-            s.work[kWorkWarpMaxSum + lane] += __ldcg(&s.work[mx]);
-            s.work[mx] = 0;
-        }
-    }
-    // depth 1
-    if (side) {
-        const int last1 = c.G - h, hi2 = c.G - h + 1;
-        u64 alive1 = 0, corrv = 0, sv = 0;
-        if (force) {  // the genes of a contiguous share, one per thread
-            const int g0 = (int)((long long)c.G * t.rank / t.size), g1 = (int)((long long)c.G * (t.rank + 1) / t.size);
-            for (int g = g0 + (int)threadIdx.x; g < g1; g += (int)blockDim.x) {
-                const u32 k = gene_uncovered(c, Ush, g);
-                s.gk[g] = k;
-                if (g <= last1) {
-                    alive1 += (u64)(k >= 1);
-                    if (k >= 2) corrv += (u64)(k - 1) * (u64)(hi2 - g);
-                }
-            }
-        } else {
-            // each gene of a covered tumor loses one uncovered tumor, and the tumor's
-            // per-sample sums of depths 2..h leave the totals: they join the running
-            // totals that the end of the round subtracts (lane k < h - 1: the visited
-            // sum of depth k + 2, lane h - 1 + k: its surviving sum)
-            const int h2 = 2 * h;
-            const bool sl = lane < 2 * (h - 1);
-            const int sd = lane < h - 1 ? lane + 2 : lane - (h - 1) + 2;
-            const int sidx = lane < h - 1 ? h + sd - 1 : sd - 1;
-            for (int smp = t.rank; smp < c.Nt; smp += t.size) {
-                if (!in_mask(Csh, smp)) continue;
-                if (sl) sv += __ldcg(s.ssum + (size_t)smp * h2 + sidx);
-                const u32 off = kLWarps > 0 ? so_sh[smp] : __ldg(c.SO + smp);
-                const int m = (int)((kLWarps > 0 ? so_sh[smp + 1] : __ldg(c.SO + smp + 1)) - off);
-                for (int q = lane; q < m; q += 32) {
-                    const int g = (int)__ldg(c.SL + off + q);
-                    const u32 old = atomicSub(s.gk + g, 1u);
-                    if (g <= last1) {
-                        if (old == 1) alive1 -= 1ull;
-                        if (old >= 2) corrv -= (u64)(hi2 - g);
-                    }
-                }
-            }
-        }
-        alive1 = warp_sum_u64(alive1);
-        corrv = warp_sum_u64(corrv);
-        if (lane == 0) {
-            deep_add(3, alive1);
-            deep_add(4, corrv);
-        }
-        __syncwarp();
-        if (sv) deep_add(lane < h - 1 ? 2 * (lane + 2) : 2 * (lane - (h - 1) + 2) + 1, sv);
-    }
-    // kept records: depth 1 (h = 2) or 2 .. h-1; the deepest are the leaf parents
-    if (force || !ft.ok) {  // their sizes and shard offsets, once per launch
-        for (int l = h == 2 ? 1 : 2; l <= h - 1; ++l) {
-            if (warp == 0) {
-                const long long nl = front_open(counts, l, f.cap[l], b.soff, lane);
-                if (nl < 0 && lane == 0) overflow = 1;
-                for (int i = lane; i <= kShards; i += 32) ft.soff[l][i] = b.soff[i];
-                if (lane == 0) ft.n[l] = nl;
-            }
-        }
-        __syncthreads();
-        if (overflow) return false;
-        if (threadIdx.x == 0) ft.ok = 1;
-    }
-    // after round 0 a warp whose live records fit its list scans the list only; a warp
-    // builds its list in the first round after round 0 in which they fit
-    const bool use_list = kLWarps > 0 && !force && ft.lok[warp] == 1;
-    const bool build_list = kLWarps > 0 && !force && ft.lok[warp] == 0;
-    int lfill = 0;
-    bool lfit = true;
-    for (int l = h == 2 ? 1 : 2; l <= h - 1; ++l) {
-        const long long n_in = ft.n[l];
-        if (build_list && lane == 0) ft.lbase[warp][l] = (short)lfill;
-        const int *soff = ft.soff[l];
-        const bool leafp = l == h - 1;
-        const int hiN = c.G - h + l;  // hi(l + 1), 0-based
-        u64 dA = 0, dV = 0, dL = 0;
-        // scanners: every block and warp in round 0; later all warps but the last of
-        // every block but the lead
-        const bool split = !force && t.size > 1 && nwarps > 1;
-        const u64 B = split ? (u64)(t.size - 1) : (u64)t.size, W = split ? (u64)(nwarps - 1) : (u64)nwarps;
-        const u64 rk = split ? (u64)(t.rank - 1) : (u64)t.rank;
-        const u64 n = (n_in < 0 || (split && (t.rank == 0 || warp == gwarp))) ? 0ull : (u64)n_in;
-        if (use_list) {
-            // this warp's live records: drop the dead ones, pick out those a covered tumor
-            // touches, and take the best cached leaf of the others
-            u32 *Lslot = lv.slot[warp] + ft.lbase[warp][l];
-            u64 *Lsig = lv.sig[warp] + ft.lbase[warp][l], *Lls = lv.ls[warp] + ft.lbase[warp][l];
-            u16 *dq = lv.dq[warp];
-            const int cnt = ft.lcnt[warp][l];
-            int wpos = 0, nd = 0;
-            u64 lmax = 0;
-            for (int j0 = 0; j0 < cnt; j0 += 32) {
-                const int j = j0 + lane;
-                u32 sl = 0;
-                u64 sg = 0, lsv = 0;
-                if (j < cnt) {
-                    sl = Lslot[j];
-                    sg = Lsig[j];
-                    lsv = Lls[j];
-                }
-                const bool keep = sg != 0;
-                const unsigned km = __ballot_sync(kFull, keep);
-                __syncwarp();
-                const int pos = wpos + __popc(km & ((1u << lane) - 1u));
-                if (keep) {
-                    Lslot[pos] = sl;
-                    Lsig[pos] = sg;
-                    Lls[pos] = lsv;
-                }
-                wpos += __popc(km);
-                const bool dirty = keep && (sg & csig) != 0;
-                const unsigned dm = __ballot_sync(kFull, dirty);
-                if (dirty) dq[nd + __popc(dm & ((1u << lane) - 1u))] = (u16)pos;
-                nd += __popc(dm);
-                if (keep && !dirty && lsv > lmax) lmax = lsv;
-            }
-            __syncwarp();
-            if (lane == 0) ft.lcnt[warp][l] = (short)wpos;
-            // the untouched records' best cached leaves: a lane's first record with the
-            // warp's largest cached score is read now and merged after the touched
-            // records (their loads overlap); further ties, rare, after that
-            const u64 wmax = leafp ? warp_max_u64(lmax) : 0ull;
-            int hitj = -1;
-            bool more = false;
-            Key kc = key_empty();
-            if (wmax != 0) {  // warp-uniform (the lanes' bests differ)
-                const bool want = wmax >= best.s;
-                for (int j0 = 0; j0 < wpos; j0 += 32) {
-                    const int j = j0 + lane;
-                    if (want && j < wpos && Lls[j] == wmax && (Lsig[j] & csig) == 0) {
-                        if (hitj < 0) hitj = j;
-                        else more = true;
-                    }
-                }
-                if (hitj >= 0) {
-                    const u32 sl = Lslot[hitj];
-                    kc.s = wmax;
-                    kc.t0 = __ldcg(&f.lb[l][sl].t0);
-                    kc.t1 = __ldcg(&f.lb[l][sl].t1);
-                    kc.t2 = __ldcg(&f.lb[l][sl].t2);
-                }
-                if (__any_sync(kFull, more)) {  // before any touched record changes its entry
-                    for (int j0 = 0; j0 < wpos; j0 += 32) {
-                        const int j = j0 + lane;
-                        if (j < wpos && j != hitj && Lls[j] == wmax && (Lsig[j] & csig) == 0) {
-                            const u32 sl = Lslot[j];
-                            Key k2;
-                            k2.s = wmax;
-                            k2.t0 = __ldcg(&f.lb[l][sl].t0);
-                            k2.t1 = __ldcg(&f.lb[l][sl].t1);
-                            k2.t2 = __ldcg(&f.lb[l][sl].t2);
-                            if (key_better(k2, best)) best = k2;
-                        }
-                    }
-                }
-            }
-            for (int d0 = 0; d0 < nd; d0 += 32) {  // the touched ones, one per lane
-                const bool act = d0 + lane < nd;
-                const int pos = act ? (int)dq[d0 + lane] : 0;
-                const u32 sl = act ? Lslot[pos] : 0u;
-                Rec &r = b.r[lane];
-                bool changed = false;
-                int kyn = 0;
-                u64 lco = 0;
-                if (act) {
-                    load_rec(&r, f.F[l] + sl);
-                    if (leafp) lco = __ldcg(f.lc[l] + sl);
-                    const int kyo = (int)r.ky;
-                    changed = refresh_record(c, Ush, Csh, l, r, false);
-                    kyn = r.ky;
-                    if (changed) {
-                        const u64 nsg = kyn >= 2 ? sample_sig(r) : 0ull;
-                        f.sig[l][sl] = nsg;
-                        Lsig[pos] = nsg;
-                        copy_rec(f.F[l] + sl, &r);
-                        if (l >= 2) {
-                            const u64 fo = kyo >= 2 ? (u64)(kyo - 1) : 0ull, fn = kyn >= 2 ? (u64)(kyn - 1) : 0ull;
-                            dA += fn - fo;
-                            dV += (fn - fo) * (u64)(hiN - prefix_gene(r.p, l - 1));
-                        }
-                    } else if (leafp) {  // nothing covered in it after all: its cached best stands
-                        const u64 lsv = Lls[pos];
-                        if (lsv != 0 && lsv >= best.s) {
-                            Key kc;
-                            kc.s = lsv;
-                            kc.t0 = __ldcg(&f.lb[l][sl].t0);
-                            kc.t1 = __ldcg(&f.lb[l][sl].t1);
-                            kc.t2 = __ldcg(&f.lb[l][sl].t2);
-                            if (key_better(kc, best)) best = kc;
-                        }
-                    }
-                }
-                const bool eval = leafp && changed && kyn >= 2;
-                if (leafp && changed && kyn < 2) {
-                    f.lb[l][sl] = key_empty();
-                    f.lc[l][sl] = 0;
-                    dL -= lco;
-                    Lls[pos] = 0;
-                }
-                bool queued = false;
-                if (eval && !is_dense(r.ky, r.kn)) {
-                    const int qp = atomicAdd(&qn, 1);
-                    if (qp < qcap) {
-                        copy_rec(&qrec[qp], &r);
-                        queue_tasks(qp, r, l);
-                        qslot[qp] = sl;
-                        qlco[qp] = lco;
-                        qidx[qp] = (short)(ft.lbase[warp][l] + pos);
-                        qwarp[qp] = (signed char)warp;
-                        queued = true;
-                    }
-                }
-                const bool here = eval && !queued;
-                if (__ballot_sync(kFull, here)) {
-                    leaf_parents_eval(c, s, b, here, l, lane);
-                    if (here) {
-                        const Key kb = b.rb[lane];
-                        f.lb[l][sl] = kb;
-                        f.lc[l][sl] = b.rc[lane];
-                        Lls[pos] = kb.s;
-                        dL += b.rc[lane] - lco;
-                        if (kb.s != 0 && key_better(kb, best)) best = kb;
-                    }
-                    __syncwarp();
-                }
-            }
-            if (hitj >= 0 && key_better(kc, best)) best = kc;
-        }
-        for (u64 k = 0; !use_list && rk + B * ((u64)warp + W * 32ull * kScanIlp * k) < n; ++k) {
-            u32 slot[kScanIlp];
-            u64 sg[kScanIlp], ls[kScanIlp];
-#pragma unroll
-            for (int u = 0; u < kScanIlp; ++u) {
-                const u64 i = rk + B * ((u64)warp + W * ((u64)lane + 32ull * (kScanIlp * k + u)));
-                slot[u] = 0;
-                sg[u] = ls[u] = 0;
-                if (i < n) {
-                    slot[u] = front_slot(f.cap[l], soff, (u32)i);
-                    sg[u] = force ? ~0ull : __ldcg(f.sig[l] + slot[u]);
-                    if (leafp && !force) ls[u] = __ldcg(&f.lb[l][slot[u]].s);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kScanIlp; ++u) {
-                const bool dirty = sg[u] != 0 && (force || (sg[u] & csig) != 0);
-                bool cached = leafp && sg[u] != 0 && !dirty;
-                if (__ballot_sync(kFull, dirty) || build_list) {
-                    Rec &r = b.r[lane];
-                    bool changed = false;
-                    int kyn = 0;
-                    u64 lco = 0;
-                    u64 nsg = sg[u];  // the record's signature after this round
-                    if (dirty) {
-                        load_rec(&r, f.F[l] + slot[u]);
-                        if (leafp && !force) lco = __ldcg(f.lc[l] + slot[u]);
-                        const int kyo = force ? 0 : (int)r.ky;  // nothing counted before round 0
-                        changed = refresh_record(c, Ush, Csh, l, r, force);
-                        kyn = r.ky;
-                        if (force && leafp && l <= kPadGenes) {  // the key genes, once
-                            u16 *po = pad_po(r);
-                            for (int q = 0; q < l; ++q) {
-                                const u16 v = c.orig[prefix_gene(r.p, q)];
-                                int k = q - 1;
-                                while (k >= 0 && po[k] > v) {
-                                    po[k + 1] = po[k];
-                                    --k;
-                                }
-                                po[k + 1] = v;
-                            }
-                        }
-                        if (changed) {
-                            nsg = kyn >= 2 ? sample_sig(r) : 0ull;
-                            f.sig[l][slot[u]] = nsg;
-                            copy_rec(f.F[l] + slot[u], &r);
-                            if (l >= 2) {
-                                const u64 fo = kyo >= 2 ? (u64)(kyo - 1) : 0ull, fn = kyn >= 2 ? (u64)(kyn - 1) : 0ull;
-                                dA += fn - fo;
-                                dV += (fn - fo) * (u64)(hiN - prefix_gene(r.p, l - 1));
-                            }
-                        } else {
-                            cached = leafp;  // nothing covered in it after all
-                        }
-                    }
-                    const bool eval = leafp && changed && kyn >= 2;
-                    if (leafp && changed && kyn < 2) {  // no longer shared: no leaf with TP >= 2
-                        f.lb[l][slot[u]] = key_empty();
-                        f.lc[l][slot[u]] = 0;
-                        dL -= lco;
-                    }
-                    // the warp's list: the records still live after this round, with their
-                    // cached best scores (a changed leaf parent's is set when it is evaluated)
-                    int lpos = -1;
-                    if (build_list) {
-                        const bool keep = nsg != 0;
-                        const unsigned km = __ballot_sync(kFull, keep);
-                        if (lfill + __popc(km) > kList) {
-                            lfit = false;
-                        } else if (lfit) {
-                            if (keep) {
-                                lpos = lfill + __popc(km & ((1u << lane) - 1u));
-                                lv.slot[warp][lpos] = slot[u];
-                                lv.sig[warp][lpos] = nsg;
-                                lv.ls[warp][lpos] = leafp && !changed ? ls[u] : 0ull;
-                            }
-                            lfill += __popc(km);
-                        }
-                    }
-                    // changed leaf parents go to the block's queue (spread over its warps
-                    // below); what does not fit is evaluated by this warp
-                    bool queued = false;
-                    if (eval && !force && !is_dense(r.ky, r.kn)) {
-                        const int pos = atomicAdd(&qn, 1);
-                        if (pos < qcap) {
-                            copy_rec(&qrec[pos], &r);
-                            queue_tasks(pos, r, l);
-                            qslot[pos] = slot[u];
-                            qlco[pos] = lco;
-                            qidx[pos] = (short)lpos;
-                            qwarp[pos] = (signed char)warp;
-                            queued = true;
-                        }
-                    }
-                    const bool here = eval && !queued;
-                    if (__ballot_sync(kFull, here)) {
-                        leaf_parents_eval(c, s, b, here, l, lane);
-                        if (here) {
-                            const Key kb = b.rb[lane];
-                            f.lb[l][slot[u]] = kb;
-                            f.lc[l][slot[u]] = b.rc[lane];
-                            if (lpos >= 0) lv.ls[warp][lpos] = kb.s;
-                            dL += b.rc[lane] - lco;
-                            if (kb.s != 0 && key_better(kb, best)) best = kb;
-                        }
-                        __syncwarp();
-                    }
-                }
-                if (cached && ls[u] != 0 && ls[u] >= best.s) {  // unchanged: its cached best
-                    Key kc;
-                    kc.s = ls[u];
-                    kc.t0 = __ldcg(&f.lb[l][slot[u]].t0);
-                    kc.t1 = __ldcg(&f.lb[l][slot[u]].t1);
-                    kc.t2 = __ldcg(&f.lb[l][slot[u]].t2);
-                    if (key_better(kc, best)) best = kc;
-                }
-            }
-        }
-        if (leafp) {
-            // the queued leaf parents: their (record, column word) items spread over all
-            // warps of the block, in tasks of up to 32 items of one record; a record's
-            // best leaf (packed) and its sum of TP - 1 meet in shared memory
-            __syncthreads();
-            const int nq = qn < qcap ? qn : qcap;
-            if (nq > 0) {
-                // every warp forms the records' task prefix itself (nq <= 64: two chunks)
-                const int i0 = lane < nq ? qtasks[lane] : 0, i1 = lane + 32 < nq ? qtasks[lane + 32] : 0;
-                const int inc0 = warp_incl_scan(i0, lane);
-                const int inc1 = __shfl_sync(kFull, inc0, 31) + warp_incl_scan(i1, lane);
-                const int T = __shfl_sync(kFull, inc1, 31), nwg = ((c.G - 1) >> 6) + 1;
-                for (int tau = warp; tau < T; tau += nwarps) {
-                    // its record: the number of records whose tasks end at or before tau
-                    const int j = __popc(__ballot_sync(kFull, lane < nq && inc0 <= tau)) +
-                                  __popc(__ballot_sync(kFull, lane + 32 < nq && inc1 <= tau));
-                    const int e0 = __shfl_sync(kFull, inc0, (j - 1) & 31), e1 = __shfl_sync(kFull, inc1, (j - 33) & 31);
-                    const int first = j == 0 ? 0 : (j <= 32 ? e0 : e1);
-                    const int lo = qlo[j];
-                    const int it = (tau - first) * 32 + lane, wi = (lo >> 6) + it;
-                    u64 pk = 0, corr = 0;
-                    if (wi < nwg) leaf_item_eval(c, s, qrec[j], wi, range_word(wi, lo, c.G - 1), corr, pk);
-                    pk = warp_max_u64(pk);
-                    const u32 cs = __reduce_add_sync(kFull, (u32)corr);
-                    if (lane == 0) {
-                        if (pk) atomicMax(&qbest[j], pk);
-                        if (cs) atomicAdd(&qcorr[j], cs);
-                    }
-                }
-                __syncthreads();
-                const int j = (int)threadIdx.x;
-                if (j < nq) {
-                    Key kb = key_empty();
-                    if (qbest[j]) {
-                        int po[kMaxH - 1];
-                        record_po(c, qrec[j], l, po);
-                        kb = unpack_leaf(qbest[j], po, l);
-                    }
-                    f.lb[l][qslot[j]] = kb;
-                    f.lc[l][qslot[j]] = qcorr[j];
-                    if (kLWarps > 0 && qidx[j] >= 0) lv.ls[qwarp[j]][qidx[j]] = kb.s;
-                    dL += qcorr[j] - qlco[j];
-                    if (kb.s != 0 && key_better(kb, best)) best = kb;
-                }
-            }
-        }
-        if (build_list && lane == 0) ft.lcnt[warp][l] = (short)(lfill - ft.lbase[warp][l]);
-        dA = warp_sum_u64(dA);
-        dV = warp_sum_u64(dV);
-        dL = warp_sum_u64(dL);
-        if (lane == 0) {
-            deep_add(2 * l + 1, dA);
-            deep_add(2 * (l + 1), dV);
-            deep_add(2 * h + 1, dL);
-        }
-    }
-    if (build_list && lane == 0) ft.lok[warp] = lfit ? 1 : 0;
-    // one block barrier, then three jobs on three warps: the block's best to its slot
-    // (first, the round's grid barrier waits for it), the depths' correction changes
-    // to the round's counters, the phase's warp cycles to the diagnostics
-    Key *wkey = warp_keys();
-    warp_cycles(acc, t0, lane);
-    {
-        const Key wb = warp_max_key(best);
-        if (lane == 0) wkey[warp] = wb;
-    }
-    __syncthreads();
-    if (warp == 0) {
-        const Key k = warp_max_key(lane < nwarps ? wkey[lane] : key_empty());
-        if (lane == 0 && io.overwrite) {
-            io.slots[t.rank] = k;
-        } else if (lane == 0 && k.s != 0) {
-            const Key old = io.slots[t.rank];
-            if (key_better(k, old)) io.slots[t.rank] = k;
-        }
-    }
-    if (warp == (nwarps > 1 ? 1 : 0)) {  // deep[i], i = 2e and 2e + 1 for depths e = 1 .. h
-        const int i = lane + 2;
-        if (i <= 2 * h + 1) {
-            u64 d = deep[i];
-            if (kLWarps > 0) {
-#pragma unroll 4
-                for (int w = 0; w < nwarps; ++w) d += wdeep[w][i];
-            }
-            if (d) atomicAdd(s.cnt + ((size_t)round * h + (i / 2 - 1)) * 2 + (i & 1), d);
-        }
-    }
-    if (warp == (nwarps > 2 ? 2 : nwarps - 1)) {
-        const u64 v = lane < nwarps ? warp_cycle_slots()[lane] : 0ull;
-        const u64 sum = warp_sum_u64(v), mx = warp_max_u64(v);
-        if (lane == 0) {
-            atomicAdd(s.work + kWorkWarpSum + 1, sum);
-            atomicMax(s.work + (io.par ? kWorkWarpMaxOdd : kWorkWarpMax) + 1, mx);
-            atomicAdd(s.work + kWorkWarpN + 1, (u64)nwarps);
-        }
-    }
-    return true;
-}
+#include "mh_levels.cuh"
 
 // End of round r of the persistent solve, run by EVERY block of the team on the
 // same inputs, so that all of them reach the same decisions without another
@@ -2883,160 +2117,155 @@ __device__ bool end_of_round(const Cohort &c, const Solve &s, int round, const K
     return done;
 }
 
-// End of an incremental round, by every block on the same inputs: warp 0 alone
-// reduces the blocks' slots to the winner, computes its TP / FP and the tumors it
-// covers, applies DelCols to the block's copy of U and keeps the covered tumors
-// (Csh) for the next round's update.  The lead block (rank 0) also records the
-// selection and finishes the round's counters: depth 1 from its surviving count,
-// depths 2..h as the per-sample sums over all tumors (tot) minus the running
-// totals (run, to which it adds the round's changes, read together with the
-// slots): the corrections, and the per-sample sums of the tumors covered so far,
-// which each round's update adds for the tumors the last winner covered.  kk: the lead's
-// count of selections; maxr: the round limit.  Returns true when the solve is done.
-__device__ bool end_of_round_inc(const Cohort &c, const Solve &s, int round, const Key *slots, int nslots,
-                                 const Team &t, u64 *Ush, const u64 *tot, u64 *Csh, u64 *run, int *kk, int maxr)
-{
-    __shared__ int os[kMaxH];
-    __shared__ int done_sh;
-    Key *wbest = warp_keys();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int h = s.h;
-    const bool lead = t.rank == 0;
-    {  // the slots, one per thread (all loads of a thread in flight together)
-        Key best = key_empty();
-        for (int i = (int)threadIdx.x; i < nslots; i += (int)blockDim.x) {
-            Key k;
-            k.s = __ldcg(&slots[i].s);
-            k.t0 = __ldcg(&slots[i].t0);
-            k.t1 = __ldcg(&slots[i].t1);
-            k.t2 = __ldcg(&slots[i].t2);
-            if (key_better(k, best)) best = k;
-        }
-        best = warp_max_key(best);
-        if (lane == 0) wbest[warp] = best;
-    }
-    __syncthreads();
-    if (warp == 0) {
-        u64 dv = 0, da = 0;
-        u64 *cv = s.cnt + ((size_t)round * h + lane) * 2;
-        if (lead && lane < h) {
-            dv = __ldcg(cv);
-            da = __ldcg(cv + 1);
-        }
-        const Key best = warp_max_key(lane < nwarps ? wbest[lane] : key_empty());
-        bool done = true;
-        u64 ycov = 0;
-        if (best.s != 0) {
-            if (lane < h) os[lane] = key_get(best, lane);
-            __syncwarp();
-            const u64 *TR = c.TO ? c.TO : c.T;
-            const u64 *NR = c.TO ? c.NO : c.N;
-            int ri[kMaxH];
-#pragma unroll
-            for (int i = 0; i < kMaxH; ++i) ri[i] = i < h ? (c.TO ? os[i] : (int)c.inv[os[i]]) : 0;
-            u64 y = 0, n = 0, u = 0;
-            if (lane < c.Wt) {
-                u = Ush[lane];
-                y = u;
-#pragma unroll
-                for (int i = 0; i < kMaxH; ++i)
-                    if (i < h) y &= __ldg(TR + (size_t)ri[i] * c.WTp + lane);
-            }
-            if (lane < c.Wn) {
-                n = ~0ull;
-#pragma unroll
-                for (int i = 0; i < kMaxH; ++i)
-                    if (i < h) n &= __ldg(NR + (size_t)ri[i] * c.WNp + lane);
-            }
-            const int tp = (int)__reduce_add_sync(kFull, (unsigned)__popcll(y));
-            const int fp = (int)__reduce_add_sync(kFull, (unsigned)__popcll(n));
-            if (lane < c.Wt) {
-                ycov = y;
-                u &= ~y;
-                Ush[lane] = u;
-                s.U[lane] = u;
-            }
-            const unsigned left = __ballot_sync(kFull, u != 0);
-            done = !left || round + 1 >= maxr;
-            if (lead && lane == 0) {
-                const int k = *kk;
-                int *r = s.res + (size_t)k * (h + 2);
-                for (int i = 0; i < h; ++i) r[i] = os[i];
-                r[h] = tp;
-                r[h + 1] = fp;
-                s.state[kStK] = k + 1;
-                *kk = k + 1;
-            }
-        }
-        if (lead && lane < h) {
-            const int l = lane + 1;
-            run[2 * l] += dv;
-            run[2 * l + 1] += da;
-            u64 vis, alive;
-            if (l == 1) {
-                vis = c.G >= h ? (u64)(c.G - h + 1) : 0ull;
-                alive = run[3];
-            } else {
-                vis = tot[h + lane] - run[2 * l];
-                alive = tot[lane] - run[2 * l + 1];
-            }
-            cv[0] = vis;
-            cv[1] = vis - alive;
-            s.run[2 * l] = run[2 * l];
-            s.run[2 * l + 1] = run[2 * l + 1];
-        }
-        Csh[lane] = ycov;  // kMaxWords == 32 words, one per lane
-        if (lead && lane < c.WTp) s.cov[lane] = ycov;
-        if (lane == 0) {
-            done_sh = done;
-            if (lead) {
-                s.state[kStRound] = round + 1;
-                if (done) s.state[kStDone] = 1;
-            }
-        }
-    }
-    __syncthreads();
-    return done_sh != 0;
-}
+// The greedy loop of one cohort run by a team of co-resident blocks.  Where every
+// tumor's champion is known the solve goes by score levels (solve_levels); otherwise a
+// round is the depth-2 .. h-1 expansions (depth 1 built on the fly from the gene rows),
+// the leaves, a barrier, and the end of round computed redundantly by every block, so
+// rounds are separated by h - 1 barriers.  Data indexed by round parity: the slots the
+// blocks' bests go to, the frontier counters and the threshold word; rank 0 clears the
+// next round's set at the start of a round (all reads of it ended before the previous
+// round's last barrier).  Returns when the solve is done, a frontier overflowed, a
+// barrier timed out (recorded in the cohort's state) or, in a batch, the barrier that
+// ended a round carried a yield request.
 
-// The greedy loop of one cohort run by a team of co-resident blocks.  A round is
-// the depth-2 .. h-1 expansions (depth 1 built on the fly from the gene rows), the
-// leaves, a barrier, and the end of round computed redundantly by every block, so
-// rounds are separated by h - 1 barriers.  Data indexed by round parity: the slots
-// the blocks' bests go to, the frontier counters and the threshold word; rank 0
-// clears the next round's set at the start of a round (all reads of it ended
-// before the previous round's last barrier).  Returns when the solve is done, a
-// frontier overflowed, a barrier timed out (recorded in the cohort's state) or,
-// in a batch, the barrier that ended a round carried a yield request.
-template <int kQueue, int kLWarps>
-__device__ void solve_team(const Cohort &c, const Solve &s, const Frontiers &f, GridSync *gsync, u32 *counts_base,
-                           const Team &t, Batch &b, int *yield = nullptr)
-{
-    __shared__ u64 Ush[kMaxWords];
-    __shared__ Key cand_sh[kCandidates];
-    __shared__ u64 tot[2 * kMaxH];
-    __shared__ u64 Csh[kMaxWords];
-    __shared__ u64 run[2 * (kMaxH + 1)];  // incremental rounds, rank 0: the corrections' running totals
-    __shared__ FrontTab ftab;
-    __shared__ int fm_sh, kk_sh;
-    const int h = s.h;
-    const bool timer = t.rank == 0 && threadIdx.x == 0;
-    u64 tm = timer ? global_ns() : 0;
-    auto lap = [&](int phase) {
-        if (timer) {
+// The time since `tm` goes to a phase's total (block 0, thread 0).
+struct PhaseTimer {
+    bool on;
+    u64 tm;
+    __device__ void lap(const Solve &s, int phase)
+    {
+        if (on) {
             const u64 now = global_ns();
             atomicAdd(s.work + kWorkPhaseNs + phase, now - tm);
             tm = now;
         }
+    }
+};
+
+// The solve by score levels (mh_levels.cuh): the kept frontiers are built and every leaf
+// parent is evaluated once; then one grid barrier per level, the members of the level
+// gathered before it and its picks made after it by every block alike; then the rounds
+// and their counters.  A launch may end between two levels (a yield request, or members
+// that outgrew their buffer, the level then being searched again): s.state holds the
+// step to go on with, s.U, s.sel, s.covsel and the bounds the rest.
+template <bool kBig>
+__device__ void solve_levels(const Cohort &c, const Solve &s, const Frontiers &f, GridSync *gsync, u32 *counts,
+                             const Team &t, Batch *scratch, u64 *Ush, int maxr, PhaseTimer &pt, int *yield)
+{
+    __shared__ LevelSh<kBig> sh;
+    __shared__ FrontTab ft;
+    Batch &b = scratch[threadIdx.x >> 5];
+    const int h = s.h;
+    const bool lead = t.rank == 0;
+    auto end_early = [&](int word, int value, int step, u64 level = 0) {
+        if (lead && threadIdx.x == 0) {
+            s.state[word] = value;
+            s.state[kStStep] = step;  // +-(i + 1): go on with step i (again) at this level
+            if (step) s.lev->lmax[((step < 0 ? -step : step) - 1) & 3] = level;
+            if (yield && word == kStOverflow) {  // the other teams stop too, so that the host can act
+                *(volatile int *)yield = 1;
+                __threadfence_system();
+            }
+        }
     };
+    const int step0 = *(volatile int *)&s.state[kStStep];
+    if (step0 == 0) {
+        const RoundIO io{Ush, s.slots, true, s.best_hint, 0, true, true};
+        if (h == 2) {
+            phase_build1(c, s, f, counts, b, t, Ush);
+            if (!grid_sync(gsync, s.state, t.size)) return;
+        }
+        for (int l = 2; l <= h - 1; ++l) {
+            if (!phase_expand(c, s, 0, l, f, counts, b, t, io)) {
+                end_early(kStOverflow, kOverFrontier, 0);
+                return;
+            }
+            if (!grid_sync(gsync, s.state, t.size)) return;
+        }
+    }
+    if (!front_table(f, counts, h, ft, b)) {
+        end_early(kStOverflow, kOverFrontier, 0);
+        return;
+    }
+    int step = 0, K = 0;
+    bool rerun = false;
+    if (step0 == 0) {
+        pt.lap(s, 1);
+        level_first<kBig>(c, s, f, sh, b, t, ft, Ush);
+        if (!grid_sync(gsync, s.state, t.size)) return;
+    } else {
+        step = (step0 < 0 ? -step0 : step0) - 1;
+        rerun = step0 < 0;
+        K = *(volatile int *)&s.state[kStK];
+    }
+    u64 Lk = __ldcg(&s.lev->lmax[step & 3]);
+    bool left;
+    for (;;) {
+        left = __syncthreads_or(threadIdx.x < kMaxWords && Ush[threadIdx.x] != 0) != 0;
+        if (Lk == 0 || !left || K >= maxr) break;
+        level_search<kBig>(c, s, f, sh, b, t, ft, Ush, Lk, step, rerun);
+        if (!grid_sync(gsync, s.state, t.size, yield)) return;
+        const bool stop = yield && *(volatile int *)&gsync->flag;
+        const u32 n = __ldcg(&s.lev->mcnt[step & 3]);
+        const u64 Ln = __ldcg(&s.lev->lmax[(step + 1) & 3]);
+        if (n > s.mcap) {
+            end_early(kStOverflow, kOverMembers, -(step + 1), Lk);
+            return;
+        }
+        u64 fallen;
+        const int got = level_select<kBig>(c, s, sh, reinterpret_cast<u64 *>(scratch), Ush, (int)n, Lk, step, K, lead,
+                                           fallen);
+        const u64 Lnext = Ln > fallen ? Ln : fallen;
+        K += got;
+        if (lead && threadIdx.x == 0) s.state[kStK] = K;
+        if (got == 0 && Lnext >= Lk) {  // cannot be: a step picks or goes down (no endless loop in any case)
+            if (lead && threadIdx.x == 0) s.state[kStError] = kErrTimeout;
+            return;
+        }
+        Lk = Lnext;
+        ++step;
+        rerun = false;
+        if (stop && Lk != 0) {
+            end_early(kStYield, 1, step + 1, Lk);
+            return;
+        }
+    }
+    pt.lap(s, 2);
+    if (!grid_sync(gsync, s.state, t.size)) return;  // the picks are complete
+    const int kept = K < maxr ? K : maxr;
+    const int R = !left && K <= maxr ? K : (K + 1 < maxr ? K + 1 : maxr);  // a last round may find nothing
+    level_rounds(c, s, t, K, R, maxr);
+    if (!grid_sync(gsync, s.state, t.size)) return;
+    level_counts<kBig>(c, s, f, sh, b, t, ft, R);
+    if (!grid_sync(gsync, s.state, t.size)) return;
+    if (!lead) return;
+    level_counts_end(c, s, R);
+    if (threadIdx.x == 0) {
+        s.state[kStK] = kept;
+        s.state[kStRound] = R;
+        s.state[kStDone] = 1;
+        if (yield) {  // the others stop after their level: the host hands out these blocks again
+            *(volatile int *)yield = 1;
+            __threadfence_system();
+        }
+    }
+    pt.lap(s, 3);
+}
+
+template <bool kBig>
+__device__ void solve_team(const Cohort &c, const Solve &s, const Frontiers &f, GridSync *gsync, u32 *counts_base,
+                           const Team &t, Batch *scratch, int *yield = nullptr)
+{
+    __shared__ u64 Ush[kMaxWords];
+    __shared__ Key cand_sh[kCandidates];
+    __shared__ int fm_sh;
+    Batch &b = scratch[threadIdx.x >> 5];
+    const int h = s.h;
+    const bool timer = t.rank == 0 && threadIdx.x == 0;
+    PhaseTimer pt{timer, timer ? global_ns() : 0};
     if (*(volatile int *)&s.state[kStDone] | *(volatile int *)&s.state[kStError]) return;
     int round = *(volatile int *)&s.state[kStRound];
     const int maxr = *(volatile int *)&s.state[kStMaxRounds];
-    for (int w = (int)threadIdx.x; w < kMaxWarpsPerBlock; w += (int)blockDim.x) ftab.lok[w] = 0;
-    if (threadIdx.x == 0) {
-        ftab.ok = 0;
-        kk_sh = *(volatile int *)&s.state[kStK];
-    }
     // start of a launch: U and the candidates left by the previous round
     for (int i = threadIdx.x; i < kMaxWords; i += blockDim.x) Ush[i] = i < c.WTp ? __ldcg(&s.U[i]) : 0ull;
     for (int i = threadIdx.x; i < kCandidates; i += blockDim.x) {
@@ -3046,39 +2275,36 @@ __device__ void solve_team(const Cohort &c, const Solve &s, const Frontiers &f, 
         cand_sh[i].t2 = __ldcg(&s.cand[i].t2);
     }
     __syncthreads();
-    if (h > 1 && t.rank == 0) block_rescore(c, s, cand_sh, Ush, s.best_hint + (round & 1));
-    if (h > 1 && round == 0 && s.prune != MH_PRUNE_OFF && c.CC) {
-        // the champions and the first round's threshold, complete before any block
-        // starts searching
-        if (s.champ && s.prune == MH_PRUNE_PAPER) phase_champions(c, s, t, b);
-        if (s.ssum && s.prune == MH_PRUNE_PAPER) phase_sample_sums(c, s, t);
-        block_seed(c, s, t, Ush, s.best_hint);
-        if (!grid_sync(gsync, s.state, t.size)) return;
-    }
-    // counting by per-sample sums when every tumor's champion is known (the
-    // champions stand for the TP = 1 leaves that this mode never visits)
-    bool fm = false;
+    // by levels when every tumor's champion is known (the champions stand for the TP = 1
+    // leaves, which that path never visits)
     if (h > 1 && s.prune == MH_PRUNE_PAPER && c.CC && s.champ && s.ssum) {
-        if (threadIdx.x == 0) fm_sh = 1;
+        if (round == 0 && *(volatile int *)&s.state[kStStep] == 0) {
+            phase_champions(c, s, t, b);
+            phase_sample_sums(c, s, t);
+            if (!grid_sync(gsync, s.state, t.size)) return;
+        }
+        // (the smallest tuples per tumor take the batch scratch)
+        if (threadIdx.x == 0) fm_sh = (size_t)((h + 3) / 4) * c.Nt * sizeof(u64) <= sizeof(Batch) * (blockDim.x >> 5);
         __syncthreads();
         for (int i = threadIdx.x; i < c.Nt; i += blockDim.x)
             if (!__ldcg(s.champ_ok + i)) fm_sh = 0;
         __syncthreads();
-        fm = fm_sh != 0;
-        if (fm && t.rank == 0) block_sample_totals(c, s, tot);
-        // incremental rounds: the tumors covered by the last round's winner
-        for (int i = threadIdx.x; i < kMaxWords; i += blockDim.x)
-            Csh[i] = (fm && round > 0 && i < c.WTp) ? __ldcg(&s.cov[i]) : 0ull;
-        for (int i = threadIdx.x; i < 2 * (kMaxH + 1); i += blockDim.x)
-            run[i] = (fm && round > 0) ? __ldcg(s.run + i) : 0ull;
-        __syncthreads();
+        if (fm_sh) {
+            solve_levels<kBig>(c, s, f, gsync, counts_base, t, scratch, Ush, maxr, pt, yield);
+            return;
+        }
+    }
+    if (h > 1 && t.rank == 0) block_rescore(c, s, cand_sh, Ush, s.best_hint + (round & 1));
+    if (h > 1 && round == 0 && s.prune != MH_PRUNE_OFF && c.CC) {
+        // the first round's threshold, complete before any block starts searching
+        block_seed(c, s, t, Ush, s.best_hint);
+        if (!grid_sync(gsync, s.state, t.size)) return;
     }
     for (;;) {
         const int par = round & 1;
-        // incremental rounds keep round 0's frontiers and their counts (set 0)
-        u32 *counts = counts_base + (size_t)(fm ? 0 : par) * kCountWords;
-        const RoundIO io{Ush, s.slots + (size_t)par * s.nslots, true, s.best_hint + par, par, fm, fm};
-        if (t.rank == 0 && !fm) {  // the next round's counters and threshold start from zero
+        u32 *counts = counts_base + (size_t)par * kCountWords;
+        const RoundIO io{Ush, s.slots + (size_t)par * s.nslots, true, s.best_hint + par, par, false, false};
+        if (t.rank == 0) {  // the next round's counters and threshold start from zero
             u32 *cn = counts_base + (size_t)(par ^ 1) * kCountWords;
             for (int i = threadIdx.x; i < kMaxH * kShards; i += blockDim.x) cn[i * kShardStride] = 0;
             if (threadIdx.x == 0) *(volatile u64 *)(s.best_hint + (par ^ 1)) = 0;
@@ -3088,7 +2314,7 @@ __device__ void solve_team(const Cohort &c, const Solve &s, const Frontiers &f, 
         // and relaunch without leaving the team's blocks idle
         auto overflow = [&]() {
             if (t.rank == 0 && threadIdx.x == 0) {
-                s.state[kStOverflow] = 1;
+                s.state[kStOverflow] = kOverFrontier;
                 if (yield) {
                     *(volatile int *)yield = 1;
                     __threadfence_system();
@@ -3097,27 +2323,7 @@ __device__ void solve_team(const Cohort &c, const Solve &s, const Frontiers &f, 
         };
         if (h == 1) {
             phase_level1(c, s, round, f, counts, t, io);
-            lap(0);
-        } else if (fm) {
-            // round 0 builds the kept frontiers; every round then updates them
-            if (round == 0) {
-                if (h == 2) {
-                    phase_build1(c, s, f, counts, b, t, Ush);
-                    if (!grid_sync(gsync, s.state, t.size)) return;
-                }
-                for (int l = 2; l <= h - 1; ++l) {
-                    if (!phase_expand(c, s, round, l, f, counts, b, t, io)) {
-                        overflow();
-                        return;
-                    }
-                    if (!grid_sync(gsync, s.state, t.size)) return;
-                }
-            }
-            lap(1);
-            if (!phase_update<kQueue, kLWarps>(c, s, round, f, counts, b, t, io, Csh, round == 0, ftab)) {
-                overflow();
-                return;
-            }
+            pt.lap(s, 0);
         } else {
             // every block reads the same shard counts after the same barrier, so an
             // overflow is seen by all of them and they leave together
@@ -3128,7 +2334,7 @@ __device__ void solve_team(const Cohort &c, const Solve &s, const Frontiers &f, 
                 }
                 if (!grid_sync(gsync, s.state, t.size)) return;
             }
-            lap(1);
+            pt.lap(s, 1);
             if (!phase_leaf(c, s, round, f, counts, b, t, io)) {
                 overflow();
                 return;
@@ -3138,10 +2344,9 @@ __device__ void solve_team(const Cohort &c, const Solve &s, const Frontiers &f, 
         // request, so that every block of the team takes the same decision
         if (!grid_sync(gsync, s.state, t.size, yield)) return;
         const bool stop = yield && *(volatile int *)&gsync->flag;
-        lap(2);
-        const bool done = fm ? end_of_round_inc(c, s, round, io.slots, t.size, t, Ush, tot, Csh, run, &kk_sh, maxr)
-                             : end_of_round(c, s, round, io.slots, t.size, t, Ush, cand_sh, s.best_hint + (par ^ 1));
-        lap(3);
+        pt.lap(s, 2);
+        const bool done = end_of_round(c, s, round, io.slots, t.size, t, Ush, cand_sh, s.best_hint + (par ^ 1));
+        pt.lap(s, 3);
         if (done) {
             // batch: a team that finished asks the others to stop after their current
             // round, so that the host can hand its blocks to the unfinished cohorts
@@ -3172,8 +2377,7 @@ __global__ void __launch_bounds__(kWarps * 32, kMinBlocks)
             GridSync *gsync, u32 *counts, int *yield)
 {
     __shared__ Batch scratch[kWarps];
-    solve_team<kMinBlocks == 1 ? kEvalQueue : 0, kMinBlocks == 1 ? kWarps : 0>(c, s, f, gsync, counts, grid_team(),
-                                                                                scratch[threadIdx.x >> 5], yield);
+    solve_team<kMinBlocks == 1>(c, s, f, gsync, counts, grid_team(), scratch, yield);
 }
 
 // SM-major number of the calling block (thread 0): SMs are ranked in the order
@@ -3238,8 +2442,7 @@ __global__ void __launch_bounds__(kWarps * 32, kMinBlocks)
         const int nsm = it.nblocks / map.per_sm;
         t.rank = (t.rank % map.per_sm) * nsm + t.rank / map.per_sm;
     }
-    solve_team<kMinBlocks == 1 ? kEvalQueue : 0, kMinBlocks == 1 ? kWarps : 0>(it.c, it.s, it.f, it.gsync, it.counts, t,
-                                                                                scratch[threadIdx.x >> 5], yield);
+    solve_team<kMinBlocks == 1>(it.c, it.s, it.f, it.gsync, it.counts, t, scratch, yield);
 }
 
 }  // namespace
@@ -3263,6 +2466,8 @@ void launch_solve_init(const Cohort &c, const Solve &s, int counter_rounds, int 
     if (s.cut) cudaMemsetAsync(s.cut, 0, sizeof(u64) * (size_t)s.h * (size_t)counter_rounds, st);
     cudaMemsetAsync(s.slots, 0, sizeof(Key) * (size_t)s.nslots * sets, st);
     cudaMemsetAsync(s.cand, 0, sizeof(Key) * (size_t)kCandidates, st);
+    if (s.lev) cudaMemsetAsync(s.lev, 0, sizeof(Level), st);
+    if (s.covsel) cudaMemsetAsync(s.covsel, 0xff, sizeof(int) * (size_t)c.Nt, st);
     cudaMemsetAsync(s.work, 0, sizeof(u64) * kWorkCount, st);
     cudaMemsetAsync(s.best_hint, 0, sizeof(u64) * sets, st);
     cudaMemsetAsync(counts, 0, sizeof(u32) * kCountWords * sets, st);

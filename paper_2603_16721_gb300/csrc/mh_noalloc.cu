@@ -240,9 +240,12 @@ extern "C" MH_API int mh_solve_noalloc(const uint64_t *d_bitmaps, int32_t G, int
     s.champ = nullptr;  // one kernel per phase: no per-sample champions
     s.champ_ok = nullptr;
     s.ssum = nullptr;
-    s.gk = nullptr;
-    s.cov = nullptr;
-    s.run = nullptr;
+    s.lev = nullptr;
+    s.mem = nullptr;
+    s.mcap = 0;
+    s.sel = nullptr;
+    s.covsel = nullptr;
+    s.cr = nullptr;
     s.cut = nullptr;
     s.shard = 0;
     s.nshards = 1;
@@ -256,7 +259,7 @@ extern "C" MH_API int mh_solve_noalloc(const uint64_t *d_bitmaps, int32_t G, int
     for (int l = 0; l < kMaxH; ++l) {
         fr.F[l] = nullptr;
         fr.cap[l] = 0;
-        fr.sig[l] = nullptr;
+        fr.ub[l] = nullptr;
         fr.lb[l] = nullptr;
         fr.lc[l] = nullptr;
     }

@@ -477,7 +477,7 @@ int ensure_frontier(mh_handle *H, int l, u64 n, bool exact = false)
 size_t level_bytes(int Nt)
 {
     const size_t nt1 = (size_t)std::max(Nt, 1);
-    return 256 + nt1 * (sizeof(Key) + sizeof(int) + sizeof(u16));
+    return kLevelBytes + nt1 * (sizeof(Key) + sizeof(int) + sizeof(u16));
 }
 
 // Room for n members of a level (at least 8192 of them, or MH_FRONTIER_MIN_RECORDS).
@@ -658,9 +658,9 @@ int prepare_solve(mh_handle *H, const mh_solve_opts *opts, Solve *s, int *max_ro
     {
         const size_t nt1 = (size_t)std::max(H->Nt, 1);
         s->lev = (Level *)H->dLevel;
-        s->sel = (Key *)(H->dLevel + 256);
-        s->covsel = (int *)(H->dLevel + 256 + nt1 * sizeof(Key));
-        s->cr = (u16 *)(H->dLevel + 256 + nt1 * (sizeof(Key) + sizeof(int)));
+        s->sel = (Key *)(H->dLevel + kLevelBytes);
+        s->covsel = (int *)(H->dLevel + kLevelBytes + nt1 * sizeof(Key));
+        s->cr = (u16 *)(H->dLevel + kLevelBytes + nt1 * (sizeof(Key) + sizeof(int)));
         s->mem = H->dMem;
         s->mcap = H->mcap;
     }
@@ -686,7 +686,6 @@ int grow_members(mh_handle *H, Solve *s, cudaStream_t st)
     if (rc) return rc;
     s->mem = H->dMem;
     s->mcap = H->mcap;
-    MH_CUDA(cudaMemsetAsync(s->lev->mcnt, 0, sizeof lev.mcnt, st));
     MH_CUDA(cudaMemsetAsync(s->state + 3, 0, sizeof(int), st));
     return MH_OK;
 }

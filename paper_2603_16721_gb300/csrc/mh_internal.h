@@ -107,8 +107,9 @@ struct StoreBuild {
     u64 *GS;
 };
 
-// A combination of the level being resolved: its tuple (as in Key), the k uncovered
-// tumors it covers, listed when few (else its rows give them).
+// A combination of the band being resolved: its tuple (as in Key; FP and TP in the low
+// bits of t2), the k = TP uncovered tumors it covers, listed when few (else its rows give
+// them).
 constexpr int kMemIds = 18;
 struct __align__(16) Member {
     u64 t0, t1, t2;
@@ -118,12 +119,18 @@ struct __align__(16) Member {
 };
 static_assert(sizeof(Member) == 64, "members are 64 bytes, read as four 16-byte words");
 
-// Step i of a solve by levels finds its level (score + 1) in lmax[i & 3] and counts its
+// Step i of a solve by levels finds the top of its band (score + 1) in lmax[i & 3] and the
+// number of bounds by their distance to the last band's top in tally[i & 3], and counts its
 // members in mcnt[i & 3]; step i - 2 clears the entries.
+constexpr int kTally = 16;     // distances 1, 2, 3, 4, 6, 8, ... 192, 256 (units of a_num)
+constexpr int kTallyMost = 256;
 struct Level {
     u64 lmax[4];
     u32 mcnt[4];
+    u32 tally[4][kTally];
 };
+constexpr size_t kLevelBytes = 512;
+static_assert(sizeof(Level) <= kLevelBytes, "the picks follow");
 // Solve::state word 3: what outgrew its memory.
 constexpr int kOverFrontier = 1, kOverMembers = 2;
 

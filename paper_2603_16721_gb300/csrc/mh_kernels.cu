@@ -2160,8 +2160,8 @@ __device__ void solve_levels(const Cohort &c, const Solve &s, const Frontiers &f
     auto end_early = [&](int word, int value, int step, u64 level = 0) {
         if (lead && threadIdx.x == 0) {
             s.state[word] = value;
-            s.state[kStStep] = step;  // +-(i + 1): go on with step i (again) at this level
-            if (step) s.lev->lmax[((step < 0 ? -step : step) - 1) & 3] = level;
+            s.state[kStStep] = step;  // i + 1: go on with step i, at this level
+            if (step) s.lev->lmax[(step - 1) & 3] = level;
             if (yield && word == kStOverflow) {  // the other teams stop too, so that the host can act
                 *(volatile int *)yield = 1;
                 __threadfence_system();
@@ -2188,43 +2188,65 @@ __device__ void solve_levels(const Cohort &c, const Solve &s, const Frontiers &f
         return;
     }
     int step = 0, K = 0;
-    bool rerun = false;
     if (step0 == 0) {
         pt.lap(s, 1);
         level_first<kBig>(c, s, f, sh, b, t, ft, Ush);
         if (!grid_sync(gsync, s.state, t.size)) return;
     } else {
-        step = (step0 < 0 ? -step0 : step0) - 1;
-        rerun = step0 < 0;
+        step = step0 - 1;
         K = *(volatile int *)&s.state[kStK];
     }
     u64 Lk = __ldcg(&s.lev->lmax[step & 3]);
+    u64 ref = Lk;        // the top that the tally counts from
+    bool wide = true;    // whether the band may take more than the top level
     bool left;
+    if (step0 == 0 && s.a_num) {
+        level_tally<kBig>(s, f, sh, t, ft, Lk, 0);
+        if (!grid_sync(gsync, s.state, t.size)) return;
+    } else {
+        wide = false;
+    }
     for (;;) {
         left = __syncthreads_or(threadIdx.x < kMaxWords && Ush[threadIdx.x] != 0) != 0;
         if (Lk == 0 || !left || K >= maxr) break;
-        level_search<kBig>(c, s, f, sh, b, t, ft, Ush, Lk, step, rerun);
+        // the band: down to the farthest distance with at most 64 bounds per block (one record
+        // to evaluate makes a step of 15 us, 16 of them one of 18 us, and most bounds only have
+        // to be lowered)
+        u64 tau = Lk;
+        if (wide && s.a_num) {
+            u32 sum = 0;
+            for (int q = 0; q < kTally; ++q) {
+                sum += __ldcg(&s.lev->tally[step & 3][q]);
+                const u64 w = s.a_num * tally_width(q);
+                if (sum > 64u * (u32)t.size || w >= 1ull << 23) break;
+                const u64 x = ref > w ? ref - w : 1ull;
+                if (x < tau) tau = x;
+            }
+        }
+        level_search<kBig>(c, s, f, sh, b, t, ft, Ush, Lk, tau, step);
         if (!grid_sync(gsync, s.state, t.size, yield)) return;
         const bool stop = yield && *(volatile int *)&gsync->flag;
         const u32 n = __ldcg(&s.lev->mcnt[step & 3]);
         const u64 Ln = __ldcg(&s.lev->lmax[(step + 1) & 3]);
-        if (n > s.mcap) {
-            end_early(kStOverflow, kOverMembers, -(step + 1), Lk);
+        ref = Lk;
+        if (n > s.mcap && tau == Lk) {  // the level is searched again with larger buffers
+            end_early(kStOverflow, kOverMembers, step + 2, Lk);
             return;
         }
-        u64 fallen;
-        const int got = level_select<kBig>(c, s, sh, reinterpret_cast<u64 *>(scratch), Ush, (int)n, Lk, step, K, lead,
-                                           fallen);
-        const u64 Lnext = Ln > fallen ? Ln : fallen;
-        K += got;
-        if (lead && threadIdx.x == 0) s.state[kStK] = K;
-        if (got == 0 && Lnext >= Lk) {  // cannot be: a step picks or goes down (no endless loop in any case)
-            if (lead && threadIdx.x == 0) s.state[kStError] = kErrTimeout;
-            return;
-        }
-        Lk = Lnext;
+        wide = n <= s.mcap;
+        if (wide) {
+            u64 fallen;
+            const int got = level_select<kBig>(c, s, sh, scratch, Ush, (int)n, Lk, tau, step, K, lead, fallen);
+            const u64 Lnext = Ln > fallen ? Ln : fallen;
+            K += got;
+            if (lead && threadIdx.x == 0) s.state[kStK] = K;
+            if (got == 0 && Lnext >= Lk) {  // cannot be: a step picks or goes down (no endless loop in any case)
+                if (lead && threadIdx.x == 0) s.state[kStError] = kErrTimeout;
+                return;
+            }
+            Lk = Lnext;
+        }  // else too many members: the top level alone, next
         ++step;
-        rerun = false;
         if (stop && Lk != 0) {
             end_early(kStYield, 1, step + 1, Lk);
             return;

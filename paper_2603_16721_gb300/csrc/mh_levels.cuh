@@ -1,17 +1,20 @@
-// Greedy rounds by score levels, and their counters by cover rounds (included by
+// Greedy rounds by bands of score levels, and their counters by cover rounds (included by
 // mh_kernels.cu, inside its anonymous namespace).
 //
 // The loop of Algorithm 1 picks one combination per round.  U only shrinks, so a
 // combination's TP, and with it its score, only falls, and the rounds visit scores in
-// descending order: while the best score is L, the rounds take combinations of score
-// L in ascending tuple order, each unless a tumor of its intersection has been covered
-// since (its score then is below L for good).  So the rounds of one level are the
-// lexicographically first set of pairwise disjoint intersections among the level's
-// combinations, and a whole level is resolved at once: a combination that no better one
-// of the level meets is picked, what it meets drops out, and so on.  The search of a
-// level is one pass over the kept leaf parents whose cached bound reaches it.  A solve
-// has 10 to 40 levels where it has 50 to 700 rounds, and each used to cost a chain of
-// about 10 us (scan, re-evaluation, grid barrier, slot reduction, winner rows).
+// descending order.  So with every combination of a score of at least tau at hand (the
+// band's members, with their tumors), the rounds down to tau need no further search: the
+// best member by key is picked, the members' scores follow from their tumors still in U,
+// and so on until the best is below tau, which is where the next band starts.  A band is one
+// pass over the kept leaf parents whose bound reaches tau and one grid barrier; its picks are
+// made by every block alike.  A solve has 7 to 20 bands where it has 50 to 700 rounds, and
+// each of these used to cost a chain of about 10 us (scan, re-evaluation, grid barrier, slot
+// reduction, winner rows).  tau is chosen so that the bounds that reach it are few (about
+// one record per block to evaluate); where a single level already has more (the last ones:
+// thousands of combinations of two or three tumors), the band is that level.  Its rounds are
+// then the lexicographically first set of pairwise disjoint intersections among the members,
+// since a member that meets a pick has fallen below the level for good.
 //
 // The counters of every round (visited and pruned nodes per depth) do not depend on
 // how the winners were found, only on the round cr(s) in which each tumor is covered:
@@ -40,15 +43,20 @@ struct LevelSh {
     int tasks[kWin];                                  // tasks of 32 column words
     u64 nb[kWin];                                     // its best leaf below the level
     int emit[kWin];                                   // whether it has members of the level
+    static constexpr int kEm = kBig ? 256 : 32;
+    u64 em[kEm];                                      // the window's members: gene, TP << 16, FP << 32, record << 48
+    u32 tally[kTally];                                // bounds below the band by distance
     u64 wmax[kMaxWarpsPerBlock];
     u64 cov[kMaxWords];
     u32 hlo[kHist], hhi[kHist];
     u16 cr[kBig ? kMaxSamples : 1];                   // the round that covers each tumor
     u16 ord[kMaxSamples];                             // the tumors by that round, last first
-    int qn, en, alive, k;
+    int qn, en, ec, nd, alive, k, more;
 };
 constexpr u32 kDenseBit = 0x80000000u;  // queue entry: an unlisted (dense) record
-constexpr u64 kEmitted = 1ull << 63;    // ub flag: emitted at the level being resolved
+// A bound word is a score + 1 (below 2^44) and a flag: the record has members in the band
+// being resolved, its leaves are looked at again in the next one.
+constexpr u64 kEmitted = 1ull << 63;
 
 struct LevelOut {
     Member *out;
@@ -72,24 +80,76 @@ __device__ __forceinline__ void prefix_po(const Cohort &c, const Prefix &p, int 
     }
 }
 
-__device__ __forceinline__ Member *new_member(const LevelOut &o, const Key &k, int tp)
+// (t2 also takes TP and FP, below the tuple's bits.)
+__device__ __forceinline__ Member *new_member(const LevelOut &o, const Key &k, int tp, int fp)
 {
     const u32 i = atomicAdd(o.count, 1u);
     if (i >= o.cap) return nullptr;
     Member *m = o.out + i;
     m->t0 = k.t0;
     m->t1 = k.t1;
-    m->t2 = k.t2;
+    m->t2 = k.t2 | (u64)fp << 16 | (u64)tp;
     m->k = (u16)tp;
     return m;
 }
 
+// The member of record r's leaf gene g, by a whole warp: a lane per gene of the tuple
+// (its place among the original indices by counting), a lane per listed tumor or row word.
+__device__ __noinline__ void emit_warp(const Cohort &c, const LevelOut &o, const Rec &r, bool dense, const u64 *Ush, int L,
+                                       int g, int tp, int fp)
+{
+    const int lane = threadIdx.x & 31;
+    u32 at = 0;
+    if (lane == 0) at = atomicAdd(o.count, 1u);
+    const int mine = lane < L ? prefix_gene(r.p, lane) : g;
+    const int v = lane <= L ? (int)__ldg(c.orig + mine) : 0x10000;
+    u64 y = 0;
+    bool has = false;
+    if (dense) {
+        if (lane < c.Wt) {
+            y = Ush[lane] & __ldg(c.T + (size_t)g * c.WTp + lane);
+#pragma unroll
+            for (int q = 0; q < kMaxH - 1; ++q)
+                if (q < L) y &= __ldg(c.T + (size_t)prefix_gene(r.p, q) * c.WTp + lane);
+        }
+    } else if (lane < (int)r.ky) {
+        has = (__ldg(c.CT + (size_t)r.ids[lane] * c.GW + (g >> 6)) >> (g & 63)) & 1ull;
+    }
+    int place = 0;
+    for (int q = 0; q <= L; ++q) place += __shfl_sync(kFull, v, q) < v ? 1 : 0;
+    const u64 x = lane <= L ? (u64)v << (16 * (3 - (place & 3))) : 0ull;
+    u64 t[3];
+#pragma unroll
+    for (int w = 0; w < 3; ++w) {
+        const u64 xw = place >> 2 == w ? x : 0ull;
+        t[w] = (u64)__reduce_or_sync(kFull, (unsigned)(xw >> 32)) << 32 | __reduce_or_sync(kFull, (unsigned)xw);
+    }
+    at = __shfl_sync(kFull, at, 0);
+    if (at >= o.cap) return;
+    Member *m = o.out + at;
+    if (lane == 0) {
+        m->t0 = t[0];
+        m->t1 = t[1];
+        m->t2 = t[2] | (u64)fp << 16 | (u64)tp;
+        m->k = (u16)tp;
+    }
+    if (tp > kMemIds) return;
+    if (dense) {
+        int n = warp_incl_scan(__popcll(y), lane) - __popcll(y);
+        for (; y; y &= y - 1) m->ids[n++] = (u16)(lane * 64 + __ffsll((long long)y) - 1);
+    } else {
+        const unsigned b = __ballot_sync(kFull, has);
+        if (has) m->ids[__popc(b & ((1u << lane) - 1u))] = r.ids[lane];
+    }
+}
+
 // A leaf of listed record r (its samples those in U) at column word wi, bit bt.
-__device__ __noinline__ void emit_listed(const Cohort &c, const LevelOut &o, const Rec &r, int L, int wi, int bt, int tp)
+__device__ __noinline__ void emit_listed(const Cohort &c, const LevelOut &o, const Rec &r, int L, int wi, int bt, int tp,
+                                         int fp)
 {
     int po[kMaxH - 1];
     prefix_po(c, r.p, L, po);
-    Member *m = new_member(o, leaf_key(0, po, L, c.orig[wi * 64 + bt]), tp);
+    Member *m = new_member(o, leaf_key(0, po, L, c.orig[wi * 64 + bt]), tp, fp);
     if (!m || tp > kMemIds) return;
     int n = 0;
     for (int q = 0; q < (int)r.ky; ++q)
@@ -98,11 +158,11 @@ __device__ __noinline__ void emit_listed(const Cohort &c, const LevelOut &o, con
 
 // A leaf of a dense record, y in ys.
 __device__ __noinline__ void emit_dense(const Cohort &c, const LevelOut &o, const Prefix &p, const u64 *ys, int L, int g,
-                                        int tp)
+                                        int tp, int fp)
 {
     int po[kMaxH - 1];
     prefix_po(c, p, L, po);
-    Member *m = new_member(o, leaf_key(0, po, L, c.orig[g]), tp);
+    Member *m = new_member(o, leaf_key(0, po, L, c.orig[g]), tp, fp);
     if (!m || tp > kMemIds) return;
     int n = 0;
     for (int w = 0; w < c.Wt; ++w)
@@ -110,10 +170,31 @@ __device__ __noinline__ void emit_dense(const Cohort &c, const LevelOut &o, cons
             m->ids[n++] = (u16)(w * 64 + __ffsll((long long)y) - 1);
 }
 
-// One (record, column word) item of a listed record at level Lk: its leaves of that
-// score are emitted, the best one below it goes to nb.
-__device__ __forceinline__ void leaf_item_level(const Cohort &c, const Solve &s, const LevelOut &o, const Rec &r, int L,
-                                                int wi, u64 rw, u64 Lk, u64 &nb, bool &emitted)
+// A record's first 64 bytes (prefix, sizes, tumors) and its other samples.
+static_assert(offsetof(Rec, ids) + sizeof(u16) * kListT <= 64, "tumors in the first four 16-byte words");
+__device__ __forceinline__ void load_rec_tumors(Rec *dst, const Rec *src)
+{
+#pragma unroll
+    for (int i = 0; i < 4; ++i) reinterpret_cast<uint4 *>(dst)[i] = __ldcg(reinterpret_cast<const uint4 *>(src) + i);
+}
+__device__ __forceinline__ void load_rec_normals(Rec *dst, const Rec *src)
+{
+    const u16 *s = src->ids + kListT;
+    for (int i = 0; i < (int)dst->kn && i < kListN; ++i) dst->ids[kListT + i] = __ldcg(s + i);
+}
+
+// Where the evaluation of a window leaves the members it finds: in the block's list, for
+// emit_warp, or beyond its room straight to the level.
+struct EmitList {
+    u64 *em;
+    int *n;
+    int cap, j;  // j: the record's place in the window
+};
+
+// One (record, column word) item of a listed record in a band: its leaves of scores from
+// tau on are emitted, the best one below goes to nb.
+__device__ __forceinline__ void leaf_item_level(const Cohort &c, const Solve &s, const LevelOut &o, const EmitList &el,
+                                                const Rec &r, int L, int wi, u64 rw, u64 tau, u64 &nb, bool &emitted)
 {
     const int ky = r.ky, kn = r.kn;
     const int pt = bit_length(ky), pn = kn ? bit_length(kn) : 0;
@@ -147,10 +228,13 @@ __device__ __forceinline__ void leaf_item_level(const Cohort &c, const Solve &s,
         m2 &= m2 - 1;
         const int tp = planes_get(tpl, bt, pt);
         const u64 b1 = s.a_num * (u64)tp + top;
-        if (b1 <= nb) continue;  // no better than what is known below the level
-        const u64 s1 = b1 - s.a_den * (u64)planes_get(fpl, bt, pn);
-        if (s1 == Lk) {
-            emit_listed(c, o, r, L, wi, bt, tp);
+        if (b1 <= nb) continue;  // no better than what is known below the band
+        const int fp = planes_get(fpl, bt, pn);
+        const u64 s1 = b1 - s.a_den * (u64)fp;
+        if (s1 >= tau) {
+            const int p = atomicAdd(el.n, 1);
+            if (p < el.cap) el.em[p] = (u64)(wi * 64 + bt) | (u64)tp << 16 | (u64)fp << 32 | (u64)el.j << 48;
+            else emit_listed(c, o, r, L, wi, bt, tp, fp);
             emitted = true;
         } else if (s1 > nb) {
             nb = s1;
@@ -186,33 +270,47 @@ __device__ __forceinline__ void wide_add8(u64 (&p)[kWide], const u64 (&x)[8], in
         }
 }
 
-// Adds column word wi of every sample set in the words ys (nonzero words: bits) to p.
-__device__ __forceinline__ void wide_columns(const u64 *C, int GW, const u64 *ys, unsigned bits, int wi, bool in,
-                                             u64 (&p)[kWide], int used)
+// Adds the column words wi of the samples set in the words ys (non-zero words: bits) to
+// the lanes' counters p: the warp's lanes form cg groups of 32 / cg words, group `grp` takes
+// every cg-th sample (listed in ids, 1536 at a time; 16 loads in flight), and the groups'
+// counters are added up in the end, so that every lane of a word holds its counts.
+constexpr int kIdWords = 24;
+__device__ void wide_columns(const u64 *C, int GW, const u64 *ys, unsigned bits, int wi, bool in, int cg, int grp,
+                             u16 *ids, u64 (&p)[kWide], int used)
 {
-    u64 cur = 0;
-    int w = 0;
-    for (;;) {
-        u64 x[8];
-        bool more = false;
+    const int lane = threadIdx.x & 31;
+    for (int w0 = 0; w0 < kMaxWords; w0 += kIdWords) {
+        const unsigned part = w0 == 0 ? bits & ((1u << kIdWords) - 1u) : bits & ~((1u << kIdWords) - 1u);
+        if (!part) continue;
+        u64 y = (part >> lane) & 1u ? ys[lane] : 0ull;
+        const int pc = __popcll(y), inc = warp_incl_scan(pc, lane), cnt = __shfl_sync(kFull, inc, 31);
+        __syncwarp();
+        for (int n = inc - pc; y; y &= y - 1) ids[n++] = (u16)(lane * 64 + __ffsll((long long)y) - 1);
+        __syncwarp();
+        for (int q0 = 0; q0 < cnt; q0 += 16 * cg) {
+            u64 x[16];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {  // the same sample for every lane of the warp
-            while (!cur && bits) {
-                w = __ffs(bits) - 1;
-                bits &= bits - 1;
-                cur = ys[w];
+            for (int u = 0; u < 16; ++u) {
+                const int q = q0 + cg * u + grp;
+                x[u] = in && q < cnt ? __ldg(C + (size_t)ids[q] * GW + wi) : 0ull;
             }
-            x[k] = 0;
-            if (cur) {
-                const int smp = w * 64 + __ffsll((long long)cur) - 1;
-                cur &= cur - 1;
-                if (in) x[k] = __ldg(C + (size_t)smp * GW + wi);
-                more = true;
+#pragma unroll
+            for (int v = 0; v < 16; v += 8) {
+                const u64 z[8] = {x[v], x[v + 1], x[v + 2], x[v + 3], x[v + 4], x[v + 5], x[v + 6], x[v + 7]};
+                wide_add8(p, z, used);
             }
         }
-        if (!more) break;
-        wide_add8(p, x, used);
-        if (!cur && !bits) break;
+    }
+    for (int off = 16; off >= 32 / cg; off >>= 1) {  // group sums: bit-sliced additions over the lanes of a word
+        u64 carry = 0;
+#pragma unroll
+        for (int i = 0; i < kWide; ++i)
+            if (i < used) {
+                const u64 o = __shfl_xor_sync(kFull, p[i], off);
+                const u64 u = p[i] ^ o, nc = (p[i] & o) | (u & carry);
+                p[i] = u ^ carry;
+                carry = nc;
+            }
     }
 }
 
@@ -241,43 +339,61 @@ __device__ __forceinline__ int dense_words(const Cohort &c, const u64 *Ush, cons
     return (int)__reduce_add_sync(kFull, (unsigned)__popcll(y));
 }
 
-// 32 column words of a dense record (its y / n words in the warp scratch, k = |y|):
-// leaves of score Lk are emitted, the best below goes to nb.  By columns, 64 leaves a
-// lane at a time: |y| + |n| coalesced loads per word where the rows of the leaf genes
-// would take 64 (Wt + Wn) scattered ones.
-__device__ __noinline__ void dense_item_level(const Cohort &c, const Solve &s, const LevelOut &o, Batch &b, const Prefix &p,
-                                              unsigned by, unsigned bn, int k, int kn, int L, int lo, int wi, u64 Lk,
-                                              u64 &nb, bool &emitted)
+// 32 / cg column words of a dense record (its y / n words in the warp scratch, k = |y|):
+// leaves of scores from tau on are emitted, the best below goes to nb.  By columns, 64 leaves a lane
+// at a time: |y| + |n| coalesced loads per word where the rows of the leaf genes would take
+// 64 (Wt + Wn) scattered ones.  With cg > 1 the samples of a word, and then its leaves, are
+// shared by cg lanes: one record is spread over all warps of the block.
+__device__ __noinline__ void dense_item_level(const Cohort &c, const Solve &s, const LevelOut &o, const EmitList &el, Batch &b,
+                                              const Prefix &p, unsigned by, unsigned bn, int k, int kn, int L, int lo,
+                                              int wi, int cg, u64 tau, u64 &nb, bool &emitted)
 {
-    const int last = (c.G - 1) >> 6;
+    const int lane = threadIdx.x & 31, grp = lane / (32 / cg), last = (c.G - 1) >> 6;
     const bool in = wi <= last;
+    u16 *ids = reinterpret_cast<u16 *>(b.r);
+    static_assert(sizeof(b.r) >= kIdWords * 64 * sizeof(u16), "the samples of kIdWords words in the records' place");
     u64 tp[kWide], fp[kWide];
 #pragma unroll
     for (int i = 0; i < kWide; ++i) tp[i] = fp[i] = 0;
-    const int pt = bit_length(k), pn = kn ? bit_length(kn) : 0;
-    wide_columns(c.CT, c.GW, b.ys, by, wi, in, tp, pt);
+    const int pt = max(bit_length(k), 3), pn = kn ? max(bit_length(kn), 3) : 0;
+    wide_columns(c.CT, c.GW, b.ys, by, wi, in, cg, grp, ids, tp, pt);
     u64 m2 = 0;
 #pragma unroll
     for (int i = 1; i < kWide; ++i) m2 |= tp[i];
     if (in) m2 &= range_word(wi, lo, c.G - 1);
     else m2 = 0;
     if (!__any_sync(kFull, m2 != 0)) return;
-    wide_columns(c.CN, c.GW, b.ns, bn, wi, in, fp, pn);
+    wide_columns(c.CN, c.GW, b.ns, bn, wi, in, cg, grp, ids, fp, pn);
     const u64 top = s.a_den * (u64)c.Nn + 1;
+    if (cg > 1) {  // the lane's share of the word's leaves
+        const int span = 64 / cg;
+        m2 &= ((1ull << span) - 1ull) << (span * grp);
+    }
     while (m2) {
         const int bt = __ffsll((long long)m2) - 1;
         m2 &= m2 - 1;
         const int t = planes_get(tp, bt, pt);
         const u64 b1 = s.a_num * (u64)t + top;
         if (b1 <= nb) continue;
-        const u64 s1 = b1 - s.a_den * (u64)planes_get(fp, bt, pn);
-        if (s1 == Lk) {
-            emit_dense(c, o, p, b.ys, L, wi * 64 + bt, t);
+        const int f = planes_get(fp, bt, pn);
+        const u64 s1 = b1 - s.a_den * (u64)f;
+        if (s1 >= tau) {
+            const int q = atomicAdd(el.n, 1);
+            if (q < el.cap) el.em[q] = (u64)(wi * 64 + bt) | (u64)t << 16 | (u64)f << 32 | (u64)el.j << 48;
+            else emit_dense(c, o, p, b.ys, L, wi * 64 + bt, t, f);
             emitted = true;
         } else if (s1 > nb) {
             nb = s1;
         }
     }
+}
+
+__device__ __forceinline__ Prefix load_prefix(const Rec *r)
+{
+    Prefix p;
+    p.w0 = __ldcg(&r->p.w0);
+    p.w1 = __ldcg(&r->p.w1);
+    return p;
 }
 
 // The kept frontiers' shard offsets and sizes, read once per launch.
@@ -341,51 +457,73 @@ __device__ __forceinline__ void block_level_max(u64 v, u64 *wmax, u64 *out)
     }
 }
 
-// Sets up window entry j of the block from queue entry e.
+// Window entry j of the block: the column words of its leaves.
 template <bool kBig>
-__device__ __forceinline__ void window_tasks(const Cohort &c, LevelSh<kBig> &sh, int j, const Prefix &p, int L)
+__device__ __forceinline__ void window_tasks(const Cohort &c, LevelSh<kBig> &sh, int j, const Prefix &p, int L, bool dense)
 {
     const int lo = prefix_gene(p, L - 1) + 1;
-    sh.tasks[j] = lo > c.G - 1 ? 0 : ((((c.G - 1) >> 6) - (lo >> 6) + 1 + 31) >> 5);
+    sh.tasks[j] = lo > c.G - 1 ? 0 : ((c.G - 1) >> 6) - (lo >> 6) + 1;
     sh.nb[j] = 0;
     sh.emit[j] = 0;
+    if (dense) atomicAdd(&sh.nd, 1);
 }
 
-// The block's window of nw records, in tasks of 32 column words spread over its warps.
+// The block's window of nw records spread over its warps: listed records in tasks of 32
+// column words, dense ones in tasks of 32 / cg words, cg the smallest that gives every
+// warp two tasks (a single dense record of 19,000 genes: 38 tasks of 8 words).  Then the
+// members found, a warp each.
 template <bool kBig>
 __device__ void window_eval(const Cohort &c, const Solve &s, const LevelOut &o, LevelSh<kBig> &sh, Batch &b, const u64 *Ush,
-                            int nw, int L, u64 Lk)
+                            int nw, int L, u64 tau)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int i0 = lane < nw ? sh.tasks[lane] : 0;
-    const int i1 = LevelSh<kBig>::kWin > 32 && lane + 32 < nw ? sh.tasks[(lane + 32) % LevelSh<kBig>::kWin] : 0;
+    int cg = 1;
+    while (cg < 16 && sh.nd * ((((c.G - 1) >> 6) + 32 / cg) / (32 / cg)) < 2 * nwarps) cg *= 2;
+    const int dw = 32 / cg;
+    auto ntasks = [&](int j) {
+        const int per = sh.ri[j] & kDenseBit ? dw : 32;
+        return (sh.tasks[j] + per - 1) / per;
+    };
+    const int i0 = lane < nw ? ntasks(lane) : 0;
+    const int i1 = LevelSh<kBig>::kWin > 32 && lane + 32 < nw ? ntasks((lane + 32) % LevelSh<kBig>::kWin) : 0;
     const int inc0 = warp_incl_scan(i0, lane);
     const int inc1 = __shfl_sync(kFull, inc0, 31) + warp_incl_scan(i1, lane);
     const int T = __shfl_sync(kFull, inc1, 31);
-    for (int tau = warp; tau < T; tau += nwarps) {
-        // its record: the number of records whose tasks end at or before tau
-        const int j = __popc(__ballot_sync(kFull, lane < nw && inc0 <= tau)) +
-                      __popc(__ballot_sync(kFull, lane + 32 < nw && inc1 <= tau));
+    EmitList el{sh.em, &sh.ec, LevelSh<kBig>::kEm, 0};
+    for (int x = warp; x < T; x += nwarps) {
+        // its record: the number of records whose tasks end at or before x
+        const int j = __popc(__ballot_sync(kFull, lane < nw && inc0 <= x)) +
+                      __popc(__ballot_sync(kFull, lane + 32 < nw && inc1 <= x));
         const int e0 = __shfl_sync(kFull, inc0, (j - 1) & 31), e1 = __shfl_sync(kFull, inc1, (j - 33) & 31);
         const int first = j == 0 ? 0 : (j <= 32 ? e0 : e1);
         const Rec &r = sh.rec[j];
         const int lo = prefix_gene(r.p, L - 1) + 1;
-        const int wi = (lo >> 6) + (tau - first) * 32 + lane;
         u64 nb = 0;
         bool emitted = false;
+        el.j = j;
         if (sh.ri[j] & kDenseBit) {
             unsigned by, bn;
             int kn;
             const int k = dense_words(c, Ush, r.p, L, b, by, bn, kn, lane);
-            dense_item_level(c, s, o, b, r.p, by, bn, k, kn, L, lo, wi, Lk, nb, emitted);
+            const int wi = (lo >> 6) + (x - first) * dw + (lane & (dw - 1));
+            dense_item_level(c, s, o, el, b, r.p, by, bn, k, kn, L, lo, wi, cg, tau, nb, emitted);
             __syncwarp();
-        } else if (wi <= (c.G - 1) >> 6) {
-            leaf_item_level(c, s, o, r, L, wi, range_word(wi, lo, c.G - 1), Lk, nb, emitted);
+        } else {
+            const int wi = (lo >> 6) + (x - first) * 32 + lane;
+            if (wi <= (c.G - 1) >> 6) leaf_item_level(c, s, o, el, r, L, wi, range_word(wi, lo, c.G - 1), tau, nb, emitted);
         }
         nb = warp_max_u64(nb);
         const bool em = __any_sync(kFull, emitted);
         if (lane == 0 && nb) atomicMax(&sh.nb[j], nb);
         if (lane == 0 && em) sh.emit[j] = 1;
+    }
+    __syncthreads();
+    const int ne = sh.ec < LevelSh<kBig>::kEm ? sh.ec : LevelSh<kBig>::kEm;
+    for (int e = warp; e < ne; e += nwarps) {
+        const u64 m = sh.em[e];
+        const int j = (int)(m >> 48);
+        emit_warp(c, o, sh.rec[j], (sh.ri[j] & kDenseBit) != 0, Ush, L, (int)(m & 0xffffull), (int)((m >> 16) & 0xffffull),
+                  (int)((m >> 32) & 0xffffull));
     }
 }
 
@@ -443,14 +581,15 @@ __device__ void level_first(const Cohort &c, const Solve &s, const Frontiers &f,
             hm &= hm - 1;
             unsigned by, bn;
             int kn;
-            const Prefix p = b.r[j].p;
+            const u32 ij = __shfl_sync(kFull, i, j);
+            const Prefix p = load_prefix(f.F[l] + front_slot(f.cap[l], ft.soff[l], ij));
             const int ky = dense_words(c, Ush, p, l, b, by, bn, kn, lane);
             const int lo = prefix_gene(p, l - 1) + 1;
             u64 nb = 0;
             bool em = false;
             for (int w0 = lo >> 6; w0 <= (c.G - 1) >> 6; w0 += 32)
-                dense_item_level(c, s, LevelOut{nullptr, nullptr, 0u}, b, p, by, bn, ky, kn, l, lo, w0 + lane, ~0ull, nb,
-                                 em);
+                dense_item_level(c, s, LevelOut{nullptr, nullptr, 0u}, EmitList{nullptr, nullptr, 0, 0}, b, p, by, bn, ky, kn,
+                                 l, lo, w0 + lane, 1, ~0ull, nb, em);
             nb = warp_max_u64(nb);
             if (lane == j) {
                 ub[i] = nb;
@@ -464,11 +603,13 @@ __device__ void level_first(const Cohort &c, const Solve &s, const Frontiers &f,
     for (int w0 = 0; w0 < nq; w0 += LevelSh<kBig>::kWin) {
         const int nw = nq - w0 < LevelSh<kBig>::kWin ? nq - w0 : LevelSh<kBig>::kWin;
         const int j = (int)threadIdx.x;
+        if (threadIdx.x == 0) sh.nd = sh.ec = 0;
+        __syncthreads();
         if (j < nw) {
             const u32 i = sh.q[w0 + j];
             load_rec(&sh.rec[j], f.F[l] + front_slot(f.cap[l], ft.soff[l], i));
             sh.ri[j] = i | kDenseBit;
-            window_tasks<kBig>(c, sh, j, sh.rec[j].p, l);
+            window_tasks<kBig>(c, sh, j, sh.rec[j].p, l, true);
         }
         __syncthreads();
         window_eval<kBig>(c, s, LevelOut{nullptr, nullptr, 0u}, sh, b, Ush, nw, l, ~0ull);
@@ -483,26 +624,81 @@ __device__ void level_first(const Cohort &c, const Solve &s, const Frontiers &f,
     block_level_max(best, sh.wmax, &s.lev->lmax[0]);
 }
 
-// One level Lk (score + 1) of step `step`: the block's share of the leaf parents and
-// champions of that score go to the level's members, and the largest bound below it to
-// the next step's level.  Every thread of the block calls it; a grid barrier follows.
+// Bounds below Lk by distance, in units of a_num: tally j counts those at most tally_width(j)
+// (and more than the next smaller one) below Lk.  16 bits each per thread, added up per block.
+__device__ __forceinline__ u32 tally_width(int j) { return j & 1 ? 2u << (j >> 1) : (j == 0 ? 1u : 3u << ((j >> 1) - 1)); }
+struct Tally {
+    u64 n[kTally / 4] = {};
+    __device__ __forceinline__ void add(u64 Lk, u64 a_num, u64 v)
+    {
+        const u64 d = Lk - v;
+        if (d > a_num * tally_width(kTally - 1)) return;
+        int j = 0;
+#pragma unroll
+        for (int q = 0; q < kTally - 1; ++q) j += a_num * tally_width(q) < d ? 1 : 0;
+#pragma unroll
+        for (int w = 0; w < kTally / 4; ++w) n[w] += j >> 2 == w ? 1ull << (16 * (j & 3)) : 0ull;
+    }
+    __device__ __forceinline__ void flush(u32 *out)
+    {
+        const int lane = threadIdx.x & 31;
+        u64 any = 0;
+#pragma unroll
+        for (int w = 0; w < kTally / 4; ++w) any |= n[w];
+        if (!__any_sync(kFull, any != 0)) return;
+#pragma unroll
+        for (int w = 0; w < kTally / 4; ++w) {
+            const u64 v = warp_sum_u64(n[w]);
+            if (lane < 4) {
+                const u32 x = (u32)((v >> (16 * lane)) & 0xffffull);
+                if (x) atomicAdd(out + 4 * w + lane, x);
+            }
+            n[w] = 0;
+        }
+    }
+};
+
+// The bounds' tally of the first band (the later ones are counted during the search).
+template <bool kBig>
+__device__ void level_tally(const Solve &s, const Frontiers &f, LevelSh<kBig> &sh, const Team &t, const FrontTab &ft, u64 Lk,
+                            int step)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const u64 *ub = f.ub[s.h - 1];
+    const Share sr((u32)ft.n[s.h - 1], (u32)t.size, (u32)nwarps, (u32)t.rank);
+    if (threadIdx.x < kTally) sh.tally[threadIdx.x] = 0;
+    __syncthreads();
+    Tally ty;
+    for (u32 k = 0; k < sr.steps(); ++k) {
+        const u32 i = sr.at(k, (u32)warp, (u32)lane);
+        if (i < sr.n) ty.add(Lk, s.a_num, __ldcg(ub + i));
+        if ((k & 63u) == 63u) ty.flush(sh.tally);
+    }
+    ty.flush(sh.tally);
+    __syncthreads();
+    if (threadIdx.x < kTally && sh.tally[threadIdx.x]) atomicAdd(&s.lev->tally[step & 3][threadIdx.x], sh.tally[threadIdx.x]);
+}
+
+// The band of step `step`, scores + 1 from tau to Lk: the block's share of the leaf parents
+// and champions whose scores reach tau leaves its members, and the largest bound below it
+// counts for the next band.  Every thread of the block calls it; a grid barrier follows.
 template <bool kBig>
 __device__ void level_search(const Cohort &c, const Solve &s, const Frontiers &f, LevelSh<kBig> &sh, Batch &b, const Team &t,
-                             const FrontTab &ft, const u64 *Ush, u64 Lk, int step, bool rerun)
+                             const FrontTab &ft, const u64 *Ush, u64 Lk, u64 tau, int step)
 {
-    constexpr int kIlpS = LevelSh<kBig>::kIlp;
+    constexpr int kIlpS = LevelSh<kBig>::kIlp, kWin = LevelSh<kBig>::kWin, kQ = LevelSh<kBig>::kQ;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int l = s.h - 1;
     u64 *ub = f.ub[l];
-    if (t.rank == 0 && threadIdx.x == 0) {  // the step after the next starts from zero
-        s.lev->lmax[(step + 2) & 3] = 0;
-        s.lev->mcnt[(step + 2) & 3] = 0;
+    if (t.rank == 0) {  // the step after the next starts from zero
+        if (threadIdx.x == 0) {
+            s.lev->lmax[(step + 2) & 3] = 0;
+            s.lev->mcnt[(step + 2) & 3] = 0;
+        }
+        if (threadIdx.x < kTally) s.lev->tally[(step + 2) & 3][threadIdx.x] = 0;
     }
     const LevelOut o{s.mem + (size_t)(step & 1) * s.mcap, &s.lev->mcnt[step & 3], s.mcap};
-    const u64 top = s.a_den * (u64)c.Nn + 1;
-    // what a record can still hold after a level it had members in: they fall by a_num at
-    // least (level_select finds to what), its other leaves are below the level already
-    const u64 fall = Lk - s.a_num;
+    const u64 top = s.a_den * (u64)c.Nn + 1, unit = s.a_num < s.a_den ? s.a_num : s.a_den;
     u64 next = 0;
     // with a_num = 0 a score does not depend on TP: a champion is the best of all the
     // combinations of its tumor, and one combination is picked per step
@@ -512,13 +708,13 @@ __device__ void level_search(const Cohort &c, const Solve &s, const Frontiers &f
         Key k = key_empty();
         if (smp < c.Nt && in_mask(Ush, smp)) {
             const u64 v = __ldcg(&s.champ[smp].s);
-            if (v == Lk) {
+            if (v >= tau) {
                 k.s = v;
                 k.t0 = __ldcg(&s.champ[smp].t0);
                 k.t1 = __ldcg(&s.champ[smp].t1);
                 k.t2 = __ldcg(&s.champ[smp].t2);
             }
-            if ((v < Lk || flat) && v > next) next = v;
+            if ((v < tau || flat) && v > next) next = v;
         }
         if (flat) {
             const Key m = warp_max_key(k);
@@ -528,76 +724,77 @@ __device__ void level_search(const Cohort &c, const Solve &s, const Frontiers &f
             k.t2 = m.t2;
         }
         if (k.s) {
-            Member *m = new_member(o, k, 1);
+            Member *m = new_member(o, k, 1, c.Nn - (int)((k.s - 1 - s.a_num) / s.a_den));
             if (m) m->ids[0] = (u16)smp;
         }
     }
     const Share sr((u32)ft.n[l], (u32)t.size, (u32)nwarps, (u32)t.rank);
     const u32 steps = flat ? 0u : sr.steps();
-    for (u32 k0 = 0; k0 < steps; k0 += kIlpS) {
-        // a segment of the scan: as many records as the queue takes
-        if (threadIdx.x == 0) sh.qn = sh.en = 0;
+    if (threadIdx.x < kTally) sh.tally[threadIdx.x] = 0;
+    Tally ty;
+    for (int pass = 0; steps > 0; ++pass) {
+        // the block's bounds; those that reach tau are queued (what does not fit is found by
+        // another scan after the queue is done: its bounds still reach tau)
+        if (threadIdx.x == 0) sh.qn = sh.en = sh.ec = sh.nd = sh.more = 0;
         __syncthreads();
-        u64 v[kIlpS];
+        for (u32 k0 = 0; k0 < steps; k0 += kIlpS) {
+            u64 v[kIlpS];
 #pragma unroll
-        for (int u = 0; u < kIlpS; ++u) {
-            const u32 i = sr.at(k0 + u, (u32)warp, (u32)lane);
-            v[u] = k0 + u < steps && i < sr.n ? __ldcg(ub + i) : 0ull;
-        }
-#pragma unroll
-        for (int u = 0; u < kIlpS; ++u) {
-            const u32 i = sr.at(k0 + u, (u32)warp, (u32)lane);
-            if (v[u] & kEmitted) {  // emitted at the level before, or at this one if it is run again
-                v[u] = rerun ? Lk : v[u] & ~kEmitted;
-                if (!rerun) ub[i] = v[u];
+            for (int u = 0; u < kIlpS; ++u) {
+                const u32 i = sr.at(k0 + u, (u32)warp, (u32)lane);
+                v[u] = k0 + u < steps && i < sr.n ? __ldcg(ub + i) : 0ull;
             }
-            if (v[u] >= Lk) sh.q[atomicAdd(&sh.qn, 1)] = i;
-            else if (v[u] > next) next = v[u];
+#pragma unroll
+            for (int u = 0; u < kIlpS; ++u) {
+                const u32 i = sr.at(k0 + u, (u32)warp, (u32)lane);
+                u64 w = v[u];
+                if (w & kEmitted) {
+                    if (pass > 0) continue;  // done in this band
+                    w &= ~kEmitted;          // members of the last band
+                    ub[i] = w;
+                }
+                if (w >= tau) {
+                    const int p = atomicAdd(&sh.qn, 1);
+                    if (p < kQ) sh.q[p] = i;
+                    else sh.more = 1;
+                } else if (w && pass == 0) {
+                    next = w > next ? w : next;
+                    ty.add(Lk, s.a_num, w);
+                }
+            }
+            if ((k0 & 63u) + kIlpS >= 64u) ty.flush(sh.tally);
         }
         __syncthreads();
-        const int nq = sh.qn;
-        if (nq == 0) {
-            __syncthreads();
-            continue;
-        }
-        // the queued records: their samples still in U; what the cheaper bound lowers is
-        // done, an untouched listed record whose best leaf takes all its samples at FP = 0
-        // gives its cached leaf, the others are evaluated (queue entries reused)
+        const int nq = sh.qn < kQ ? sh.qn : kQ;
+        const bool more = sh.more != 0;
+        auto lowered = [&](u32 i, u64 v) {
+            ub[i] = v;
+            next = v > next ? v : next;
+            if (v) ty.add(Lk, s.a_num, v);
+        };
+        // the queued records: their samples still in U; what the cheaper bound lowers is done,
+        // an untouched listed record whose best leaf takes all its samples at FP = 0 gives its
+        // cached leaf (if no other can reach tau), the others are evaluated (queue entries reused)
         for (int q0 = 0; q0 < nq; q0 += (int)blockDim.x) {
-            const int qi = q0 + (int)threadIdx.x;
+            const int qi = q0 + lane * nwarps + warp;  // few entries: one per warp
             const bool act = qi < nq;
             const u32 i = act ? sh.q[qi] : 0u;
             __syncthreads();  // entries of this pass are read before evaluations overwrite them
             Rec &r = b.r[lane];
             bool dense = false, eval = false;
-            int k = 0;
+            int k = 0, k0y = 0;
+            const Rec *src = nullptr;
             if (act) {
-                load_rec(&r, f.F[l] + front_slot(f.cap[l], ft.soff[l], i));
+                src = f.F[l] + front_slot(f.cap[l], ft.soff[l], i);
+                load_rec_tumors(&r, src);
                 dense = is_dense(r.ky, r.kn);
+                k0y = r.ky;
                 if (!dense) {
-                    const int k0y = r.ky;
                     for (int q = 0; q < k0y; ++q) {
                         const int smp = r.ids[q];
                         if (in_mask(Ush, smp)) r.ids[k++] = (u16)smp;
                     }
                     r.ky = (u16)k;
-                    const u64 bound = k >= 2 ? s.a_num * (u64)k + top : 0ull;
-                    if (bound < Lk) {
-                        ub[i] = bound;
-                        next = bound > next ? bound : next;
-                    } else if (k == k0y && bound == Lk) {
-                        Key kc;
-                        kc.t0 = __ldcg(&f.lb[l][i].t0);
-                        kc.t1 = __ldcg(&f.lb[l][i].t1);
-                        kc.t2 = __ldcg(&f.lb[l][i].t2);
-                        Member *m = new_member(o, kc, k);
-                        if (m && k <= kMemIds)
-                            for (int q = 0; q < k; ++q) m->ids[q] = r.ids[q];
-                        // (looked at again at the next level: what is left of it is known then)
-                        ub[i] = (Lk - (s.a_num < s.a_den ? s.a_num : s.a_den)) | kEmitted;
-                    } else {
-                        eval = true;
-                    }
                 }
             }
             __syncwarp();
@@ -613,33 +810,45 @@ __device__ void level_search(const Cohort &c, const Solve &s, const Frontiers &f
                         if (q < l) y &= __ldg(c.T + (size_t)prefix_gene(b.r[j].p, q) * c.WTp + lane);
                 }
                 const int ky = (int)__reduce_add_sync(kFull, (unsigned)__popcll(y));
-                if (lane == j) {
-                    const u64 bound = ky >= 2 ? s.a_num * (u64)ky + top : 0ull;
-                    if (bound < Lk) {
-                        ub[i] = bound;
-                        next = bound > next ? bound : next;
-                    } else {
-                        eval = true;
-                    }
+                if (lane == j) k = ky;
+            }
+            if (act) {
+                const u64 bound = k >= 2 ? s.a_num * (u64)k + top : 0ull;
+                if (bound < tau) {
+                    lowered(i, bound);
+                } else if (!dense && k == k0y && bound - unit < tau && __ldcg(&f.lb[l][i].s) == bound) {
+                    Key kc;
+                    kc.t0 = __ldcg(&f.lb[l][i].t0);
+                    kc.t1 = __ldcg(&f.lb[l][i].t1);
+                    kc.t2 = __ldcg(&f.lb[l][i].t2);
+                    Member *m = new_member(o, kc, k, 0);
+                    if (m && k <= kMemIds)
+                        for (int q = 0; q < k; ++q) m->ids[q] = r.ids[q];
+                    ub[i] = bound | kEmitted;
+                } else {
+                    eval = true;
                 }
             }
             if (eval) {
                 const int p = atomicAdd(&sh.en, 1);
-                if (p < LevelSh<kBig>::kWin) {  // the first window is filled here
+                if (p < kWin) {  // the first window is filled here
+                    load_rec_normals(&r, src);
                     copy_rec(&sh.rec[p], &r);
                     sh.ri[p] = i | (dense ? kDenseBit : 0u);
-                    window_tasks<kBig>(c, sh, p, r.p, l);
+                    window_tasks<kBig>(c, sh, p, r.p, l, dense);
                 } else {
-                    sh.q[p] = i;  // p <= the entries read so far
+                    sh.q[p] = i;  // p < the entries read so far
                 }
             }
             __syncthreads();
         }
         const int ne = sh.en;
-        for (int w0 = 0; w0 < ne; w0 += LevelSh<kBig>::kWin) {
-            const int nw = ne - w0 < LevelSh<kBig>::kWin ? ne - w0 : LevelSh<kBig>::kWin;
+        for (int w0 = 0; w0 < ne; w0 += kWin) {
+            const int nw = ne - w0 < kWin ? ne - w0 : kWin;
             const int j = (int)threadIdx.x;
             if (w0 > 0) {
+                if (threadIdx.x == 0) sh.nd = sh.ec = 0;
+                __syncthreads();
                 if (j < nw) {
                     const u32 i = sh.q[w0 + j];
                     Rec &r = sh.rec[j];
@@ -654,91 +863,369 @@ __device__ void level_search(const Cohort &c, const Solve &s, const Frontiers &f
                         r.ky = (u16)k;
                     }
                     sh.ri[j] = i | (dense ? kDenseBit : 0u);
-                    window_tasks<kBig>(c, sh, j, r.p, l);
+                    window_tasks<kBig>(c, sh, j, r.p, l, dense);
                 }
                 __syncthreads();
             }
-            window_eval<kBig>(c, s, o, sh, b, Ush, nw, l, Lk);
+            window_eval<kBig>(c, s, o, sh, b, Ush, nw, l, tau);
             __syncthreads();
             if (j < nw) {
-                // the best leaf below the level, or what its members fall to
-                const u64 v = sh.nb[j];
-                ub[sh.ri[j] & ~kDenseBit] = sh.emit[j] ? (fall > v ? fall : v) | kEmitted : v;
-                next = v > next ? v : next;
+                // the best leaf below the band; with members, the record is looked at again
+                const u32 i = sh.ri[j] & ~kDenseBit;
+                if (sh.emit[j]) {
+                    ub[i] = Lk | kEmitted;
+                    next = sh.nb[j] > next ? sh.nb[j] : next;
+                } else {
+                    lowered(i, sh.nb[j]);
+                }
             }
             __syncthreads();
         }
+        if (!more) break;
     }
+    ty.flush(sh.tally);
     block_level_max(next, sh.wmax, &s.lev->lmax[(step + 1) & 3]);
+    if (threadIdx.x < kTally && sh.tally[threadIdx.x])
+        atomicAdd(&s.lev->tally[(step + 1) & 3][threadIdx.x], sh.tally[threadIdx.x]);
 }
 
-// The picks of a level from its n members, by every block on the same input: repeatedly,
-// a member none of whose tumors has a better member is picked (the lexicographically
-// first set, whatever the order of the list), and members that meet what was picked drop
-// out.  U of the block is brought up to date; the lead block (rank 0) records the picks
-// from position K on.  Returns their number; fallen: the largest score + 1 that a member
-// left over still has (a listed record's cached leaf takes all its tumors at FP = 0, so
-// that score bounds the record).  Every thread of the block calls it.
+// The picks of a band from its n members, by every block on the same input.  U of the block
+// is brought up to date; the lead block (rank 0) records the picks from position K on.
+// Returns their number; fallen: the largest score + 1 that a member left over still has (a
+// listed record's cached leaf takes all its tumors at FP = 0, so that score bounds the
+// record).  Every thread of the block calls it.
+
+// Row words of the tumors that carry all genes of k, lane w: word w.
+__device__ __forceinline__ u64 key_rows(const Cohort &c, const Key &k, int h, int lane)
+{
+    u64 y = lane < c.Wt ? ~0ull : 0ull;
+#pragma unroll
+    for (int q = 0; q < kMaxH; ++q)
+        if (q < h && lane < c.Wt) y &= __ldg(c.TO + (size_t)key_get(k, q) * c.WTp + lane);
+    return y;
+}
+__device__ __forceinline__ Key member_key(const Member *m)
+{
+    Key k;
+    k.t0 = __ldcg(&m->t0);
+    k.t1 = __ldcg(&m->t1);
+    k.t2 = __ldcg(&m->t2);
+    k.s = 0;
+    return k;
+}
+// Score + 1 of a member with tp tumors (FP beside the tuple in t2).
+__device__ __forceinline__ u64 member_score(const Cohort &c, const Solve &s, u64 t2, int tp)
+{
+    return s.a_num * (u64)tp + s.a_den * (u64)(c.Nn - (int)((t2 >> 16) & 0xffffull)) + 1;
+}
+constexpr u64 kTupleBits = ~0xffffffffull;  // of t2
+// A pick: its key, TP in the low bits of t2.
+__device__ __forceinline__ void record_pick(const Solve &s, const Key &k, u64 score, int pos, int tp)
+{
+    s.sel[pos] = Key{score, k.t0, k.t1, (k.t2 & kTupleBits) | (u64)tp};
+}
+
+// a_num = 0: one pick, the best member, with every uncovered tumor it covers.
 template <bool kBig>
-__device__ int level_select(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, u64 *best, u64 *Ush, int n, u64 Lk, int step,
-                            int K, bool lead, u64 &fallen)
+__device__ int select_flat(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, u64 *Ush, const Member *mem, int n, u64 Lk,
+                           int K, bool lead)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    Key k = key_empty();
+    for (int i = (int)threadIdx.x; i < n; i += (int)blockDim.x) {
+        Key m = member_key(mem + i);
+        m.s = Lk;
+        if (key_better(m, k)) k = m;
+    }
+    Key *wk = warp_keys();
+    k = warp_max_key(k);
+    if (lane == 0) wk[warp] = k;
+    __syncthreads();
+    if (warp == 0) {
+        k = warp_max_key(lane < nwarps ? wk[lane] : key_empty());
+        if (k.s) {
+            const u64 y = key_rows(c, k, s.h, lane) & (lane < c.Wt ? Ush[lane] : 0ull);
+            const int tp = (int)__reduce_add_sync(kFull, (unsigned)__popcll(y));
+            if (lane < c.Wt) Ush[lane] &= ~y;
+            if (lead)
+                for (u64 x = y; x; x &= x - 1) s.covsel[lane * 64 + __ffsll((long long)x) - 1] = K;
+            if (lane == 0) {
+                sh.k = 1;
+                if (lead) record_pick(s, k, Lk, K, tp);
+            }
+        }
+    }
+    __syncthreads();
+    return sh.k;
+}
+
+// A pool of members (list: their indexes): their tumors as row words on chip (word-major, so
+// that neighbouring threads read neighbouring words), a member per thread.  A member's place
+// in the tuple order is found once, so that its key is one word (score above tau, then place)
+// and the best one is found by one or two 32-bit warp maxima; every warp then takes the pick's
+// tumors out of its own copy of U.  Only the warps that hold members take part (up to 32
+// members: one warp, no barrier).  Whole keys and a block barrier took 1.15 us per pick.  Ends
+// when the best is below tau, or picks all that are left at once when each has one tumor.
+// (Scores above tau fit 24 bits, see the choice of tau.)
+constexpr int kPoolMax = 256;
+struct PoolSh {
+    u64 U[kPoolMax / 32][kMaxWords];
+    u32 w[2][kPoolMax / 32];
+    u32 pr[2][kPoolMax / 32];
+    u64 left;
+    int got;
+    u32 one[kMaxSamples];  // best key of a tumor
+    Key key[kPoolMax];
+    u32 list[kPoolMax];
+    u16 ord[kPoolMax];  // by place: the member
+    u64 y[1];           // Wt x n
+};
+template <bool kBig>
+__device__ int select_pool(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, PoolSh &ps, u64 *Ush, const Member *mem, int n,
+                           u64 tau, int K, bool lead, u64 &fallen)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    for (int i = warp; i < n; i += nwarps) {
+        const Member *src = mem + ps.list[i];
+        const Key k = member_key(src);
+        const int m = (int)__ldcg(&src->k);
+        const int id = lane < kMemIds ? (int)__ldcg(&src->ids[lane]) : 0;
+        u64 y = 0;
+        if (m <= kMemIds) {
+            for (int q = 0; q < m; ++q) {
+                const int x = __shfl_sync(kFull, id, q);
+                if ((x >> 6) == lane) y |= 1ull << (x & 63);
+            }
+        } else {
+            y = key_rows(c, k, s.h, lane) & (lane < c.Wt ? Ush[lane] : 0ull);
+        }
+        if (lane < c.Wt) ps.y[(size_t)lane * n + i] = y;
+        if (lane == 0) ps.key[i] = k;
+    }
+    const int aw = (n + 31) / 32;
+    if (warp < aw) ps.U[warp][lane] = Ush[lane];
+    for (int x = (int)threadIdx.x; x < c.Nt; x += (int)blockDim.x) ps.one[x] = 0;
+    if (threadIdx.x == 0) ps.left = 0;
+    __syncthreads();
+    if (warp < aw) {
+        const auto meet = [&]() {
+            if (aw > 1) asm volatile("bar.sync 1, %0;" ::"r"(32 * aw) : "memory");
+            else __syncwarp();
+        };
+        u64 *U = ps.U[warp];
+        const int i = (int)threadIdx.x;
+        const bool in = i < n;
+        const Key mine = in ? ps.key[i] : key_empty();
+        int place = 0;
+        if (in) {
+            for (int j = 0; j < n; ++j) {  // (equal tuples: a champion and the leaf it is, the same pick)
+                const u64 t0 = ps.key[j].t0;
+                if (t0 < mine.t0) ++place;
+                else if (t0 == mine.t0 && j != i) {
+                    const u64 a1 = ps.key[j].t1, a2 = ps.key[j].t2 & kTupleBits, b2 = mine.t2 & kTupleBits;
+                    if (a1 < mine.t1 || (a1 == mine.t1 && (a2 < b2 || (a2 == b2 && j < i)))) ++place;
+                }
+            }
+            ps.ord[place] = (u16)i;
+        }
+        const u64 base = s.a_den * (u64)(c.Nn - (int)((mine.t2 >> 16) & 0xffffull)) + 1;
+        auto tumors = [&]() {
+            int tp = 0;
+            if (in)
+                for (int w = 0; w < c.Wt; ++w) tp += __popcll(ps.y[(size_t)w * n + i] & U[w]);
+            return tp;
+        };
+        auto cover = [&](u64 y, int pos) {
+            for (u64 b = y; b; b &= b - 1) s.covsel[lane * 64 + __ffsll((long long)b) - 1] = pos;
+        };
+        int got = 0, tp = 0;
+        u32 key = 0;
+        bool ones = false;
+        for (int it = 0;; ++it) {
+            tp = tumors();
+            const u64 sc = base + s.a_num * (u64)tp;
+            key = tp && sc >= tau ? (u32)(sc - tau + 1) << 8 | (u32)(255 - place) : 0u;
+            u32 best = __reduce_max_sync(kFull, key);
+            bool pairs = __any_sync(kFull, key != 0 && tp > 1);
+            if (aw > 1) {  // (two copies: one is read while the next iteration writes the other)
+                if (lane == 0) {
+                    ps.w[it & 1][warp] = best;
+                    ps.pr[it & 1][warp] = pairs;
+                }
+                meet();
+                best = __reduce_max_sync(kFull, lane < aw ? ps.w[it & 1][lane] : 0u);
+                pairs = __any_sync(kFull, lane < aw && ps.pr[it & 1][lane]);
+            } else {
+                __syncwarp();
+            }
+            if (best == 0) break;
+            if (!pairs) {  // a tumor each
+                ones = true;
+                break;
+            }
+            const int win = ps.ord[255 - (best & 255u)];
+            const u64 y = lane < c.Wt ? ps.y[(size_t)lane * n + win] & U[lane] : 0ull;
+            if (lead && warp == aw - 1) {
+                const int t = (int)__reduce_add_sync(kFull, (unsigned)__popcll(y));
+                if (lane == 0) record_pick(s, ps.key[win], (u64)(best >> 8) - 1 + tau, K + got, t);
+                cover(y, K + got);
+            }
+            ++got;
+            __syncwarp();
+            if (lane < c.Wt) U[lane] &= ~y;
+            __syncwarp();
+        }
+        if (ones) {  // the best member of each tumor
+            if (threadIdx.x == 0) ps.got = got;
+            int smp = 0;
+            if (key)
+                for (int w = 0; w < c.Wt; ++w) {
+                    const u64 y = ps.y[(size_t)w * n + i] & U[w];
+                    if (y) smp = w * 64 + __ffsll((long long)y) - 1;
+                }
+            if (key) atomicMax(&ps.one[smp], key);
+            meet();
+            const bool pick = key && ps.one[smp] == key;
+            int pos = 0;
+            if (pick) {
+                pos = atomicAdd(&ps.got, 1);
+                if (lead) {
+                    record_pick(s, mine, (u64)(key >> 8) - 1 + tau, K + pos, 1);
+                    s.covsel[smp] = K + pos;
+                }
+                for (int w = 0; w < aw; ++w) atomicAnd((unsigned long long *)&ps.U[w][smp >> 6], ~(1ull << (smp & 63)));
+            }
+            meet();
+            got = ps.got;
+        }
+        // what the members left over still have (TP = 1 is the champions')
+        tp = tumors();
+        const u64 left = warp_max_u64(in && tp >= 2 ? base + s.a_num * (u64)tp : 0ull);
+        if (lane == 0 && left) atomicMax(&ps.left, left);
+        if (warp == 0) {
+            Ush[lane] = U[lane];
+            if (lane == 0) ps.got = got;
+        }
+    }
+    __syncthreads();
+    fallen = max(fallen, ps.left);
+    return ps.got;
+}
+
+// A level of many members (those of score Lk), most of them pairs: repeatedly, a member none
+// of whose tumors has a better member is picked, and what meets the picks drops out (the
+// lexicographically first set of disjoint ones, whatever the order of the list, in a few
+// repetitions).  Members of up to four tumors and one tuple word (h <= 4)
+// are worked on in shared memory, the smallest tuple per tumor as two 32-bit minima (native
+// atomics; a 64-bit minimum is a loop of exchanges).
+constexpr int kMany = 4096;
+struct ManySh {
+    u64 t[kMany];    // tuple (~0: dropped)
+    u64 id[kMany];   // tumors, 16 bits each, 0xffff: none
+    u32 hi[kMaxSamples], lo[kMaxSamples];
+};
+template <bool kBig>
+__device__ int select_many(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, ManySh &ms, u64 *Ush, const Member *mem, int n,
+                           u64 Lk, int K, bool lead, u64 &fallen)
+{
+    u32 *cov32 = reinterpret_cast<u32 *>(sh.cov);
+    const int T = (int)blockDim.x;
+    for (int i = (int)threadIdx.x; i < n; i += T) {
+        const uint4 *p = reinterpret_cast<const uint4 *>(mem + i);
+        const uint4 a = __ldcg(p), d = __ldcg(p + 1);
+        const int k = (int)(d.z & 0xffffu);
+        const u64 raw = (u64)(d.z >> 16) | (u64)d.w << 16;          // ids 0 .. 2
+        const u64 id3 = k > 3 ? (u64)__ldcg(&mem[i].ids[3]) : 0xffffull;
+        u64 id = raw | id3 << 48;
+        if (k < 4) id |= ~0ull << (16 * k);
+        const bool in = member_score(c, s, (u64)d.y << 32 | d.x, k) == Lk;
+        ms.t[i] = in ? (u64)a.y << 32 | a.x : ~0ull;
+        ms.id[i] = id;
+    }
+    auto each = [&](u64 id, auto &&fn) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int x = (int)((id >> (16 * q)) & 0xffffull);
+            if (x != 0xffff) fn(x);
+        }
+    };
+    int picked = 0;
+    for (;;) {
+        for (int i = (int)threadIdx.x; i < c.Nt; i += T) ms.hi[i] = ms.lo[i] = ~0u;
+        if (threadIdx.x < kMaxWords) sh.cov[threadIdx.x] = 0;
+        if (threadIdx.x == 0) sh.alive = 0;
+        __syncthreads();
+        int live = 0;
+        for (int i = (int)threadIdx.x; i < n; i += T) {
+            const u64 t = ms.t[i], id = ms.id[i];
+            if (t == ~0ull) continue;
+            bool alive = true;
+            each(id, [&](int x) { alive = alive && in_mask(Ush, x); });
+            if (!alive) {
+                ms.t[i] = ~0ull;
+                continue;
+            }
+            ++live;
+            each(id, [&](int x) { atomicMin(&ms.hi[x], (u32)(t >> 32)); });
+        }
+        live = (int)__reduce_add_sync(kFull, (unsigned)live);
+        if ((threadIdx.x & 31) == 0 && live) atomicAdd(&sh.alive, live);
+        __syncthreads();
+        if (sh.alive == 0) break;
+        for (int i = (int)threadIdx.x; i < n; i += T) {
+            const u64 t = ms.t[i], id = ms.id[i];
+            if (t == ~0ull) continue;
+            each(id, [&](int x) { if (ms.hi[x] == (u32)(t >> 32)) atomicMin(&ms.lo[x], (u32)t); });
+        }
+        __syncthreads();
+        for (int i = (int)threadIdx.x; i < n; i += T) {
+            const u64 t = ms.t[i], id = ms.id[i];
+            if (t == ~0ull) continue;
+            bool top = true;
+            each(id, [&](int x) { top = top && ms.hi[x] == (u32)(t >> 32) && ms.lo[x] == (u32)t; });
+            if (!top) continue;
+            const int pos = atomicAdd(&sh.k, 1);
+            int k = 0;
+            each(id, [&](int x) {
+                ++k;
+                atomicOr(&cov32[x >> 5], 1u << (x & 31));
+                if (lead) s.covsel[x] = K + pos;
+            });
+            if (lead) record_pick(s, Key{Lk, t, 0ull, 0ull}, Lk, K + pos, k);
+        }
+        __syncthreads();
+        const int alive = sh.alive, now = sh.k;
+        if (threadIdx.x < kMaxWords) Ush[threadIdx.x] &= ~sh.cov[threadIdx.x];
+        __syncthreads();
+        if (alive == now - picked) break;  // every live member was picked
+        picked = now;
+    }
+    const int got = sh.k;
+    if (got < n) {
+        u64 left = 0;
+        for (int i = (int)threadIdx.x; i < n; i += T) {
+            int kl = 0;
+            each(ms.id[i], [&](int x) { kl += in_mask(Ush, x) ? 1 : 0; });
+            if (kl) left = max(left, member_score(c, s, __ldcg(&mem[i].t2), kl));
+        }
+        left = warp_max_u64(left);
+        if ((threadIdx.x & 31) == 0) sh.wmax[threadIdx.x >> 5] = left;
+        __syncthreads();
+        for (int w = 0; w < T / 32; ++w) fallen = max(fallen, sh.wmax[w]);
+    }
+    return got;
+}
+
+// The same for members of any size and any h, read from memory in every pass; members of
+// more than kMemIds tumors from their rows, a word per lane.
+template <bool kBig>
+__device__ int select_any(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, u64 *best, u64 *Ush, const Member *mem, int n,
+                          u64 Lk, int K, bool lead, u64 &fallen)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int h = s.h, nk = (h + 3) / 4, Nt = c.Nt;
-    const Member *mem = s.mem + (size_t)(step & 1) * s.mcap;
     u32 *cov32 = reinterpret_cast<u32 *>(sh.cov);
     auto key_word = [](const Key &k, int p) { return p == 0 ? k.t0 : (p == 1 ? k.t1 : k.t2); };
-    auto load_key = [&](int i) {
-        Key k;
-        k.s = Lk;
-        k.t0 = __ldcg(&mem[i].t0);
-        k.t1 = __ldcg(&mem[i].t1);
-        k.t2 = __ldcg(&mem[i].t2);
-        return k;
-    };
-    // lane w: word w of the tumors that carry all genes of k
-    auto key_rows = [&](const Key &k) {
-        u64 y = lane < c.Wt ? ~0ull : 0ull;
-#pragma unroll
-        for (int q = 0; q < kMaxH; ++q)
-            if (q < h && lane < c.Wt) y &= __ldg(c.TO + (size_t)key_get(k, q) * c.WTp + lane);
-        return y;
-    };
-    auto record = [&](const Key &k, int pos, int tp) {
-        Key r = k;
-        r.t2 |= (u64)tp;  // below the tuple's bits
-        s.sel[K + pos] = r;
-    };
-    fallen = 0;
-    if (threadIdx.x == 0) sh.k = 0;
-    if (s.a_num == 0) {  // one pick: the best member, with every uncovered tumor it covers
-        Key k = key_empty();
-        for (int i = (int)threadIdx.x; i < n; i += (int)blockDim.x) {
-            const Key m = load_key(i);
-            if (key_better(m, k)) k = m;
-        }
-        Key *wk = warp_keys();
-        k = warp_max_key(k);
-        if (lane == 0) wk[warp] = k;
-        __syncthreads();
-        if (warp == 0) {
-            k = warp_max_key(lane < nwarps ? wk[lane] : key_empty());
-            if (k.s) {
-                const u64 y = key_rows(k) & (lane < c.Wt ? Ush[lane] : 0ull);
-                const int tp = (int)__reduce_add_sync(kFull, (unsigned)__popcll(y));
-                if (lane < c.Wt) Ush[lane] &= ~y;
-                if (lead)
-                    for (u64 x = y; x; x &= x - 1) s.covsel[lane * 64 + __ffsll((long long)x) - 1] = K;
-                if (lane == 0) {
-                    sh.k = 1;
-                    if (lead) record(k, 0, tp);
-                }
-            }
-        }
-        __syncthreads();
-        if (lead && (int)threadIdx.x < c.WTp) s.U[threadIdx.x] = Ush[threadIdx.x];
-        return sh.k;
-    }
     int picked = 0;
     for (;;) {
         for (int i = (int)threadIdx.x; i < nk * Nt; i += (int)blockDim.x) best[i] = ~0ull;
@@ -761,11 +1248,14 @@ __device__ int level_select(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, 
                 Key key = key_empty();
                 key.s = Lk;
                 u32 idw[kMemIds / 2];
+                bool in = false;  // a member of the level
                 if (i < n) {
                     key.t0 = (u64)v[0].y << 32 | v[0].x;
                     key.t1 = (u64)v[0].w << 32 | v[0].z;
                     key.t2 = (u64)v[1].y << 32 | v[1].x;
                     k = (int)(v[1].z & 0xffffu);
+                    in = member_score(c, s, key.t2, k) == Lk;
+                    key.t2 &= kTupleBits;
                     const u32 w[9] = {(v[1].z >> 16) | (v[1].w << 16), (v[1].w >> 16) | (v[2].x << 16),
                                       (v[2].x >> 16) | (v[2].y << 16), (v[2].y >> 16) | (v[2].z << 16),
                                       (v[2].z >> 16) | (v[2].w << 16), (v[2].w >> 16) | (v[3].x << 16),
@@ -774,7 +1264,7 @@ __device__ int level_select(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, 
 #pragma unroll
                     for (int q = 0; q < 9; ++q) idw[q] = w[q];
                 }
-                const bool listed = i < n && k <= kMemIds;
+                const bool listed = in && k <= kMemIds;
                 auto visit = [&](auto &&f) {  // f(tumor) for the listed member's tumors
 #pragma unroll
                     for (int q = 0; q < kMemIds; ++q)
@@ -804,12 +1294,12 @@ __device__ int level_select(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, 
                         visit([&](int smp) { top = top && tied(key, smp, nk); });
                         if (top) {
                             const int pos = atomicAdd(&sh.k, 1);
-                            if (lead) record(key, pos, k);
+                            if (lead) record_pick(s, key, Lk, K + pos, k);
                             visit([&](int smp) { cover(smp, pos); });
                         }
                     }
                 }
-                unsigned big = __ballot_sync(kFull, i < n && !listed), lives = __ballot_sync(kFull, alive);
+                unsigned big = __ballot_sync(kFull, in && !listed), lives = __ballot_sync(kFull, alive);
                 while (big) {  // many tumors: from the rows, a word per lane
                     const int src = __ffs(big) - 1;
                     big &= big - 1;
@@ -818,7 +1308,7 @@ __device__ int level_select(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, 
                     kk.t1 = __shfl_sync(kFull, key.t1, src);
                     kk.t2 = __shfl_sync(kFull, key.t2, src);
                     const int kb = __shfl_sync(kFull, k, src);
-                    const u64 y = key_rows(kk) & (lane < c.Wt ? Ush[lane] : 0ull);
+                    const u64 y = key_rows(c, kk, h, lane) & (lane < c.Wt ? Ush[lane] : 0ull);
                     if ((int)__reduce_add_sync(kFull, (unsigned)__popcll(y)) != kb) continue;
                     lives |= 1u << src;
                     if (pass < nk) {
@@ -833,7 +1323,7 @@ __device__ int level_select(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, 
                         int pos = 0;
                         if (lane == 0) pos = atomicAdd(&sh.k, 1);
                         pos = __shfl_sync(kFull, pos, 0);
-                        if (lead && lane == 0) record(kk, pos, kb);
+                        if (lead && lane == 0) record_pick(s, kk, Lk, K + pos, kb);
                         for (u64 x = y; x; x &= x - 1) cover(lane * 64 + __ffsll((long long)x) - 1, pos);
                     }
                 }
@@ -849,9 +1339,8 @@ __device__ int level_select(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, 
         if (live == now - picked) break;
         picked = now;
     }
-    if (lead && (int)threadIdx.x < c.WTp) s.U[threadIdx.x] = Ush[threadIdx.x];
     const int K1 = sh.k;
-    if (K1 < n) {  // what the members left over fall to (TP = 1 is the champions')
+    if (K1 < n) {  // what the members left over still have (the champions among them too)
         u64 left = 0;
         for (int base = warp * 32; base < n; base += nwarps * 32) {
             const int i = base + lane;
@@ -859,14 +1348,15 @@ __device__ int level_select(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, 
             int kl = 0;
             if (k <= kMemIds)
                 for (int q = 0; q < k; ++q) kl += in_mask(Ush, (int)__ldcg(&mem[i].ids[q])) ? 1 : 0;
-            if (kl >= 2) left = max(left, Lk - s.a_num * (u64)(k - kl));
+            if (kl) left = max(left, member_score(c, s, __ldcg(&mem[i].t2), kl));
             unsigned big = __ballot_sync(kFull, k > kMemIds);
             while (big) {
                 const int src = __ffs(big) - 1;
                 big &= big - 1;
-                const u64 y = key_rows(load_key(base + src)) & (lane < c.Wt ? Ush[lane] : 0ull);
-                const int kb = (int)__reduce_add_sync(kFull, (unsigned)__popcll(y)), k0 = __shfl_sync(kFull, k, src);
-                if (kb >= 2) left = max(left, Lk - s.a_num * (u64)(k0 - kb));
+                const Key ks = member_key(mem + base + src);
+                const u64 y = key_rows(c, ks, h, lane) & (lane < c.Wt ? Ush[lane] : 0ull);
+                const int kb = (int)__reduce_add_sync(kFull, (unsigned)__popcll(y));
+                if (kb) left = max(left, member_score(c, s, ks.t2, kb));
             }
         }
         left = warp_max_u64(left);
@@ -875,6 +1365,86 @@ __device__ int level_select(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, 
         for (int w = 0; w < nwarps; ++w) fallen = max(fallen, sh.wmax[w]);
     }
     return K1;
+}
+
+template <bool kBig>
+__device__ int level_select(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, Batch *scratch, u64 *Ush, int n, u64 Lk,
+                            u64 tau, int step, int K, bool lead, u64 &fallen)
+{
+    const Member *mem = s.mem + (size_t)(step & 1) * s.mcap;
+    fallen = 0;
+    if (n == 0) return 0;
+    static_assert(sizeof(ManySh) <= 16 * sizeof(Batch), "in the batch scratch");
+    PoolSh &ps = *reinterpret_cast<PoolSh *>(scratch);
+    const int room = (int)((sizeof(Batch) * (blockDim.x >> 5) - sizeof(PoolSh)) / (8 * (size_t)c.Wt));
+    const int pool = min(min(kPoolMax, (int)blockDim.x), room), T = (int)blockDim.x;
+    int got = 0, take = n;
+    if (threadIdx.x == 0) sh.k = 0;
+    if (s.a_num == 0) {
+        got = select_flat<kBig>(c, s, sh, Ush, mem, n, Lk, K, lead);
+    } else {
+        if (n > pool && tau < Lk) {
+            // the best members that the pool takes: a histogram by distance to the top, in units
+            // of a_num; the others' best score goes on to the next band
+            constexpr int kBins = kTallyMost + 2;
+            static_assert(kBins <= kMaxSamples, "the histogram in the place of PoolSh::one");
+            u32 *hist = ps.one;
+            for (int i = (int)threadIdx.x; i < kBins; i += T) hist[i] = 0;
+            __syncthreads();
+            auto bin = [&](int i) {
+                const u64 sc = member_score(c, s, __ldcg(&mem[i].t2), (int)__ldcg(&mem[i].k));
+                return (int)((Lk - sc + s.a_num - 1) / s.a_num);  // <= tally_width(kTally - 1) < kBins
+            };
+            for (int i = (int)threadIdx.x; i < n; i += T) atomicAdd(&hist[bin(i)], 1u);
+            __syncthreads();
+            int q = 0;
+            u32 sum = hist[0];
+            take = 0;
+            while (sum <= (u32)pool) {
+                take = (int)sum;
+                if (++q >= kBins) break;
+                sum += hist[q];
+            }
+            --q;  // bins 0 .. q are in the pool
+            if (q >= 0) tau = max(tau, Lk - s.a_num * (u64)q);
+            __syncthreads();
+            u64 out = 0;
+            for (int i = (int)threadIdx.x; i < n; i += T) {
+                if (q >= 0 && bin(i) <= q) {
+                    const int p = atomicAdd(&sh.k, 1);
+                    ps.list[p] = (u32)i;
+                } else {
+                    out = max(out, member_score(c, s, __ldcg(&mem[i].t2), (int)__ldcg(&mem[i].k)));
+                }
+            }
+            out = warp_max_u64(out);
+            if ((threadIdx.x & 31) == 0) sh.wmax[threadIdx.x >> 5] = out;
+            __syncthreads();
+            if (q >= 0)
+                for (int w = 0; w < T / 32; ++w) fallen = max(fallen, sh.wmax[w]);
+            if (threadIdx.x == 0) sh.k = 0;
+            __syncthreads();
+            if (q < 0) take = n;  // the top level alone is more
+        } else if (n <= pool && (tau < Lk || n <= 32)) {
+            for (int i = (int)threadIdx.x; i < n; i += T) ps.list[i] = (u32)i;
+            __syncthreads();
+        }
+        if (take <= pool && (tau < Lk || take <= 32)) {
+            got = take ? select_pool<kBig>(c, s, sh, ps, Ush, mem, take, tau, K, lead, fallen) : 0;
+        } else {  // the top level alone (if there are others, their records are looked at again)
+            bool small = kBig && s.h <= 4 && n <= kMany;
+            if (small) {  // the same answer in every block
+                bool ok = true;
+                for (int i = (int)threadIdx.x; i < n; i += T) ok = ok && __ldcg(&mem[i].k) <= 4;
+                small = __syncthreads_and(ok) != 0;
+            }
+            if (small) got = select_many<kBig>(c, s, sh, *reinterpret_cast<ManySh *>(scratch), Ush, mem, n, Lk, K, lead, fallen);
+            else got = select_any<kBig>(c, s, sh, reinterpret_cast<u64 *>(scratch), Ush, mem, n, Lk, K, lead, fallen);
+        }
+    }
+    if (lead && (int)threadIdx.x < c.WTp) s.U[threadIdx.x] = Ush[threadIdx.x];
+    __syncthreads();  // the scratch and sh.k are free again
+    return got;
 }
 
 // The rounds of a finished solve: the K picks in key order (score, then tuple), the first
@@ -939,9 +1509,7 @@ __device__ __noinline__ void dense_counts(const Cohort &c, const CountOut &out, 
                                           const Rec *src, int l, int ch)
 {
     const int lane = threadIdx.x & 31;
-    Prefix p;
-    p.w0 = __ldcg(&src->p.w0);
-    p.w1 = __ldcg(&src->p.w1);
+    const Prefix p = load_prefix(src);
     const int lo = prefix_gene(p, l - 1) + 1, wi = ch * 32 + lane;
     if (lo > c.G - 1 || ch * 32 + 31 < (lo >> 6)) return;
     u64 y = lane < c.Wt ? ~0ull : 0ull;
@@ -1176,9 +1744,9 @@ __device__ void level_counts(const Cohort &c, const Solve &s, const Frontiers &f
         __syncthreads();
         const int l = h - 1, nchunk = (((c.G - 1) >> 6) + 1 + 31) >> 5;
         if (nq <= LevelSh<kBig>::kQ) {
-            for (int tau = warp; tau < nq * nchunk; tau += nwarps) {
-                const Rec *src = f.F[l] + front_slot(f.cap[l], ft.soff[l], sh.q[tau / nchunk]);
-                dense_counts(c, out, cr, sh.ord, b, src, l, tau % nchunk);
+            for (int x = warp; x < nq * nchunk; x += nwarps) {
+                const Rec *src = f.F[l] + front_slot(f.cap[l], ft.soff[l], sh.q[x / nchunk]);
+                dense_counts(c, out, cr, sh.ord, b, src, l, x % nchunk);
             }
         } else {
             const Share sr((u32)ft.n[l], (u32)t.size, (u32)nwarps, (u32)t.rank);

@@ -1664,10 +1664,16 @@ __device__ void block_rescore(const Cohort &c, const Solve &s, const Key *keys, 
 // single-sample subtrees are then searched and scored like the rest.
 constexpr int kChampBudget = 1 << 15;
 
+// The normal rows of the sample's genes are taken on chip when they fit (kChampWords words):
+// a sample whose few genes are all mutated in normals goes through hundreds of prefixes, each
+// a chain of two or three L2 loads otherwise (the slowest sample of 19,000 genes took 125 us).
+// A prefix that no normal carries gives FP = 0 with its first gene, without looking further.
+constexpr int kChampWords = kBatch * (int)sizeof(Rec) / 8;
 __device__ void phase_champions(const Cohort &c, const Solve &s, const Team &t, Batch &b)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int h = s.h;
+    u64 *rows = reinterpret_cast<u64 *>(b.r);
     for (int smp = t.rank * nwarps + warp; smp < c.Nt; smp += t.size * nwarps) {
         const u32 off = __ldg(c.SO + smp);
         const int m = (int)(__ldg(c.SO + smp + 1) - off);
@@ -1675,6 +1681,16 @@ __device__ void phase_champions(const Cohort &c, const Solve &s, const Team &t, 
         Key best = key_empty();
         int ok = 1;
         if (m >= h) {
+            const int stride = c.Wn | 1;  // odd: neighbouring genes in different banks
+            const bool chip = m * stride <= kChampWords;
+            if (chip) {
+                for (int i = lane; i < m * c.Wn; i += 32) {
+                    const int j = i / c.Wn, w = i - j * c.Wn;
+                    rows[j * stride + w] = __ldg(c.NO + (size_t)__ldg(go + j) * c.WNp + w);
+                }
+                __syncwarp();
+            }
+            auto row = [&](int j) -> const u64 * { return chip ? rows + j * stride : c.NO + (size_t)__ldg(go + j) * c.WNp; };
             int idx[kMaxH];  // positions of the prefix genes 0 .. h-2 (the same in every lane)
             for (int q = 0; q < h - 1; ++q) idx[q] = q;
             int best_fp = 0x7fffffff, best_j = 0, evaluated = 0;
@@ -1685,16 +1701,22 @@ __device__ void phase_champions(const Cohort &c, const Solve &s, const Team &t, 
                 u64 pn = 0;
                 if (lane < c.Wn) {
                     pn = ~0ull;
-                    for (int q = 0; q < h - 1; ++q) pn &= c.N[(size_t)c.inv[go[idx[q]]] * c.WNp + lane];
+                    for (int q = 0; q < h - 1; ++q) pn &= row(idx[q])[lane];
+                }
+                bool zero = false;
+                if (!__any_sync(kFull, pn != 0)) {  // FP = 0 with any gene: the first one
+                    best_fp = 0;
+                    best_j = idx[h - 2] + 1;
+                    for (int q = 0; q < h - 1; ++q) best_idx[q] = idx[q];
+                    break;
                 }
                 b.ns[lane] = pn;
                 __syncwarp();
-                bool zero = false;
                 for (int j0 = idx[h - 2] + 1; j0 < m; j0 += 32) {
                     const int j = j0 + lane;
                     unsigned v = 0xffffffffu;  // (FP, lane): least FP, then the first in order
                     if (j < m) {
-                        const u64 *nrow = c.N + (size_t)c.inv[go[j]] * c.WNp;
+                        const u64 *nrow = row(j);
                         int fp = 0;
                         for (int w = 0; w < c.Wn; ++w) fp += __popcll(b.ns[w] & nrow[w]);
                         v = ((unsigned)fp << 5) | (unsigned)lane;
@@ -1726,8 +1748,8 @@ __device__ void phase_champions(const Cohort &c, const Solve &s, const Team &t, 
             }
             if (ok) {
                 best.s = s.a_num + s.a_den * (u64)(c.Nn - best_fp) + 1;
-                for (int q = 0; q < h - 1; ++q) key_put(best, q, go[best_idx[q]]);
-                key_put(best, h - 1, go[best_j]);
+                for (int q = 0; q < h - 1; ++q) key_put(best, q, __ldg(go + best_idx[q]));
+                key_put(best, h - 1, __ldg(go + best_j));
             }
         }
         if (lane == 0) {
@@ -1800,34 +1822,52 @@ __device__ void block_seed(const Cohort &c, const Solve &s, const Team &t, const
 // positions): with f_k(b) the in-bound k-prefixes of s's genes ending at b,
 // f_1(b) = [b <= hi(1)], f_k(b) = [b <= hi(k)] * sum_{b' < b} f_{k-1}(b'),
 // A_k = sum_b f_k(b) and V_{k+1} = sum_b f_k(b) (hi(k+1) - b).
+// One warp per tumor, a lane per gene: the sums over the earlier genes are warp prefix sums
+// (a thread per tumor walked up to 400 genes one after another: 57 us for 19,000 genes and
+// 800 tumors, now 5).
+__device__ __forceinline__ u64 warp_incl_scan_u64(u64 v, int lane)
+{
+    for (int off = 1; off < 32; off <<= 1) {
+        const u64 o = __shfl_up_sync(kFull, v, off);
+        if (lane >= off) v += o;
+    }
+    return v;
+}
 __device__ __noinline__ void phase_sample_sums(const Cohort &c, const Solve &s, const Team &t)
 {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int h = s.h;
     const int hi0 = c.G - h - 1;  // hi(k) = hi0 + k (0-based, inclusive)
-    for (int smp = t.rank * (int)blockDim.x + (int)threadIdx.x; smp < c.Nt; smp += t.size * (int)blockDim.x) {
+    for (int smp = t.rank * nwarps + warp; smp < c.Nt; smp += t.size * nwarps) {
         const u32 off = __ldg(c.SO + smp);
         const int m = (int)(__ldg(c.SO + smp + 1) - off);
-        u64 S[kMaxH + 1], A[kMaxH + 1], V[kMaxH + 1];
+        u64 S[kMaxH + 1], A[kMaxH + 1], V[kMaxH + 2];  // S: uniform; A, V: the lane's share
 #pragma unroll
         for (int k = 0; k <= kMaxH; ++k) S[k] = A[k] = V[k] = 0;
-        for (int i = 0; i < m; ++i) {
-            const int b = (int)__ldg(c.SL + off + i);
-            // descending k: f_k reads the sum of f_{k-1} over the earlier genes
+        V[kMaxH + 1] = 0;
+        for (int i0 = 0; i0 < m; i0 += 32) {
+            const int b = i0 + lane < m ? (int)__ldg(c.SL + off + i0 + lane) : 0x7fffffff - kMaxH;
+            u64 before = 1;  // sum of f_{k-1} over the earlier genes
 #pragma unroll
-            for (int k = kMaxH; k >= 1; --k) {
-                if (k > h || b > hi0 + k) continue;
-                const u64 f = k == 1 ? 1ull : S[k - 1];
+            for (int k = 1; k <= kMaxH; ++k) {
+                if (k > h) break;
+                const u64 f = b <= hi0 + k ? before : 0ull;
                 A[k] += f;
-                S[k] += f;
-                if (k < h) V[k + 1] += f * (u64)(hi0 + k + 1 - b);
+                if (k < h) V[k + 1] += f * (u64)(b <= hi0 + k ? hi0 + k + 1 - b : 0);
+                const u64 inc = warp_incl_scan_u64(f, lane);
+                before = S[k] + inc - f;
+                S[k] += __shfl_sync(kFull, inc, 31);
             }
         }
         u64 *out = s.ssum + (size_t)smp * 2 * h;
 #pragma unroll
         for (int k = 1; k <= kMaxH; ++k) {
             if (k > h) break;
-            out[k - 1] = A[k];
-            out[h + k - 1] = V[k];
+            const u64 a = warp_sum_u64(A[k]), v = warp_sum_u64(V[k]);
+            if (lane == 0) {
+                out[k - 1] = a;
+                out[h + k - 1] = v;
+            }
         }
     }
 }
@@ -2198,13 +2238,16 @@ __device__ void solve_levels(const Cohort &c, const Solve &s, const Frontiers &f
     }
     u64 Lk = __ldcg(&s.lev->lmax[step & 3]);
     u64 ref = Lk;        // the top that the tally counts from
-    bool wide = true;    // whether the band may take more than the top level
+    // the farthest distance that a band may take (index of tally_width; -1: the top level
+    // alone): nearer when the last band had several times the members that a pool takes,
+    // farther when it had few
+    int qmax = 7;
     bool left;
     if (step0 == 0 && s.a_num) {
         level_tally<kBig>(s, f, sh, t, ft, Lk, 0);
         if (!grid_sync(gsync, s.state, t.size)) return;
     } else {
-        wide = false;
+        qmax = -1;
     }
     for (;;) {
         left = __syncthreads_or(threadIdx.x < kMaxWords && Ush[threadIdx.x] != 0) != 0;
@@ -2213,13 +2256,15 @@ __device__ void solve_levels(const Cohort &c, const Solve &s, const Frontiers &f
         // to evaluate makes a step of 15 us, 16 of them one of 18 us, and most bounds only have
         // to be lowered)
         u64 tau = Lk;
-        if (wide && s.a_num) {
+        int far = -1;
+        if (s.a_num) {
             u32 sum = 0;
-            for (int q = 0; q < kTally; ++q) {
+            for (int q = 0; q <= qmax; ++q) {
                 sum += __ldcg(&s.lev->tally[step & 3][q]);
                 const u64 w = s.a_num * tally_width(q);
                 if (sum > 64u * (u32)t.size || w >= 1ull << 23) break;
                 const u64 x = ref > w ? ref - w : 1ull;
+                far = q;
                 if (x < tau) tau = x;
             }
         }
@@ -2233,8 +2278,9 @@ __device__ void solve_levels(const Cohort &c, const Solve &s, const Frontiers &f
             end_early(kStOverflow, kOverMembers, step + 2, Lk);
             return;
         }
-        wide = n <= s.mcap;
-        if (wide) {
+        if (n > 4u * kPoolMax) qmax = max(far - (n > s.mcap ? 6 : 3), -1);
+        else qmax = min((n > kPoolMax ? far : qmax) + (n > kPoolMax / 2 ? 0 : 3), kTally - 1);
+        if (n <= s.mcap) {
             u64 fallen;
             const int got = level_select<kBig>(c, s, sh, scratch, Ush, (int)n, Lk, tau, step, K, lead, fallen);
             const u64 Lnext = Ln > fallen ? Ln : fallen;

@@ -1504,12 +1504,11 @@ struct CountOut {
 };
 
 // Chunk `ch` (32 column words) of a dense leaf parent's leaves: its tumors' columns in
-// cover order (ord), eight loads in flight.
+// cover order (ord), 16 loads in flight, the sums of 16 tumors added by 16 lanes together.
 __device__ __noinline__ void dense_counts(const Cohort &c, const CountOut &out, const u16 *cr, const u16 *ord, Batch &b,
-                                          const Rec *src, int l, int ch)
+                                          const Prefix &p, int l, int ch)
 {
     const int lane = threadIdx.x & 31;
-    const Prefix p = load_prefix(src);
     const int lo = prefix_gene(p, l - 1) + 1, wi = ch * 32 + lane;
     if (lo > c.G - 1 || ch * 32 + 31 < (lo >> 6)) return;
     u64 y = lane < c.Wt ? ~0ull : 0ull;
@@ -1522,32 +1521,39 @@ __device__ __noinline__ void dense_counts(const Cohort &c, const CountOut &out, 
     const bool on = wi <= (c.G - 1) >> 6 && wi >= (lo >> 6);
     const u64 rw = on ? range_word(wi, lo, c.G - 1) : 0ull;
     u64 m = 0;
-    for (int q0 = 0; q0 < c.Nt; q0 += 32) {
-        const int s0 = q0 + lane < c.Nt ? (int)ord[q0 + lane] : 0;
-        unsigned hit = __ballot_sync(kFull, q0 + lane < c.Nt && in_mask(b.ys, s0));
-        while (hit) {
-            int id[8], n = 0;
-            u64 x[8];
+    int id = 0, n = 0;  // lane q < n: the q-th tumor waiting
+    auto batch = [&](int k) {  // the first k <= 16 of them
+        u64 x[16];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                id[q] = 0;
-                if (hit) {
-                    id[q] = __shfl_sync(kFull, s0, __ffs(hit) - 1);
-                    hit &= hit - 1;
-                    n = q + 1;
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < 8; ++q) x[q] = on && q < n ? __ldg(c.CT + (size_t)id[q] * c.GW + wi) & rw : 0ull;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                if (q >= n) break;
-                const u32 v = __reduce_add_sync(kFull, (u32)__popcll(x[q] & m));
-                m |= x[q];
-                if (lane == 0 && v) out.add(cr[id[q]], 2 * l + 1, v);
-            }
+        for (int q = 0; q < 16; ++q) {
+            const int smp = __shfl_sync(kFull, id, q);
+            x[q] = on && q < k ? __ldg(c.CT + (size_t)smp * c.GW + wi) & rw : 0ull;
         }
+        u32 mine = 0;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            const u32 v = __reduce_add_sync(kFull, (u32)__popcll(x[q] & m));
+            m |= x[q];
+            if (lane == q) mine = v;
+        }
+        if (lane < k && mine) out.add(cr[id], 2 * l + 1, mine);
+        id = __shfl_sync(kFull, id, (lane + k) & 31);
+        n -= k;
+    };
+    for (int q0 = 0; q0 < c.Nt; q0 += 16) {  // the next 16 candidates: lanes 16 .. 31 hold them
+        const int s0 = lane >= 16 && q0 + lane - 16 < c.Nt ? (int)ord[q0 + lane - 16] : -1;
+        const unsigned hit = __ballot_sync(kFull, s0 >= 0 && in_mask(b.ys, s0 < 0 ? 0 : s0));
+        const int k = __popc(hit);
+        if (!k) continue;
+        // append: lane n + i takes the i-th hit
+        const int want = lane - n;
+        const int src = want >= 0 && want < k ? (int)__fns(hit, 0, want + 1) : lane;
+        const int v = __shfl_sync(kFull, s0, src & 31);
+        if (want >= 0 && want < k) id = v;
+        n += k;
+        if (n >= 16) batch(16);
     }
+    if (n) batch(n);
 }
 
 // The counters of all R rounds from cr: see the head of this file.  Every block adds its
@@ -1633,27 +1639,16 @@ __device__ void level_counts(const Cohort &c, const Solve &s, const Frontiers &f
             }
             if (in && !dense) {
                 k = r.ky;
-                const u32 wt = (u32)(hiN - prefix_gene(r.p, l - 1));
-                // its tumors by cover round, last first
-                for (int q = 1; q < k; ++q) {
-                    const u16 id = r.ids[q];
-                    const int x = cr[id];
-                    int p = q - 1;
-                    while (p >= 0 && (int)cr[r.ids[p]] < x) {
-                        r.ids[p + 1] = r.ids[p];
-                        --p;
-                    }
-                    r.ids[p + 1] = id;
-                }
-                if (l >= 2)
-                    for (int q = 1; q < k; ++q) {
-                        const int x = cr[r.ids[q]];
+                if (k == 2) {  // a lane each: the tumor covered first
+                    const int x = min((int)cr[r.ids[0]], (int)cr[r.ids[1]]);
+                    if (l >= 2) {
                         out.add(x, 2 * (l - 1) + 1, 1u);
-                        out.add(x, 2 * l, wt);
+                        out.add(x, 2 * l, (u32)(hiN - prefix_gene(r.p, l - 1)));
                     }
-                if (leafp && k == 2) {  // both tumors: every leaf with TP = 2
-                    const u64 lc = __ldcg(f.lc[l] + i);
-                    if (lc) out.add(cr[r.ids[1]], h2 - 1, (u32)lc);
+                    if (leafp) {  // every leaf of both
+                        const u64 lc = __ldcg(f.lc[l] + i);
+                        if (lc) out.add(x, h2 - 1, (u32)lc);
+                    }
                 }
             }
             __syncwarp();
@@ -1682,48 +1677,97 @@ __device__ void level_counts(const Cohort &c, const Solve &s, const Frontiers &f
                     const int lead = __ffs(__ballot_sync(kFull, mx == top)) - 1;
                     if (lane != lead && mx >= 0) put(mx);
                 }
-            if (!leafp) continue;
-            if (dense) {
+            if (leafp && dense) {
                 const int p = atomicAdd(&sh.qn, 1);
                 if (p < LevelSh<kBig>::kQ) sh.q[p] = i;  // more of them: a second scan below
             }
-            // leaves of the listed leaf parents with three tumors or more: the tumors'
-            // columns in that order; a leaf seen before (it holds a later-covered tumor)
-            // counts at the cover round of each further one
+            // listed nodes of three tumors or more, the warp on one at a time: a lane per tumor
+            // finds its place in the cover order (last first) by counting; all but the first add
+            // the node's weight; then the leaves of a leaf parent, by the tumors' columns in that
+            // order: a leaf seen before (it holds a later-covered tumor) counts at the cover
+            // round of each further one
             unsigned todo = __ballot_sync(kFull, in && !dense && k >= 3);
             while (todo) {
                 const int j = __ffs(todo) - 1;
                 todo &= todo - 1;
-                const Rec &rj = b.r[j];
+                Rec &rj = b.r[j];
                 const int kj = rj.ky, lo = prefix_gene(rj.p, l - 1) + 1;
-                u32 acc[kListT];
+                const int id = lane < kj ? (int)rj.ids[lane] : 0, x = lane < kj ? (int)cr[id] : -1;
+                int place = 0;
+                for (int q = 0; q < kj; ++q) {
+                    const int o = __shfl_sync(kFull, x, q);
+                    place += o > x || (o == x && q < lane) ? 1 : 0;
+                }
+                if (l >= 2 && lane < kj && place > 0) {
+                    out.add(x, 2 * (l - 1) + 1, 1u);
+                    out.add(x, 2 * l, (u32)(hiN - lo + 1));
+                }
+                if (!leafp || lo > c.G - 1) continue;
+                __syncwarp();
+                if (lane < kj) rj.ids[place] = (u16)id;
+                __syncwarp();
+                u32 mine = 0;  // lane q: the sum of the q-th tumor
+                const int w1 = (c.G - 1) >> 6;
+                if (kj <= 4) {  // four words a lane at once
+                    u32 acc[4] = {0, 0, 0, 0};
+                    for (int w0 = lo >> 6; w0 <= w1; w0 += 128) {
+                        u64 v[4][4];
 #pragma unroll
-                for (int q = 0; q < kListT; ++q) acc[q] = 0;
-                for (int w0 = lo >> 6; w0 <= (c.G - 1) >> 6; w0 += 32) {
-                    const int wi = w0 + lane;
-                    const bool on = wi <= (c.G - 1) >> 6;
-                    u64 m = 0;
-                    const u64 rw = on && lo <= c.G - 1 ? range_word(wi, lo, c.G - 1) : 0ull;
+                        for (int u = 0; u < 4; ++u) {
+                            const int wi = w0 + 32 * u + lane;
 #pragma unroll
-                    for (int q0 = 0; q0 < kListT; q0 += 4) {
-                        if (q0 >= kj) break;
-                        u64 x[4];
+                            for (int q = 0; q < 4; ++q)
+                                v[u][q] = wi <= w1 && q < kj ? __ldg(c.CT + (size_t)rj.ids[q] * c.GW + wi) : 0ull;
+                        }
 #pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            x[q] = on && q0 + q < kj ? __ldg(c.CT + (size_t)rj.ids[q0 + q] * c.GW + wi) & rw : 0ull;
+                        for (int u = 0; u < 4; ++u) {
+                            const int wi = w0 + 32 * u + lane;
+                            u64 m = 0;
+                            const u64 rw = wi <= w1 ? range_word(wi, lo, c.G - 1) : 0ull;
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            acc[q0 + q] += (u32)__popcll(x[q] & m);
-                            m |= x[q];
+                            for (int q = 0; q < 4; ++q) {
+                                const u64 z = v[u][q] & rw;
+                                acc[q] += (u32)__popcll(z & m);
+                                m |= z;
+                            }
                         }
                     }
-                }
 #pragma unroll
-                for (int q = 1; q < kListT; ++q) {
-                    if (q >= kj) break;
-                    const u32 v = __reduce_add_sync(kFull, acc[q]);
-                    if (lane == 0 && v) out.add(cr[rj.ids[q]], h2 - 1, v);
+                    for (int q = 1; q < 4; ++q) {
+                        const u32 v = __reduce_add_sync(kFull, acc[q]);
+                        if (lane == q) mine = v;
+                    }
+                } else {
+                    u32 acc[kListT];
+#pragma unroll
+                    for (int q = 0; q < kListT; ++q) acc[q] = 0;
+                    for (int w0 = lo >> 6; w0 <= w1; w0 += 32) {
+                        const int wi = w0 + lane;
+                        u64 m = 0;
+                        const u64 rw = wi <= w1 ? range_word(wi, lo, c.G - 1) : 0ull;
+#pragma unroll
+                        for (int q0 = 0; q0 < kListT; q0 += 10) {
+                            if (q0 >= kj) break;
+                            u64 v[10];
+#pragma unroll
+                            for (int q = 0; q < 10; ++q)
+                                v[q] = wi <= w1 && q0 + q < kj ? __ldg(c.CT + (size_t)rj.ids[q0 + q] * c.GW + wi) & rw : 0ull;
+#pragma unroll
+                            for (int q = 0; q < 10; ++q) {
+                                acc[q0 + q] += (u32)__popcll(v[q] & m);
+                                m |= v[q];
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int q = 1; q < kListT; ++q) {
+                        if (q >= kj) break;
+                        const u32 v = __reduce_add_sync(kFull, acc[q]);
+                        if (lane == q) mine = v;
+                    }
                 }
+                if (mine) out.add(cr[rj.ids[lane]], h2 - 1, mine);
+                __syncwarp();
             }
         }
     }
@@ -1746,7 +1790,7 @@ __device__ void level_counts(const Cohort &c, const Solve &s, const Frontiers &f
         if (nq <= LevelSh<kBig>::kQ) {
             for (int x = warp; x < nq * nchunk; x += nwarps) {
                 const Rec *src = f.F[l] + front_slot(f.cap[l], ft.soff[l], sh.q[x / nchunk]);
-                dense_counts(c, out, cr, sh.ord, b, src, l, x % nchunk);
+                dense_counts(c, out, cr, sh.ord, b, load_prefix(src), l, x % nchunk);
             }
         } else {
             const Share sr((u32)ft.n[l], (u32)t.size, (u32)nwarps, (u32)t.rank);
@@ -1758,7 +1802,7 @@ __device__ void level_counts(const Cohort &c, const Solve &s, const Frontiers &f
                     const int j = __ffs(dm) - 1;
                     dm &= dm - 1;
                     const Rec *sj = (const Rec *)__shfl_sync(kFull, (u64)src, j);
-                    for (int ch = 0; ch < nchunk; ++ch) dense_counts(c, out, cr, sh.ord, b, sj, l, ch);
+                    for (int ch = 0; ch < nchunk; ++ch) dense_counts(c, out, cr, sh.ord, b, load_prefix(sj), l, ch);
                 }
             }
         }

@@ -2278,7 +2278,8 @@ __device__ void solve_levels(const Cohort &c, const Solve &s, const Frontiers &f
             end_early(kStOverflow, kOverMembers, step + 2, Lk);
             return;
         }
-        if (n > 4u * kPoolMax) qmax = max(far - (n > s.mcap ? 6 : 3), -1);
+        // (a band that did not fit always comes nearer, also where the buffers are smaller than a pool)
+        if (n > s.mcap || n > 4u * kPoolMax) qmax = max(far - (n > s.mcap ? 6 : 3), -1);
         else qmax = min((n > kPoolMax ? far : qmax) + (n > kPoolMax / 2 ? 0 : 3), kTally - 1);
         if (n <= s.mcap) {
             u64 fallen;

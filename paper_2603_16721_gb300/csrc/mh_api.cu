@@ -241,8 +241,14 @@ struct mh_handle {
     u32 *dInv = nullptr;
     // solve workspace (grown on demand)
     int ws_h = 0, ws_rounds = 0, ws_slots = 0;
-    u64 *dU = nullptr, *dCnt = nullptr, *dWork = nullptr, *dCut = nullptr;
+    u64 *dU = nullptr;
+    // what a solve leaves for the host, one block read back in one copy: the state, the
+    // diagnostics, then (by the solve's h and round limit) selections, counters and cuts
+    unsigned char *dOut = nullptr;
     int *dState = nullptr, *dRes = nullptr;
+    u64 *dWork = nullptr, *dCnt = nullptr, *dCut = nullptr;
+    int out_rounds = 0, out_h = 0;        // of the current solve
+    bool out_cut = false;
     Key *dSlots = nullptr, *dCand = nullptr, *dChamp = nullptr;
     int *dChampOk = nullptr;
     u64 *dSsum = nullptr;                 // per-sample sums of the counters (Nt x 2h)
@@ -260,16 +266,16 @@ struct mh_handle {
     int coop = 0, pgrid = 0;              // cooperative launch supported; persistent grid size
     std::vector<int> m_s;                 // mutated genes per tumor sample (work estimate of a batch)
     int64_t frontier_bytes = 0;
-    cudaEvent_t evk[2] = {};              // around each cooperative launch of a persistent solve
+    cudaEvent_t evk[4] = {};              // around the cooperative launch of a persistent solve, around the solve
     bool presized[kMaxH] = {};            // frontier of depth l sized from its bound
 
     // device memory goes back to the pool in the order of the handle's stream
     ~mh_handle()
     {
-        for (int i = 0; i < 2; ++i)
+        for (int i = 0; i < 4; ++i)
             if (evk[i]) cudaEventDestroy(evk[i]);
         for (void *p : {(void *)dStore, (void *)dU,
-                        (void *)dCnt, (void *)dCut, (void *)dWork, (void *)dState, (void *)dRes, (void *)dSlots, (void *)dCand, (void *)dChamp, (void *)dChampOk, (void *)dSsum,
+                        (void *)dOut, (void *)dSlots, (void *)dCand, (void *)dChamp, (void *)dChampOk, (void *)dSsum,
                         (void *)dCounts, (void *)dSync})
             dfree(p, stream);
         for (int l = 0; l < kMaxH; ++l) {
@@ -515,6 +521,21 @@ int grow_overflowed(mh_handle *H, int h, const u32 *hc)
 
 int leaf_grid(const mh_handle *H) { return std::max(1, H->num_sms * 4); }
 
+// Offsets of the pieces of dOut for a solve of h hits with room for `rounds` rounds; what a
+// solve without cuts copies back ends at `cut`.
+struct OutLayout {
+    size_t work, res, cnt, cut, end;
+    OutLayout(int rounds, int h)
+    {
+        work = 64;  // after the state
+        res = work + ((sizeof(u64) * (kWorkCount + 2) + 15) & ~(size_t)15);
+        cnt = (res + sizeof(int) * (size_t)rounds * (h + 2) + 15) & ~(size_t)15;
+        cut = cnt + sizeof(u64) * 2 * (size_t)rounds * h;
+        end = cut + sizeof(u64) * (size_t)rounds * h;
+    }
+};
+static_assert(sizeof(int) * kStateWords <= 64, "the state's place in dOut");
+
 int ensure_workspace(mh_handle *H, int h)
 {
     const int rounds = H->Nt + 2;
@@ -527,8 +548,7 @@ int ensure_workspace(mh_handle *H, int h)
     // each piece on its own, so that a call after a failed allocation completes the set
     auto need = [&](auto **p, size_t n) { return *p ? MH_OK : dalloc(p, n, &H->device_bytes, dev, st); };
     const size_t nt1 = (size_t)std::max(H->Nt, 1);
-    if ((rc = need(&H->dU, (size_t)H->c.WTp)) || (rc = need(&H->dState, (size_t)kStateWords)) ||
-        (rc = need(&H->dWork, (size_t)kWorkCount + 2)) || (rc = need(&H->dCounts, (size_t)kCountSets * kCountWords)) ||
+    if ((rc = need(&H->dU, (size_t)H->c.WTp)) || (rc = need(&H->dCounts, (size_t)kCountSets * kCountWords)) ||
         (rc = need(&H->dCand, (size_t)kCandidates)) || (rc = need(&H->dChamp, nt1)) ||
         (rc = need(&H->dChampOk, nt1)) || (rc = need(&H->dSsum, nt1 * 2 * kMaxH)) ||
         (rc = need(&H->dLevel, level_bytes(H->Nt))) || (rc = need(&H->dSync, (size_t)1)))
@@ -539,16 +559,13 @@ int ensure_workspace(mh_handle *H, int h)
         if (!(H->hState = pinned_state_get())) return fail(MH_ENOMEM, "pinned host allocation failed");
     }
     if (h > H->ws_h || rounds > H->ws_rounds) {
-        dfree(H->dCnt, st);
-        dfree(H->dRes, st);
-        dfree(H->dCut, st);
-        H->dCnt = nullptr;
-        H->dRes = nullptr;
-        H->dCut = nullptr;
+        dfree(H->dOut, st);
+        H->dOut = nullptr;
         const int hh = std::max(h, H->ws_h);
-        if ((rc = dalloc(&H->dCnt, (size_t)rounds * hh * 2, &H->device_bytes, dev, st))) return rc;
-        if ((rc = dalloc(&H->dCut, (size_t)rounds * hh, &H->device_bytes, dev, st))) return rc;
-        if ((rc = dalloc(&H->dRes, (size_t)rounds * (hh + 2), &H->device_bytes, dev, st))) return rc;
+        if ((rc = dalloc(&H->dOut, OutLayout(rounds, hh).end, &H->device_bytes, dev, st))) {
+            H->ws_h = H->ws_rounds = 0;
+            return rc;
+        }
         H->ws_h = hh;
         H->ws_rounds = rounds;
     }
@@ -644,6 +661,17 @@ int prepare_solve(mh_handle *H, const mh_solve_opts *opts, Solve *s, int *max_ro
     s->a_num = (u64)opts->alpha.num;
     s->a_den = (u64)opts->alpha.den;
     s->U = H->dU;
+    *max_rounds = H->Nt + 1;
+    if (opts->max_rounds > 0) *max_rounds = std::min(*max_rounds, (int)opts->max_rounds);
+    H->out_rounds = std::min(H->ws_rounds, *max_rounds + 1);
+    H->out_h = h;
+    H->out_cut = opts->prune == MH_PRUNE_BOUND;
+    const OutLayout ol(H->out_rounds, h);
+    H->dState = (int *)H->dOut;
+    H->dWork = (u64 *)(H->dOut + ol.work);
+    H->dRes = (int *)(H->dOut + ol.res);
+    H->dCnt = (u64 *)(H->dOut + ol.cnt);
+    H->dCut = (u64 *)(H->dOut + ol.cut);
     s->state = H->dState;
     s->res = H->dRes;
     s->cnt = H->dCnt;
@@ -670,8 +698,6 @@ int prepare_solve(mh_handle *H, const mh_solve_opts *opts, Solve *s, int *max_ro
     s->xbest = nullptr;
     s->work = H->dWork;
     s->best_hint = H->dWork + kWorkCount;
-    *max_rounds = H->Nt + 1;
-    if (opts->max_rounds > 0) *max_rounds = std::min(*max_rounds, (int)opts->max_rounds);
     return MH_OK;
 }
 
@@ -707,22 +733,11 @@ Frontiers frontiers_of(const mh_handle *H)
     return f;
 }
 
-// Reads a finished solve back into a new mh_result.  kms: the four phase times
-// measured by the caller (used unless the persistent kernel measured them).
-int collect_result(mh_handle *H, int h, bool persistent, double solve_ms, const double *kms_in,
-                   int64_t launches, int64_t leaf_launches, mh_result **out, double kernel_ms = 0.0)
+// Queues the copy of a solve's block dOut into the handle's pinned buffer.
+int queue_result(mh_handle *H)
 {
-    cudaStream_t st = H->stream;
-    // the state, selections, counters, cuts and diagnostics (the arrays at their
-    // capacity: Nt + 2 rounds) into one pinned buffer, one wait
-    const int cap = std::max(1, H->ws_rounds);
-    const size_t bState = sizeof(int) * kStateWords;
-    const size_t oRes = (bState + 15) & ~(size_t)15;
-    const size_t bRes = sizeof(int) * (size_t)cap * (h + 2);
-    const size_t bCnt = sizeof(u64) * (size_t)cap * h * 2;
-    const size_t bCut = sizeof(u64) * (size_t)cap * h;
-    const size_t oCnt = (oRes + bRes + 15) & ~(size_t)15, oCut = oCnt + bCnt, oWork = oCut + bCut;
-    const size_t need = oWork + sizeof(u64) * kWorkCount;
+    const OutLayout ol(H->out_rounds, H->out_h);
+    const size_t need = H->out_cut ? ol.end : ol.cut;
     if (H->hRes_bytes < need) {
         pinned_res_put(H->hRes, H->hRes_bytes);
         H->hRes_bytes = 0;
@@ -732,18 +747,29 @@ int collect_result(mh_handle *H, int h, bool persistent, double solve_ms, const 
             return fail(MH_ENOMEM, "pinned host allocation of the result failed");
         }
     }
-    unsigned char *hb = (unsigned char *)H->hRes;
-    cudaError_t e = cudaMemcpyAsync(hb, H->dState, bState, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && H->dRes) e = cudaMemcpyAsync(hb + oRes, H->dRes, bRes, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && H->dCnt) e = cudaMemcpyAsync(hb + oCnt, H->dCnt, bCnt, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && H->dCut) e = cudaMemcpyAsync(hb + oCut, H->dCut, bCut, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(hb + oWork, H->dWork, sizeof(u64) * kWorkCount, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    const cudaError_t e = cudaMemcpyAsync(H->hRes, H->dOut, need, cudaMemcpyDeviceToHost, H->stream);
     if (e != cudaSuccess) return fail(MH_ECUDA, "reading the result back failed: %s", cudaGetErrorString(e));
+    return MH_OK;
+}
+
+// A finished solve as a new mh_result, from the block that queue_result copied (`read`: it
+// has arrived; otherwise it is queued and waited for here).  kms: the four phase times
+// measured by the caller (used unless the persistent kernel measured them).
+int collect_result(mh_handle *H, int h, bool persistent, double solve_ms, const double *kms_in,
+                   int64_t launches, int64_t leaf_launches, mh_result **out, double kernel_ms = 0.0, bool read = false)
+{
+    if (!read) {
+        const int rc = queue_result(H);
+        if (rc) return rc;
+        const cudaError_t e = cudaStreamSynchronize(H->stream);
+        if (e != cudaSuccess) return fail(MH_ECUDA, "reading the result back failed: %s", cudaGetErrorString(e));
+    }
+    const OutLayout ol(H->out_rounds, H->out_h);
+    const int cap = std::max(1, H->out_rounds);
+    const unsigned char *hb = (const unsigned char *)H->hRes;
     const int *hs = (const int *)hb;
-    const int *res = (const int *)(hb + oRes);
-    const u64 *cnt = (const u64 *)(hb + oCnt), *cut = (const u64 *)(hb + oCut), *work = (const u64 *)(hb + oWork);
+    const int *res = (const int *)(hb + ol.res);
+    const u64 *cnt = (const u64 *)(hb + ol.cnt), *cut = (const u64 *)(hb + ol.cut), *work = (const u64 *)(hb + ol.work);
     const int k = hs[0];
     const int rounds = hs[4];
     if (k < 0 || rounds < 0 || rounds > cap || k > cap) return fail(MH_ECUDA, "inconsistent solve state (k=%d, rounds=%d)", k, rounds);
@@ -762,7 +788,7 @@ int collect_result(mh_handle *H, int h, bool persistent, double solve_ms, const 
         mh_result_free(R);
         return fail(MH_ENOMEM, "host allocation of the result failed");
     }
-    if (rounds) memcpy(R->cut, cut, sizeof(u64) * (size_t)rounds * h);
+    if (rounds && H->out_cut) memcpy(R->cut, cut, sizeof(u64) * (size_t)rounds * h);
     for (int i = 0; i < k; ++i) {
         for (int j = 0; j < h; ++j) R->genes[i * h + j] = res[(size_t)i * (h + 2) + j];
         R->tp[i] = res[(size_t)i * (h + 2) + h];
@@ -910,9 +936,9 @@ MH_API int mh_solve_ex(mh_handle *H, const mh_solve_opts *opts, mh_result **out)
     cudaStream_t st = H->stream;
     const Cohort &c = H->c;
 
-    EventPair total;
-    MH_CUDA(cudaEventCreate(&total.a));
-    MH_CUDA(cudaEventCreate(&total.b));
+    for (int i = 0; i < 4; ++i)
+        if (!H->evk[i]) MH_CUDA(cudaEventCreate(&H->evk[i]));
+    const EventPair total{H->evk[2], H->evk[3]};
     // with time_kernels, events around each kernel of a round: level1 | expand | leaf | finalize
     struct RoundEvents {
         cudaEvent_t ev[5];
@@ -920,8 +946,6 @@ MH_API int mh_solve_ex(mh_handle *H, const mh_solve_opts *opts, mh_result **out)
     };
     std::vector<RoundEvents> round_ev;
     auto destroy_events = [&]() {
-        cudaEventDestroy(total.a);
-        cudaEventDestroy(total.b);
         for (auto &e : round_ev)
             for (int i = 0; i < 5; ++i) cudaEventDestroy(e.ev[i]);
     };
@@ -930,7 +954,7 @@ MH_API int mh_solve_ex(mh_handle *H, const mh_solve_opts *opts, mh_result **out)
     u32 *counts = H->dCounts;
 
     MH_CUDA(cudaEventRecord(total.a, st));
-    launch_solve_init(c, s, H->ws_rounds, max_rounds, counts, kCountSets, st);
+    launch_solve_init(c, s, H->out_rounds, max_rounds, counts, kCountSets, st, H->dSync);
     ++launches;
     const bool persistent = opts->mode == MH_MODE_PERSISTENT && H->pgrid > 0 && H->pgrid <= H->ws_slots;
     // one block of 16 warps per SM unless MH_PERSISTENT_BUILD=large
@@ -939,48 +963,39 @@ MH_API int mh_solve_ex(mh_handle *H, const mh_solve_opts *opts, mh_result **out)
     int rounds_done = 0;
     bool done = H->Nt == 0;  // every tumor covered from the start
     double kernel_ms = 0.0;  // the cooperative launches alone
+    bool read = false;
     if (persistent) {
-        for (int i = 0; i < 2; ++i)
-            if (!H->evk[i]) MH_CUDA(cudaEventCreate(&H->evk[i]));
-        // One cooperative launch runs every round; it returns early only when a
-        // frontier overflowed (grown here, then the round is run again).
+        // One cooperative launch runs every round; it returns early only when a frontier or
+        // the members of a band overflowed (grown here, then it goes on).  Its results are
+        // copied back behind it: one wait per launch.
         while (!done) {
             const Frontiers f = frontiers_of(H);
-            MH_CUDA(cudaMemsetAsync(H->dSync, 0, sizeof(GridSync), st));
+            if (launches > 1) MH_CUDA(cudaMemsetAsync(H->dSync, 0, sizeof(GridSync), st));
             MH_CUDA(cudaEventRecord(H->evk[0], st));
             MH_CUDA(launch_solve_persistent(c, s, f, H->dSync, counts, pgrid, large, st));
             MH_CUDA(cudaEventRecord(H->evk[1], st));
             ++launches;
-            MH_CUDA(cudaMemcpyAsync(H->hState, H->dState, sizeof(int) * kStateWords, cudaMemcpyDeviceToHost, st));
+            if ((rc = queue_result(H))) return rc;
+            MH_CUDA(cudaEventRecord(total.b, st));
             MH_CUDA(cudaStreamSynchronize(st));
-            const int *hs = H->hState;
+            const int *hs = (const int *)H->hRes;
             const u32 *hc = (const u32 *)(H->hState + kStateWords);
             rounds_done = hs[4];
             float kx = 0.f;
             cudaEventElapsedTime(&kx, H->evk[0], H->evk[1]);
             kernel_ms += kx;
-            if (fault_fires(g_fault_timeout)) {
-                destroy_events();
+            if (fault_fires(g_fault_timeout))
                 return fail(MH_ETIMEOUT, "injected timeout (mh_set_fault) after round %d", rounds_done);
-            }
-            if (hs[2]) {
-                destroy_events();
+            if (hs[2])
                 return fail(MH_ETIMEOUT, "a grid barrier of the persistent solve timed out in round %d", rounds_done);
-            }
-            if (hs[3] == kOverMembers) {  // the level is searched again
-                if ((rc = grow_members(H, &s, st))) {
-                    destroy_events();
-                    return rc;
-                }
+            if (hs[3] == kOverMembers) {  // the band is searched again
+                if ((rc = grow_members(H, &s, st))) return rc;
                 continue;
             }
             if (hs[3]) {  // the frontier counters of the overflowed round (its parity's set)
                 MH_CUDA(cudaMemcpy(H->hState + kStateWords, counts + (size_t)(rounds_done & 1) * kCountWords,
                                    sizeof(u32) * kCountWords, cudaMemcpyDeviceToHost));
-                if ((rc = grow_overflowed(H, h, hc))) {
-                    destroy_events();
-                    return rc;
-                }
+                if ((rc = grow_overflowed(H, h, hc))) return rc;
                 MH_CUDA(cudaMemsetAsync(H->dCnt + (size_t)rounds_done * h * 2, 0, sizeof(u64) * 2 * h, st));
                 MH_CUDA(cudaMemsetAsync(H->dCut + (size_t)rounds_done * h, 0, sizeof(u64) * h, st));
                 MH_CUDA(cudaMemsetAsync(counts, 0, sizeof(u32) * kCountSets * kCountWords, st));
@@ -988,6 +1003,7 @@ MH_API int mh_solve_ex(mh_handle *H, const mh_solve_opts *opts, mh_result **out)
                 continue;
             }
             done = true;
+            read = true;
         }
     }
     // Rounds are enqueued in growing batches without waiting: every kernel reads
@@ -1054,10 +1070,15 @@ MH_API int mh_solve_ex(mh_handle *H, const mh_solve_opts *opts, mh_result **out)
         done = hs[1] != 0 || rounds_done >= max_rounds;
         batch = std::min(batch * 2, 64);
     }
-    MH_CUDA(cudaEventRecord(total.b, st));
-    MH_CUDA(cudaStreamSynchronize(st));
-    int rounds = 0;
-    MH_CUDA(cudaMemcpy(&rounds, H->dState + 4, sizeof(int), cudaMemcpyDeviceToHost));
+    if (!read) {
+        if ((rc = queue_result(H))) {
+            destroy_events();
+            return rc;
+        }
+        MH_CUDA(cudaEventRecord(total.b, st));
+        MH_CUDA(cudaStreamSynchronize(st));
+    }
+    const int rounds = ((const int *)H->hRes)[4];
     float ms = 0.f;
     cudaEventElapsedTime(&ms, total.a, total.b);
     // kernel times of the rounds that ran (launches after the last round return at once)
@@ -1074,7 +1095,7 @@ MH_API int mh_solve_ex(mh_handle *H, const mh_solve_opts *opts, mh_result **out)
     }
     destroy_events();
     const int64_t ll = opts->time_kernels && !persistent ? (h >= 2 ? timed : 0) : leaf_launches;
-    return collect_result(H, h, persistent, ms, kms, launches, ll, out, kernel_ms);
+    return collect_result(H, h, persistent, ms, kms, launches, ll, out, kernel_ms, true);
 }
 
 }  // extern "C"
@@ -1261,7 +1282,7 @@ int run_batch(mh_handle *const *hs, const mh_solve_opts *opts, int n, const std:
     bool init_pending = true;
     auto issue_init = [&]() {
         for (int i = 0; i < n; ++i)
-            launch_solve_init(hs[i]->c, ss[i], hs[i]->ws_rounds, maxr[i], hs[i]->dCounts, kCountSets, st);
+            launch_solve_init(hs[i]->c, ss[i], hs[i]->out_rounds, maxr[i], hs[i]->dCounts, kCountSets, st, hs[i]->dSync);
     };
     std::lock_guard<std::mutex> lock(g_items_mutex);
     if (g_items_cap < n) {
@@ -1318,7 +1339,7 @@ int run_batch(mh_handle *const *hs, const mh_solve_opts *opts, int n, const std:
                 key.insert(key.end(), (const char *)p, (const char *)p + bytes);
             };
             for (int i = 0; i < n; ++i) {
-                put(&hs[i]->ws_rounds, sizeof(int));
+                put(&hs[i]->out_rounds, sizeof(int));
                 put(&maxr[i], sizeof(int));
             }
             put(&st, sizeof st);
@@ -1434,9 +1455,8 @@ int run_in_turn(mh_handle *const *hs, const mh_solve_opts *opts, int n, double *
     MH_CUDA(cudaEventRecord(a, st));
     for (int i = 0; i < n; ++i) {
         mh_handle *H = hs[i];
-        launch_solve_init(H->c, ss[i], H->ws_rounds, maxr[i], H->dCounts, kCountSets, st);
+        launch_solve_init(H->c, ss[i], H->out_rounds, maxr[i], H->dCounts, kCountSets, st, H->dSync);
         if (H->Nt == 0) continue;
-        MH_CUDA(cudaMemsetAsync(H->dSync, 0, sizeof(GridSync), st));
         const bool large = use_large_build(H, opts[i].h);
         MH_CUDA(launch_solve_persistent(H->c, ss[i], frontiers_of(H), H->dSync, H->dCounts,
                                         persistent_grid(H->num_sms, large), large, st));
@@ -1622,8 +1642,11 @@ extern "C" MH_API int mh_solve_batch(mh_handle *const *handles, const mh_solve_o
         }
     }
     if (rc) return rc;
+    for (int i = 0; i < n; ++i)  // all the copies queued, each on its handle's stream, then the waits
+        if ((rc = queue_result(handles[i]))) return rc;
     for (int i = 0; i < n; ++i) {
-        rc = collect_result(handles[i], opts[i].h, true, ms, nullptr, 1, 0, &out[i], ms);
+        if (i == 0 || handles[i]->stream != handles[i - 1]->stream) MH_CUDA(cudaStreamSynchronize(handles[i]->stream));
+        rc = collect_result(handles[i], opts[i].h, true, ms, nullptr, 1, 0, &out[i], ms, true);
         if (rc == MH_OK) {
             out[i]->diag[6] = (uint64_t)smm;
             out[i]->diag[7] = (uint64_t)graphed;
@@ -1829,7 +1852,7 @@ struct mh_server {
                 cudaEventDestroy(r->built);
                 r->built = nullptr;
             }
-            launch_solve_init(r->H->c, r->s, r->H->ws_rounds, r->maxr, r->H->dCounts, kCountSets, st);
+            launch_solve_init(r->H->c, r->s, r->H->out_rounds, r->maxr, r->H->dCounts, kCountSets, st, r->H->dSync);
             if (r->Nt == 0) {
                 const int one = 1;
                 cudaMemcpyAsync(r->H->dState + 1, &one, sizeof(int), cudaMemcpyHostToDevice, st);
@@ -1965,10 +1988,14 @@ struct mh_server {
         cudaEventRecord(ev, st);
         // while the launch runs, upload queued requests that fit and ask the launch
         // to end at the next round boundary once one is ready to join
+        // (a launch mostly takes well under a millisecond: no sleep, which is 100 us with the
+        // timer's slack, before two milliseconds have passed)
+        const double t_poll = now_s();
         while (cudaEventQuery(ev) == cudaErrorNotReady) {
             admit_one();
             if (!ready.empty()) *(volatile int *)h_yield = 1;
-            std::this_thread::sleep_for(std::chrono::microseconds(50));
+            if (now_s() - t_poll > 2e-3) std::this_thread::sleep_for(std::chrono::microseconds(50));
+            else std::this_thread::yield();
         }
         cudaEventDestroy(ev);
     }
@@ -2242,7 +2269,7 @@ MH_API int mh_shard_begin(mh_handle *H, const mh_solve_opts *opts, int32_t shard
     X->s.shard = shard;
     X->s.nshards = nshards;
     X->s.xbest = X->dX;
-    launch_solve_init(H->c, X->s, H->ws_rounds, X->max_rounds, H->dCounts, kCountSets, H->stream);
+    launch_solve_init(H->c, X->s, H->out_rounds, X->max_rounds, H->dCounts, kCountSets, H->stream);
     ++X->launches;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {

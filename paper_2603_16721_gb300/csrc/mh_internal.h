@@ -236,9 +236,10 @@ cudaError_t launch_store_build(const StoreBuild &b, cudaStream_t st);
 // overflow flags from Solve::state, so the host can enqueue many rounds ahead.
 // counts: kCountWords u32 (see shard_slot); cap values are per shard.
 // sets: frontier counter sets (and slot arrays, threshold words) to clear: 1 for the
-// one-kernel-per-phase path, kCountSets for a persistent solve.
+// one-kernel-per-phase path, kCountSets for a persistent solve (whose barrier gsync is
+// cleared too).
 void launch_solve_init(const Cohort &c, const Solve &s, int counter_rounds, int max_rounds, u32 *counts, int sets,
-                       cudaStream_t st);
+                       cudaStream_t st, GridSync *gsync = nullptr);
 void launch_level1(const Cohort &c, const Solve &s, const Frontiers &f, u32 *counts, cudaStream_t st);
 void launch_expand(const Cohort &c, const Solve &s, int level, const Frontiers &f, u32 *counts, int grid,
                    cudaStream_t st);

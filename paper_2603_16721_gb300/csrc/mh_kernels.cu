@@ -27,6 +27,8 @@
 // items of the batch's sparse prefixes are spread over the 32 lanes, so
 // neighbouring lanes read neighbouring column words; dense prefixes are taken by
 // the whole warp, one at a time.
+#include <atomic>
+
 #include "mh.h"
 #include "mh_internal.h"
 
@@ -1496,8 +1498,24 @@ __global__ void k_transpose(int G, const u64 *rows, int row_stride, int samples,
     cols[t] = word;
 }
 
-__global__ void k_solve_init(Cohort c, Solve s, int max_rounds)
+// Everything a solve starts from, in one launch instead of ten (with the one copy back, what a
+// solve takes beside its kernel went from 105-130 to 45-65 us): up to kInitParts regions of
+// 8-byte words cleared, covsel set to -1, U and the state.
+constexpr int kInitParts = 10;
+static_assert(sizeof(Key) % 8 == 0 && sizeof(Level) % 8 == 0 && sizeof(GridSync) % 8 == 0 && kCountWords % 2 == 0,
+              "cleared in 8-byte words");
+struct InitParts {
+    u64 *p[kInitParts];
+    u32 n[kInitParts];  // words
+};
+__global__ void k_solve_init(Cohort c, Solve s, int max_rounds, InitParts z)
 {
+    const u32 t = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    for (int k = 0; k < kInitParts; ++k)
+        for (u32 i = t; i < z.n[k]; i += stride) z.p[k][i] = 0;
+    if (s.covsel)
+        for (u32 i = t; i < (u32)c.Nt; i += stride) s.covsel[i] = -1;
+    if (blockIdx.x) return;
     const int w = threadIdx.x;
     if (w < c.WTp) {
         const int rem = c.Nt - 64 * w;
@@ -2529,18 +2547,28 @@ void launch_transpose(const Cohort &c, const u64 *rows, int row_stride, int samp
 }
 
 void launch_solve_init(const Cohort &c, const Solve &s, int counter_rounds, int max_rounds, u32 *counts, int sets,
-                       cudaStream_t st)
+                       cudaStream_t st, GridSync *gsync)
 {
-    cudaMemsetAsync(s.cnt, 0, sizeof(u64) * 2 * (size_t)s.h * (size_t)counter_rounds, st);
-    if (s.cut) cudaMemsetAsync(s.cut, 0, sizeof(u64) * (size_t)s.h * (size_t)counter_rounds, st);
-    cudaMemsetAsync(s.slots, 0, sizeof(Key) * (size_t)s.nslots * sets, st);
-    cudaMemsetAsync(s.cand, 0, sizeof(Key) * (size_t)kCandidates, st);
-    if (s.lev) cudaMemsetAsync(s.lev, 0, sizeof(Level), st);
-    if (s.covsel) cudaMemsetAsync(s.covsel, 0xff, sizeof(int) * (size_t)c.Nt, st);
-    cudaMemsetAsync(s.work, 0, sizeof(u64) * kWorkCount, st);
-    cudaMemsetAsync(s.best_hint, 0, sizeof(u64) * sets, st);
-    cudaMemsetAsync(counts, 0, sizeof(u32) * kCountWords * sets, st);
-    k_solve_init<<<1, 64, 0, st>>>(c, s, max_rounds);
+    InitParts z = {};
+    int n = 0;
+    u64 words = 0;
+    auto clear = [&](void *p, size_t bytes) {
+        if (!p) return;
+        z.p[n] = (u64 *)p;
+        z.n[n++] = (u32)(bytes / 8);
+        words += bytes / 8;
+    };
+    clear(s.cnt, sizeof(u64) * 2 * (size_t)s.h * (size_t)counter_rounds);
+    if (s.prune == MH_PRUNE_BOUND) clear(s.cut, sizeof(u64) * (size_t)s.h * (size_t)counter_rounds);
+    clear(s.slots, sizeof(Key) * (size_t)s.nslots * sets);
+    clear(s.cand, sizeof(Key) * (size_t)kCandidates);
+    clear(s.lev, sizeof(Level));
+    clear(s.work, sizeof(u64) * kWorkCount);
+    clear(s.best_hint, sizeof(u64) * sets);
+    clear(counts, sizeof(u32) * kCountWords * sets);
+    clear(gsync, sizeof(GridSync));
+    const u64 blocks = (words + 1023) / 1024;  // four words a thread
+    k_solve_init<<<(unsigned)(blocks < 1 ? 1 : (blocks > 256 ? 256 : blocks)), 256, 0, st>>>(c, s, max_rounds, z);
 }
 
 int level1_grid(const Cohort &c) { return (c.G + kThreads - 1) / kThreads; }
@@ -2600,14 +2628,33 @@ void launch_finalize_split(const Cohort &c, const Solve &s, u32 *counts, int ste
     k_finalize_split<<<1, kThreads, 0, st>>>(c, s, counts, step);
 }
 
+// Blocks per SM of a kernel on the current device, asked for once per device (an occupancy
+// query takes about 3 us, and a solve asks for four of them).
+constexpr int kMaxDev = 64;
+template <class F>
+static int blocks_per_sm(std::atomic<int> *cache, F &&query)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) return query();
+    int v = cache[dev].load(std::memory_order_relaxed);
+    if (v == 0) {
+        v = query();
+        if (v > 0) cache[dev].store(v, std::memory_order_relaxed);
+    }
+    return v;
+}
+
 int persistent_grid(int num_sms, bool large)
 {
-    int per_sm = 0;
-    const cudaError_t e = large
-        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve<4, kWarpsPerBlock>, kThreads, 0)
-        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve<1, kSmallWarps>, kSmallWarps * 32, 0);
-    if (e != cudaSuccess || per_sm < 1) return 0;
-    return (large ? per_sm : 1) * num_sms;
+    static std::atomic<int> cache[2][kMaxDev];
+    return blocks_per_sm(cache[large], [&] {
+        int per_sm = 0;
+        const cudaError_t e = large
+            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve<4, kWarpsPerBlock>, kThreads, 0)
+            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve<1, kSmallWarps>, kSmallWarps * 32, 0);
+        if (e != cudaSuccess || per_sm < 1) return 0;
+        return large ? per_sm : 1;
+    }) * num_sms;
 }
 
 cudaError_t launch_barrier_probe(GridSync *g, int *state, cudaStream_t st)
@@ -2618,7 +2665,9 @@ cudaError_t launch_barrier_probe(GridSync *g, int *state, cudaStream_t st)
 
 int batch_blocks_per_sm(int build)
 {
-    int per_sm = 0;
+    static std::atomic<int> cache[3][kMaxDev];
+    return blocks_per_sm(cache[build == 1 ? 0 : (build == 3 ? 1 : 2)], [&] {
+        int per_sm = 0;
     const cudaError_t e =
         build == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_batch<1, kSmallWarps>,
                                                                    kSmallWarps * 32, 0)
@@ -2626,8 +2675,9 @@ int batch_blocks_per_sm(int build)
                                                                      kThreads, 0)
                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_batch<4, kWarpsPerBlock>,
                                                                      kThreads, 0);
-    if (e != cudaSuccess) return 0;
-    return build == 1 ? (per_sm >= 1 ? 1 : 0) : per_sm;
+        if (e != cudaSuccess) return 0;
+        return build == 1 ? (per_sm >= 1 ? 1 : 0) : per_sm;
+    });
 }
 
 int batch_grid(int num_sms, int build) { return batch_blocks_per_sm(build) * num_sms; }

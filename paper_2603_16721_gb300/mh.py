@@ -285,7 +285,13 @@ class Result:
 def _to_result(p) -> Result:
     r = p.contents
     k, h, rounds = r.k, r.h, r.rounds
-    arr = lambda ptr, n, dt: np.ctypeslib.as_array(ptr, shape=(n,)).astype(dt, copy=True) if n else np.zeros(0, dt)
+
+    def arr(ptr, n, dt):  # one copy of n values (as_array builds a ctypes type per call: 5 us)
+        a = np.empty(n, dt)
+        if n:
+            ctypes.memmove(a.ctypes.data, ptr, a.nbytes)
+        return a
+
     out = Result(h=h,
                  genes=arr(r.genes, k * h, np.int32).reshape(k, h),
                  tp=arr(r.tp, k, np.int32), fp=arr(r.fp, k, np.int32),

@@ -1,9 +1,11 @@
-"""Edges of the solve by score levels against the CPU oracle (whole numbers: equal).
+"""Edges of the solve by score levels and of the expansions beside it, against the
+CPU oracle (whole numbers: equal).
 
 Cases: weights from 0 (a level is one TP count) to far above the normals' term, two
 to nine hits, sample counts at word boundaries and at the largest, thousands of equal
 scores (bands beyond the pool of picks), buffers of one record (grown on the way,
-bands that do not fit), rows too dense to list."""
+bands that do not fit), rows too dense to list; and the allocation-free solve inside
+and beyond its lists."""
 import numpy as np
 import pytest
 
@@ -60,3 +62,21 @@ def test_edges_match_the_oracle(mh, case, monkeypatch):
                 else:
                     assert np.array_equal(got.visited, ref.visited[:n]) and np.array_equal(got.pruned, ref.pruned[:n])
                     assert not got.cut.any()
+
+
+@pytest.mark.parametrize("G,Nt,Nn,h,dt", [(1, 1, 0, 1, 1.0), (33, 64, 1, 2, 0.2), (300, 65, 0, 3, 0.05), (8192, 1024, 64, 1, 0.01),
+                                          (4096, 257, 30, 2, 0.9), (4600, 257, 30, 2, 0.9)])  # 0.95 and 1.06 million mutations
+def test_noalloc_matches_the_solve(mh, G, Nt, Nn, h, dt):
+    import torch
+
+    bm, _, _ = _random_cohort(np.random.default_rng(G + Nt), G, Nt, Nn, dt, 0.1)
+    with mh.mh_create(bm, G, Nt, Nn) as H:
+        ref = mh.mh_solve(H, h)
+    d = torch.from_numpy(bm.view(np.int64)).to("cuda")
+    out = [torch.full((n,), -1, dtype=torch.int32, device="cuda") for n in (Nt * h, Nt, Nt)]
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    k, rounds = mh.mh_solve_noalloc(d.data_ptr(), G, Nt, Nn, h, (1, 10), stream.cuda_stream, *(x.data_ptr() for x in out), Nt)
+    g, tp, fp = (x.cpu().numpy() for x in out)
+    assert [(tuple(g[i * h:(i + 1) * h].tolist()), int(tp[i]), int(fp[i])) for i in range(k)] == ref.records()
+    assert rounds == ref.rounds and (tp[k:] == -1).all()

@@ -1064,8 +1064,42 @@ __device__ bool phase_expand(const Cohort &c, const Solve &s, int round, int lev
     u64 leaf_vis = 0, leaf_alive = 0;  // closed-form leaves of single-sample children (level = h - 1)
     u64 *deep = acc + kAccDeep;
     const int h = s.h;
-    Dispenser disp((u32)nw, (u32)gw, count, dispenser_counters(counts, level - 2));
-    for (u64 first = disp.next(lane); first < count; first = disp.next(lane)) {
+    // With pruning off and fewer records than the warps' batches hold, a task is 32 children of
+    // a record, from the rows: at G = 300 the 298 depth-1 records kept 298 of 2432 warps busy
+    // with up to 298 children each (32 us per round; 9 us spread over all of them).
+    const bool by_children = all_children && (u64)count < (u64)kBatch * nw;
+    if (by_children) {
+        const u32 nch = (u32)(c.G + 31) / 32;
+        for (u64 x = gw; x < (u64)count * nch; x += nw) {
+            const u32 i = (u32)(x / nch), ch = (u32)(x % nch);
+            Prefix p;
+            p.w0 = (u64)i;
+            p.w1 = 0;
+            if (!io.Ush) p = front_rec(Fin, cap_in, b.soff, i)->p;
+            const int lo = prefix_gene(p, L - 1) + 1, g = (int)ch * 32 + lane;
+            if (ch == 0 && lane == 0 && hi_bound >= lo) visited += (u64)(hi_bound - lo + 1);
+            const bool root = ch == 0 && io.Ush;  // depth 1 is counted here
+            if (!root && ((int)ch * 32 + 31 < lo || (int)ch * 32 > hi_bound)) continue;
+            unsigned by, bn;
+            dense_setup(c, s, p, L, b, by, bn, lane);
+            if (root && lane == 0) {
+                ++d1.visited;
+                d1.pruned += by ? 0 : 1;
+            }
+            const bool in = g >= lo && g <= hi_bound;
+            Rec child;
+            if (in) {
+                child.pad[0] = child.pad[1] = child.pad[2] = 0;
+                child_from_rows(c, b, by, bn, p, L, g, child);
+                alive += (u64)(child.ky > 0);
+            }
+            const u32 pos = warp_reserve(in ? 1 : 0, my_count, lane);
+            if (in && pos < cap) copy_rec(&Fout[pos], &child);
+            __syncwarp();
+        }
+    }
+    Dispenser disp((u32)nw, (u32)gw, by_children ? 0 : count, dispenser_counters(counts, level - 2));
+    for (u64 first = disp.next(lane); !by_children && first < count; first = disp.next(lane)) {
         unsigned dense;
         // the best score known to exist in the round decides whether single-sample
         // subtrees may be counted in closed form

@@ -4,8 +4,9 @@ CPU oracle (whole numbers: equal).
 Cases: weights from 0 (a level is one TP count) to far above the normals' term, two
 to nine hits, sample counts at word boundaries and at the largest, thousands of equal
 scores (bands beyond the pool of picks), buffers of one record (grown on the way,
-bands that do not fit), rows too dense to list; and the allocation-free solve inside
-and beyond its lists."""
+bands that do not fit), rows too dense to list; the exhaustive enumeration by 32
+children of a record, the score bound, and the allocation-free solve inside and
+beyond its lists."""
 import numpy as np
 import pytest
 
@@ -39,6 +40,12 @@ CASES = [
     (90, 2047, 65, 2, 0.3, 0.2, (1, 10), None, "paper"),     # dense: no listed samples
     (40, 2048, 2048, 3, 0.1, 0.05, (1, 10), None, "paper"),
     (120, 2048, 16, 2, 0.004, 0.1, (3, 1), None, "paper"),
+    (33, 70, 70, 3, 0.1, 0.1, (1, 10), None, "off"),         # a word of children and one more
+    (64, 40, 20, 4, 0.2, 0.2, (1, 10), None, "off"),         # and its depth-2 records
+    (97, 500, 300, 2, 0.3, 0.3, (1, 10), 1, "off"),
+    (120, 257, 31, 3, 0.06, 0.05, (1, 2), None, "bound"),    # listed parents
+    (60, 300, 20, 3, 0.4, 0.1, (2, 1), None, "bound"),       # dense ones
+    (22, 200, 64, 5, 0.3, 0.2, (1, 10), 1, "bound"),
 ]
 
 

@@ -284,7 +284,7 @@ MH_API void mh_server_destroy(mh_server *server);
  * code running while another component owns all device memory through its own
  * pool, plug-ins handed fixed buffers by a host framework, or latency-critical
  * streams that must not see allocator traffic -- every piece of scratch lives
- * in one file-scope __device__ array of about 30 MB that every GPU loading this
+ * in one file-scope __device__ array of about 54 MB that every GPU loading this
  * library keeps until the process exits.  It returns the same selections as
  * mh_solve(h, alpha) with MH_PRUNE_PAPER.
  *   d_bitmaps : DEVICE pointer to packed rows (layout above), caller-owned, read only.

@@ -1643,10 +1643,17 @@ extern "C" MH_API int mh_solve_batch(mh_handle *const *handles, const mh_solve_o
     }
     if (rc) return rc;
     for (int i = 0; i < n; ++i)  // all the copies queued, each on its handle's stream, then the waits
-        if ((rc = queue_result(handles[i]))) return rc;
+        if ((rc = queue_result(handles[i]))) {
+            for (int j = 0; j < i; ++j) cudaStreamSynchronize(handles[j]->stream);  // nothing left in flight
+            return rc;
+        }
     for (int i = 0; i < n; ++i) {
-        if (i == 0 || handles[i]->stream != handles[i - 1]->stream) MH_CUDA(cudaStreamSynchronize(handles[i]->stream));
-        rc = collect_result(handles[i], opts[i].h, true, ms, nullptr, 1, 0, &out[i], ms, true);
+        const cudaError_t e = i == 0 || handles[i]->stream != handles[i - 1]->stream
+                                  ? cudaStreamSynchronize(handles[i]->stream)
+                                  : cudaSuccess;
+        rc = e == cudaSuccess
+                 ? collect_result(handles[i], opts[i].h, true, ms, nullptr, 1, 0, &out[i], ms, true)
+                 : fail(MH_ECUDA, "reading the result back failed: %s", cudaGetErrorString(e));
         if (rc == MH_OK) {
             out[i]->diag[6] = (uint64_t)smm;
             out[i]->diag[7] = (uint64_t)graphed;

@@ -2405,15 +2405,15 @@ __device__ void solve_team(const Cohort &c, const Solve &s, const Frontiers &f, 
     }
     __syncthreads();
     // by levels when every tumor's champion is known (the champions stand for the TP = 1
-    // leaves, which that path never visits)
+    // leaves, which that path never visits): a property of the cohort, so that every launch of
+    // a solve takes the same way, whatever its build
     if (h > 1 && s.prune == MH_PRUNE_PAPER && c.CC && s.champ && s.ssum) {
         if (round == 0 && *(volatile int *)&s.state[kStStep] == 0) {
             phase_champions(c, s, t, b);
             phase_sample_sums(c, s, t);
             if (!grid_sync(gsync, s.state, t.size)) return;
         }
-        // (the smallest tuples per tumor take the batch scratch)
-        if (threadIdx.x == 0) fm_sh = (size_t)((h + 3) / 4) * c.Nt * sizeof(u64) <= sizeof(Batch) * (blockDim.x >> 5);
+        if (threadIdx.x == 0) fm_sh = 1;
         __syncthreads();
         for (int i = threadIdx.x; i < c.Nt; i += blockDim.x)
             if (!__ldcg(s.champ_ok + i)) fm_sh = 0;

@@ -1218,17 +1218,28 @@ __device__ int select_many(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, M
 
 // The same for members of any size and any h, read from memory in every pass; members of
 // more than kMemIds tumors from their rows, a word per lane.
+// Per tumor the smallest tuple of a live member: words 0 and 1 (h <= 8: no third), and the one
+// gene of word 2 that h = 9 has (the top of it, in 32 bits, so that the most tumors fit beside
+// the scratch of 8 warps: every build takes every solve by levels, and a solve that a
+// batch stops in one build goes on in any other).
+struct BestSh {
+    u64 w[2][kMaxSamples];
+    u32 last[kMaxSamples];
+};
+static_assert(kMaxH <= 9 && sizeof(BestSh) <= kWarpsPerBlock * sizeof(Batch), "in the batch scratch of the smallest build");
 template <bool kBig>
-__device__ int select_any(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, u64 *best, u64 *Ush, const Member *mem, int n,
-                          u64 Lk, int K, bool lead, u64 &fallen)
+__device__ int select_any(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, BestSh &best, u64 *Ush, const Member *mem,
+                          int n, u64 Lk, int K, bool lead, u64 &fallen)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int h = s.h, nk = (h + 3) / 4, Nt = c.Nt;
     u32 *cov32 = reinterpret_cast<u32 *>(sh.cov);
-    auto key_word = [](const Key &k, int p) { return p == 0 ? k.t0 : (p == 1 ? k.t1 : k.t2); };
     int picked = 0;
     for (;;) {
-        for (int i = (int)threadIdx.x; i < nk * Nt; i += (int)blockDim.x) best[i] = ~0ull;
+        for (int i = (int)threadIdx.x; i < Nt; i += (int)blockDim.x) {
+            best.w[0][i] = best.w[1][i] = ~0ull;
+            best.last[i] = ~0u;
+        }
         if (threadIdx.x < kMaxWords) sh.cov[threadIdx.x] = 0;
         if (threadIdx.x == 0) sh.alive = 0;
         __syncthreads();
@@ -1272,13 +1283,14 @@ __device__ int select_any(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, u6
                 };
                 // whether the member's tuple is the best at tumor smp as far as words < p
                 auto tied = [&](const Key &kk, int smp, int p) {
-                    bool e = true;
-                    for (int a = 0; a < p; ++a) e = e && best[a * Nt + smp] == key_word(kk, a);
-                    return e;
+                    bool e = p < 1 || best.w[0][smp] == kk.t0;
+                    e = e && (p < 2 || best.w[1][smp] == kk.t1);
+                    return e && (p < 3 || best.last[smp] == (u32)(kk.t2 >> 32));
                 };
                 auto lower = [&](const Key &kk, int smp, int p) {
-                    const u64 x = key_word(kk, p);
-                    if (x < best[p * Nt + smp]) atomicMin(&best[p * Nt + smp], x);
+                    const u64 x = p == 0 ? kk.t0 : kk.t1;
+                    if (p == 2) atomicMin(&best.last[smp], (u32)(kk.t2 >> 32));
+                    else if (x < best.w[p][smp]) atomicMin(&best.w[p][smp], x);
                 };
                 auto cover = [&](int smp, int pos) {
                     atomicOr(&cov32[smp >> 5], 1u << (smp & 31));
@@ -1439,7 +1451,7 @@ __device__ int level_select(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, 
                 small = __syncthreads_and(ok) != 0;
             }
             if (small) got = select_many<kBig>(c, s, sh, *reinterpret_cast<ManySh *>(scratch), Ush, mem, n, Lk, K, lead, fallen);
-            else got = select_any<kBig>(c, s, sh, reinterpret_cast<u64 *>(scratch), Ush, mem, n, Lk, K, lead, fallen);
+            else got = select_any<kBig>(c, s, sh, *reinterpret_cast<BestSh *>(scratch), Ush, mem, n, Lk, K, lead, fallen);
         }
     }
     if (lead && (int)threadIdx.x < c.WTp) s.U[threadIdx.x] = Ush[threadIdx.x];

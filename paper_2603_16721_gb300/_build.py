@@ -18,7 +18,7 @@ BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libmh.so")
 
 SOURCES = ["mh_kernels.cu", "mh_api.cu", "mh_noalloc.cu", "mh_diag.cu", "mh_store.cu"]
-HEADERS = ["mh_internal.h", "mh_levels.cuh"]
+HEADERS = ["mh_internal.h", "mh_barrier.h", "mh_levels.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

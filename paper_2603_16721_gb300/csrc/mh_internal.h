@@ -218,10 +218,10 @@ constexpr size_t kSlotBytes = sizeof(Rec) + 2 * sizeof(u64) + sizeof(Key);
 
 // Grid-wide barrier state of the persistent solve (zeroed before each launch):
 // arrived counts the blocks' arrivals over the launch's barriers; flag is raised by
-// a block that found the batch's yield request set when it arrived.
+// a block that found the batch's yield request set when it arrived (see mh_barrier.h).
 struct GridSync {
     unsigned arrived;
-    int flag;
+    unsigned flag;
     unsigned pad[2];
 };
 

@@ -30,6 +30,7 @@
 #include <atomic>
 
 #include "mh.h"
+#include "mh_barrier.h"
 #include "mh_internal.h"
 
 namespace mh {
@@ -1611,8 +1612,9 @@ __global__ void __launch_bounds__(kThreads) k_finalize_split(const __grid_consta
 // One atomic per block: arrivals count up across the barriers of a launch (the
 // word starts at zero), so barrier k ends when the count reaches (k + 1) * nblocks,
 // and a block learns k from the count it found.  With `sample`, a block that finds
-// *sample set raises g->flag before it arrives; after the barrier every block reads
-// the same flag (the OR of what the blocks found), so they take the same decision.
+// *sample set raises g->flag for this barrier before it arrives; after the barrier one
+// thread of every block reads it (*stop: whether a block found the request before this
+// barrier, see mh_barrier.h), so all threads of all blocks take the same decision.
 // Arrival with release and acquire semantics at GPU scope (the block's writes,
 // ordered before thread 0 by the block barrier, become visible to the blocks that
 // see the arrival), and the waiters' acquiring load.
@@ -1628,13 +1630,15 @@ __device__ __forceinline__ unsigned load_acquire(const unsigned *p)
     asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-__device__ __forceinline__ bool grid_sync(GridSync *g, int *state, int nblocks, const int *sample = nullptr)
+__device__ __forceinline__ bool grid_sync(GridSync *g, int *state, int nblocks, const int *sample = nullptr,
+                                          bool *stop = nullptr)
 {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         ok = 1;
-        if (sample && *(volatile const int *)sample) *(volatile int *)&g->flag = 1;
+        if (sample && *(volatile const int *)sample)
+            *(volatile unsigned *)&g->flag = yield_flag(load_acquire(&g->arrived), (unsigned)nblocks);
         const unsigned old = arrive_acq_rel(&g->arrived);
         const unsigned target = (old / (unsigned)nblocks + 1u) * (unsigned)nblocks;
         // the last block to arrive goes on at once; the others wait for the count
@@ -1647,8 +1651,10 @@ __device__ __forceinline__ bool grid_sync(GridSync *g, int *state, int nblocks, 
                 break;
             }
         }
+        if (ok && sample && yield_stops(*(volatile unsigned *)&g->flag, old, (unsigned)nblocks)) ok = 2;
     }
     __syncthreads();
+    if (stop) *stop = ok == 2;
     return ok != 0;
 }
 
@@ -2328,8 +2334,8 @@ __device__ void solve_levels(const Cohort &c, const Solve &s, const Frontiers &f
             }
         }
         level_search<kBig>(c, s, f, sh, b, t, ft, Ush, Lk, tau, step);
-        if (!grid_sync(gsync, s.state, t.size, yield)) return;
-        const bool stop = yield && *(volatile int *)&gsync->flag;
+        bool stop;
+        if (!grid_sync(gsync, s.state, t.size, yield, &stop)) return;
         const u32 n = __ldcg(&s.lev->mcnt[step & 3]);
         const u64 Ln = __ldcg(&s.lev->lmax[(step + 1) & 3]);
         ref = Lk;
@@ -2475,8 +2481,8 @@ __device__ void solve_team(const Cohort &c, const Solve &s, const Frontiers &f, 
         }
         // the round's last barrier; in a batch its releasing block samples the yield
         // request, so that every block of the team takes the same decision
-        if (!grid_sync(gsync, s.state, t.size, yield)) return;
-        const bool stop = yield && *(volatile int *)&gsync->flag;
+        bool stop;
+        if (!grid_sync(gsync, s.state, t.size, yield, &stop)) return;
         pt.lap(s, 2);
         const bool done = end_of_round(c, s, round, io.slots, t.size, t, Ush, cand_sh, s.best_hint + (par ^ 1),
                                        bound ? &thr_sh : nullptr);

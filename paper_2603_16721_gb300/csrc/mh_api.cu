@@ -486,21 +486,29 @@ size_t level_bytes(int Nt)
     return kLevelBytes + nt1 * (sizeof(Key) + sizeof(int) + sizeof(u16));
 }
 
-// Room for n members of a level (at least 8192 of them, or MH_FRONTIER_MIN_RECORDS).
+// Room for n <= kMemberLimit members of a level (at least 8192 of them, or
+// MH_FRONTIER_MIN_RECORDS).  Growing the buffers keeps to the frontier budget; the old ones
+// stay when there is no room for larger ones.
 int ensure_members(mh_handle *H, u64 n)
 {
     if (n <= H->mcap) return MH_OK;
     u64 least = 1u << 13;
     const char *mn = getenv("MH_FRONTIER_MIN_RECORDS");
     if (mn && *mn && atoll(mn) > 0) least = (u64)atoll(mn);
-    const u64 want = std::max<u64>(n + n / 4, least);
-    if (want > 0x7fffffffull) return fail(MH_ENOMEM, "a level of %llu members", (unsigned long long)n);
-    dfree(H->dMem, H->stream);
-    H->dMem = nullptr;
-    H->device_bytes -= (int64_t)(2 * sizeof(Member) * (size_t)H->mcap);
-    H->mcap = 0;
-    const int rc = dalloc(&H->dMem, 2 * (size_t)want, &H->device_bytes, H->dev, H->stream);
+    const u64 want = std::min<u64>(std::max<u64>(n + n / 4, least), kMemberLimit);
+    const int64_t old_bytes = (int64_t)(2 * sizeof(Member) * (size_t)H->mcap);
+    const int64_t new_bytes = (int64_t)(2 * sizeof(Member) * (size_t)want);
+    if (H->mcap) {
+        const char *fixed = getenv("MH_FRONTIER_BUDGET_MB");
+        if ((size_t)(new_bytes + (fixed && *fixed ? H->frontier_bytes : 0)) > frontier_budget(H->dev))
+            return fail(MH_ENOMEM, "%llu members are above the frontier budget", (unsigned long long)n);
+    }
+    Member *p = nullptr;
+    const int rc = dalloc(&p, 2 * (size_t)want, &H->device_bytes, H->dev, H->stream);
     if (rc) return rc;
+    dfree(H->dMem, H->stream);  // stream-ordered: after the kernels that used it
+    H->device_bytes -= old_bytes;
+    H->dMem = p;
     H->mcap = (u32)want;
     return MH_OK;
 }
@@ -691,6 +699,7 @@ int prepare_solve(mh_handle *H, const mh_solve_opts *opts, Solve *s, int *max_ro
         s->cr = (u16 *)(H->dLevel + kLevelBytes + nt1 * (sizeof(Key) + sizeof(int)));
         s->mem = H->dMem;
         s->mcap = H->mcap;
+        s->mlimit = kMemberLimit;
     }
     s->cut = H->dCut;
     s->shard = 0;
@@ -701,17 +710,26 @@ int prepare_solve(mh_handle *H, const mh_solve_opts *opts, Solve *s, int *max_ro
     return MH_OK;
 }
 
-// After a level outgrew the member buffers: larger ones (the largest count seen sets the
-// size), and the level's count starts over.
+// After the level of the step before the last outgrew the member buffers (the solve goes on
+// with it, state word 7 is that step + 2): larger ones; where there is no room for them the
+// solve picks such levels without a list.  st: the stream of the launches.
 int grow_members(mh_handle *H, Solve *s, cudaStream_t st)
 {
     Level lev;
+    int word = 0;
     MH_CUDA(cudaMemcpyAsync(&lev, s->lev, sizeof lev, cudaMemcpyDeviceToHost, st));
+    MH_CUDA(cudaMemcpyAsync(&word, s->state + 7, sizeof word, cudaMemcpyDeviceToHost, st));
     MH_CUDA(cudaStreamSynchronize(st));
-    const int rc = ensure_members(H, *std::max_element(lev.mcnt, lev.mcnt + 4));
-    if (rc) return rc;
-    s->mem = H->dMem;
-    s->mcap = H->mcap;
+    const int rc = ensure_members(H, std::min(lev.mcnt[(word - 2) & 3], kMemberLimit));
+    if (rc == MH_ENOMEM) {
+        cudaGetLastError();
+        s->mlimit = H->mcap;
+    } else if (rc == MH_OK) {
+        s->mem = H->dMem;
+        s->mcap = H->mcap;
+        if (H->stream != st) MH_CUDA(cudaStreamSynchronize(H->stream));  // the new buffers exist for st
+    }
+    if (rc != MH_OK && rc != MH_ENOMEM) return rc;
     MH_CUDA(cudaMemsetAsync(s->state + 3, 0, sizeof(int), st));
     return MH_OK;
 }
@@ -1733,7 +1751,7 @@ int64_t estimate_footprint(const uint64_t *bm, int G, int Nt, int Nn, int h, dou
         bytes += (int64_t)(frontier_records_estimate(sets[l], l) * 1.25 * (double)kSlotBytes) +
                  (int64_t)(2048 * kShards) * (int64_t)kSlotBytes;
     *work = (double)G + sets[h - 1];  // as work_estimate(H, h - 1)
-    return bytes + (64 << 20);
+    return bytes + (64 << 20);  // (the members' buffers, two of 16.8 MB at most, among the rest)
 }
 
 }  // namespace

@@ -119,9 +119,16 @@ struct __align__(16) Member {
 };
 static_assert(sizeof(Member) == 64, "members are 64 bytes, read as four 16-byte words");
 
+// The most members a solve has room for (two buffers of 16.8 MB, grown on demand from 8192).
+// A level with more of them, or with so many that its picks are dearer from the list than one
+// by one, has no list: its best member is found and picked one step at a time (see
+// mh_levels.cuh), which needs no memory.
+constexpr u32 kMemberLimit = 1u << 18;
+
 // Step i of a solve by levels finds the top of its band (score + 1) in lmax[i & 3] and the
 // number of bounds by their distance to the last band's top in tally[i & 3], and counts its
-// members in mcnt[i & 3]; step i - 2 clears the entries.
+// members in mcnt[i & 3] (up to the number that the step has use for); step i - 2 clears the
+// entries.
 constexpr int kTally = 16;     // distances 1, 2, 3, 4, 6, 8, ... 192, 256 (units of a_num)
 constexpr int kTallyMost = 256;
 struct Level {
@@ -165,12 +172,12 @@ struct Solve {
     // mh_kernels.cu).  nullptr: the counters are counted node by node.
     u64 *ssum;
     // Solve by score levels (see mh_levels.cuh; the others leave them nullptr): the
-    // levels' maxima and member counts, two buffers of mcap members, the picks (Nt
-    // entries: score + 1, tuple, TP in the low bits of t2), per tumor the pick that
-    // covers it (-1: none) and the round it is covered in.
+    // levels' maxima and member counts, two buffers of mcap members (which the host can
+    // enlarge to mlimit), the picks (Nt entries: score + 1, tuple, TP in the low bits of t2),
+    // per tumor the pick that covers it (-1: none) and the round it is covered in.
     Level *lev;
     Member *mem;
-    u32 mcap;
+    u32 mcap, mlimit;
     Key *sel;
     int *covsel;
     u16 *cr;
@@ -203,9 +210,10 @@ enum {
 
 // Frontier buffers (depth l at index l): kShards regions of cap[l] records each.
 // A solve by levels keeps for every leaf parent i (depth h-1, by record index): ub = a
-// bound on the score + 1 of its leaves with TP >= 2 (0: none), and over all tumors lb =
-// the best key among those leaves and lc = the sum of TP - 1 over them.  nullptr where
-// not allocated.
+// bound on the score + 1 of its leaves with TP >= 2 (0: none), lb = the best key among those
+// leaves (over the tumors in U when x of them were the record's, x in the low 16 bits of t2;
+// x = 0: over all its tumors; empty: not known) and lc = the sum of TP - 1 over the leaves,
+// over all tumors.  nullptr where not allocated.
 struct Frontiers {
     Rec *F[kMaxH];
     u32 cap[kMaxH];

@@ -2253,8 +2253,9 @@ struct PhaseTimer {
 // and their counters.  A launch may end between two levels (a yield request, or members
 // that outgrew their buffer, the level then being searched again): s.state holds the
 // step to go on with, s.U, s.sel, s.covsel and the bounds the rest.
+constexpr int kOneStep = 1 << 30;  // in kStStep: the step picks one member without a list
 template <bool kBig>
-__device__ void solve_levels(const Cohort &c, const Solve &s, const Frontiers &f, GridSync *gsync, u32 *counts,
+__device__ __forceinline__ void solve_levels(const Cohort &c, const Solve &s, const Frontiers &f, GridSync *gsync, u32 *counts,
                              const Team &t, Batch *scratch, u64 *Ush, int maxr, PhaseTimer &pt, int *yield)
 {
     __shared__ LevelSh<kBig> sh;
@@ -2262,10 +2263,10 @@ __device__ void solve_levels(const Cohort &c, const Solve &s, const Frontiers &f
     Batch &b = scratch[threadIdx.x >> 5];
     const int h = s.h;
     const bool lead = t.rank == 0;
-    auto end_early = [&](int word, int value, int step, u64 level = 0) {
+    auto end_early = [&](int word, int value, int step, u64 level = 0, bool one = false) {
         if (lead && threadIdx.x == 0) {
             s.state[word] = value;
-            s.state[kStStep] = step;  // i + 1: go on with step i, at this level
+            s.state[kStStep] = step | (one ? kOneStep : 0);  // i + 1: go on with step i, at this level
             if (step) s.lev->lmax[(step - 1) & 3] = level;
             if (yield && word == kStOverflow) {  // the other teams stop too, so that the host can act
                 *(volatile int *)yield = 1;
@@ -2273,7 +2274,8 @@ __device__ void solve_levels(const Cohort &c, const Solve &s, const Frontiers &f
             }
         }
     };
-    const int step0 = *(volatile int *)&s.state[kStStep];
+    const int step0 = *(volatile int *)&s.state[kStStep] & ~kOneStep;
+    bool one = (*(volatile int *)&s.state[kStStep] & kOneStep) != 0;
     if (step0 == 0) {
         const RoundIO io{Ush, s.slots, true, s.best_hint, 0, true, true, nullptr};
         if (h == 2) {
@@ -2315,14 +2317,15 @@ __device__ void solve_levels(const Cohort &c, const Solve &s, const Frontiers &f
         qmax = -1;
     }
     for (;;) {
-        left = __syncthreads_or(threadIdx.x < kMaxWords && Ush[threadIdx.x] != 0) != 0;
+        const u32 open = __reduce_add_sync(kFull, (u32)__popcll(Ush[threadIdx.x & 31]));  // uncovered tumors
+        left = open != 0;
         if (Lk == 0 || !left || K >= maxr) break;
         // the band: down to the farthest distance with at most 64 bounds per block (one record
         // to evaluate makes a step of 15 us, 16 of them one of 18 us, and most bounds only have
         // to be lowered)
         u64 tau = Lk;
         int far = -1;
-        if (s.a_num) {
+        if (s.a_num && !one) {
             u32 sum = 0;
             for (int q = 0; q <= qmax; ++q) {
                 sum += __ldcg(&s.lev->tally[step & 3][q]);
@@ -2333,23 +2336,43 @@ __device__ void solve_levels(const Cohort &c, const Solve &s, const Frontiers &f
                 if (x < tau) tau = x;
             }
         }
-        level_search<kBig>(c, s, f, sh, b, t, ft, Ush, Lk, tau, step);
+        const u32 limit = tau == Lk && !one ? level_worth(c, s, Lk, open) : s.mcap;
+        if (__builtin_expect(one, 0))
+            level_search_one<kBig>(c, s, f.F[h - 1], f.cap[h - 1], f.ub[h - 1], f.lb[h - 1], sh, b, t, ft, Ush, Lk, step);
+        else
+            level_search<kBig>(c, s, f, sh, b, t, ft, Ush, Lk, tau, step, limit);
         bool stop;
         if (!grid_sync(gsync, s.state, t.size, yield, &stop)) return;
         const u32 n = __ldcg(&s.lev->mcnt[step & 3]);
         const u64 Ln = __ldcg(&s.lev->lmax[(step + 1) & 3]);
         ref = Lk;
-        if (n > s.mcap && tau == Lk) {  // the level is searched again with larger buffers
+        int got = -1;  // nothing resolved: the top level alone, next
+        u64 Lnext = Lk;
+        if (__builtin_expect(one, 0)) {
+            got = select_one<kBig>(c, s, sh, Ush, step, t.size, Lk, K, lead);
+            if (!got) {  // the level is done
+                Lnext = Ln;
+                one = false;
+            }
+            qmax = -1;  // (its steps do not count the bounds)
+        } else if (tau == Lk && n > limit) {
+            one = true;
+        } else if (n > s.mcap && tau == Lk) {  // the level is searched again with larger buffers
             end_early(kStOverflow, kOverMembers, step + 2, Lk);
             return;
+        } else {
+            // (a band that did not fit always comes nearer, also where the buffers are smaller than a pool)
+            if (n > s.mcap || n > 4u * kPoolMax) qmax = max(far - (n > s.mcap ? 6 : 3), -1);
+            else qmax = min((n > kPoolMax ? far : qmax) + (n > kPoolMax / 2 ? 0 : 3), kTally - 1);
+            if (n <= s.mcap) {
+                u64 fallen;
+                got = level_select<kBig>(c, s, sh, scratch, Ush, (int)n, Lk, tau, step, K, lead, fallen, open);
+                if (got >= 0) Lnext = Ln > fallen ? Ln : fallen;
+                else if (tau == Lk) one = true;
+                else qmax = -1;
+            }
         }
-        // (a band that did not fit always comes nearer, also where the buffers are smaller than a pool)
-        if (n > s.mcap || n > 4u * kPoolMax) qmax = max(far - (n > s.mcap ? 6 : 3), -1);
-        else qmax = min((n > kPoolMax ? far : qmax) + (n > kPoolMax / 2 ? 0 : 3), kTally - 1);
-        if (n <= s.mcap) {
-            u64 fallen;
-            const int got = level_select<kBig>(c, s, sh, scratch, Ush, (int)n, Lk, tau, step, K, lead, fallen);
-            const u64 Lnext = Ln > fallen ? Ln : fallen;
+        if (got >= 0) {
             K += got;
             if (lead && threadIdx.x == 0) s.state[kStK] = K;
             if (got == 0 && Lnext >= Lk) {  // cannot be: a step picks or goes down (no endless loop in any case)
@@ -2357,10 +2380,10 @@ __device__ void solve_levels(const Cohort &c, const Solve &s, const Frontiers &f
                 return;
             }
             Lk = Lnext;
-        }  // else too many members: the top level alone, next
+        }
         ++step;
         if (stop && Lk != 0) {
-            end_early(kStYield, 1, step + 1, Lk);
+            end_early(kStYield, 1, step + 1, Lk, one);
             return;
         }
     }
@@ -2386,8 +2409,12 @@ __device__ void solve_levels(const Cohort &c, const Solve &s, const Frontiers &f
     pt.lap(s, 3);
 }
 
+// (Forced in line, and solve_levels with it: when the kernel grew past the compiler's limit and
+// solve_team became a function, its arguments, kernel parameters before, were read through
+// pointers: 5000 genes, 500 + 300 samples, three hits 537 us to 605, with the score bound
+// 4.87 ms to 5.85.)
 template <bool kBig>
-__device__ void solve_team(const Cohort &c, const Solve &s, const Frontiers &f, GridSync *gsync, u32 *counts_base,
+__device__ __forceinline__ void solve_team(const Cohort &c, const Solve &s, const Frontiers &f, GridSync *gsync, u32 *counts_base,
                            const Team &t, Batch *scratch, int *yield = nullptr)
 {
     __shared__ u64 Ush[kMaxWords];

@@ -52,16 +52,28 @@ struct LevelSh {
     u16 cr[kBig ? kMaxSamples : 1];                   // the round that covers each tumor
     u16 ord[kMaxSamples];                             // the tumors by that round, last first
     int qn, en, ec, nd, alive, k, more;
+    int full;                                         // enough members were counted
 };
 constexpr u32 kDenseBit = 0x80000000u;  // queue entry: an unlisted (dense) record
 // A bound word is a score + 1 (below 2^44) and a flag: the record has members in the band
 // being resolved, its leaves are looked at again in the next one.
 constexpr u64 kEmitted = 1ull << 63;
 
+// The members go to out while there is room (cap) and are counted up to `limit`: the block that
+// passes it raises its flag `full` and counts no more, so that neither the counter nor the time
+// spent on it grows with a level that has no list anyway.
 struct LevelOut {
     Member *out;
     u32 *count;
-    u32 cap;
+    u32 cap, limit;
+    int *full;
+    __device__ __forceinline__ u32 take() const { return *(volatile int *)full ? 0xffffffffu : atomicAdd(count, 1u); }
+    __device__ __forceinline__ bool room(u32 i) const  // of what take returned (its latency ends here)
+    {
+        if (i < cap) return true;
+        if (i >= limit) *(volatile int *)full = 1;
+        return false;
+    }
 };
 
 // Ascending original indices of a prefix of L genes.
@@ -83,8 +95,8 @@ __device__ __forceinline__ void prefix_po(const Cohort &c, const Prefix &p, int 
 // (t2 also takes TP and FP, below the tuple's bits.)
 __device__ __forceinline__ Member *new_member(const LevelOut &o, const Key &k, int tp, int fp)
 {
-    const u32 i = atomicAdd(o.count, 1u);
-    if (i >= o.cap) return nullptr;
+    const u32 i = o.take();
+    if (!o.room(i)) return nullptr;
     Member *m = o.out + i;
     m->t0 = k.t0;
     m->t1 = k.t1;
@@ -100,7 +112,7 @@ __device__ __noinline__ void emit_warp(const Cohort &c, const LevelOut &o, const
 {
     const int lane = threadIdx.x & 31;
     u32 at = 0;
-    if (lane == 0) at = atomicAdd(o.count, 1u);
+    if (lane == 0) at = o.take();
     const int mine = lane < L ? prefix_gene(r.p, lane) : g;
     const int v = lane <= L ? (int)__ldg(c.orig + mine) : 0x10000;
     u64 y = 0;
@@ -125,7 +137,7 @@ __device__ __noinline__ void emit_warp(const Cohort &c, const LevelOut &o, const
         t[w] = (u64)__reduce_or_sync(kFull, (unsigned)(xw >> 32)) << 32 | __reduce_or_sync(kFull, (unsigned)xw);
     }
     at = __shfl_sync(kFull, at, 0);
-    if (at >= o.cap) return;
+    if (!o.room(at)) return;
     Member *m = o.out + at;
     if (lane == 0) {
         m->t0 = t[0];
@@ -184,11 +196,14 @@ __device__ __forceinline__ void load_rec_normals(Rec *dst, const Rec *src)
 }
 
 // Where the evaluation of a window leaves the members it finds: in the block's list, for
-// emit_warp, or beyond its room straight to the level.
+// emit_warp, or beyond its room straight to the level; with `least` only the smallest original
+// index of a record's leaf genes is kept, in least[2 j] (with the record's prefix the smallest
+// tuple: a smaller gene more makes a smaller tuple).
 struct EmitList {
     u64 *em;
     int *n;
     int cap, j;  // j: the record's place in the window
+    u32 *least;
 };
 
 // One (record, column word) item of a listed record in a band: its leaves of scores from
@@ -232,10 +247,14 @@ __device__ __forceinline__ void leaf_item_level(const Cohort &c, const Solve &s,
         const int fp = planes_get(fpl, bt, pn);
         const u64 s1 = b1 - s.a_den * (u64)fp;
         if (s1 >= tau) {
+            emitted = true;
+            if (__builtin_expect(el.least != nullptr, 0)) {
+                atomicMin(el.least + 2 * el.j, (u32)__ldg(c.orig + wi * 64 + bt));
+                continue;
+            }
             const int p = atomicAdd(el.n, 1);
             if (p < el.cap) el.em[p] = (u64)(wi * 64 + bt) | (u64)tp << 16 | (u64)fp << 32 | (u64)el.j << 48;
             else emit_listed(c, o, r, L, wi, bt, tp, fp);
-            emitted = true;
         } else if (s1 > nb) {
             nb = s1;
         }
@@ -378,10 +397,14 @@ __device__ __noinline__ void dense_item_level(const Cohort &c, const Solve &s, c
         const int f = planes_get(fp, bt, pn);
         const u64 s1 = b1 - s.a_den * (u64)f;
         if (s1 >= tau) {
+            emitted = true;
+            if (__builtin_expect(el.least != nullptr, 0)) {
+                atomicMin(el.least + 2 * el.j, (u32)__ldg(c.orig + wi * 64 + bt));
+                continue;
+            }
             const int q = atomicAdd(el.n, 1);
             if (q < el.cap) el.em[q] = (u64)(wi * 64 + bt) | (u64)t << 16 | (u64)f << 32 | (u64)el.j << 48;
             else emit_dense(c, o, p, b.ys, L, wi * 64 + bt, t, f);
-            emitted = true;
         } else if (s1 > nb) {
             nb = s1;
         }
@@ -471,10 +494,11 @@ __device__ __forceinline__ void window_tasks(const Cohort &c, LevelSh<kBig> &sh,
 // The block's window of nw records spread over its warps: listed records in tasks of 32
 // column words, dense ones in tasks of 32 / cg words, cg the smallest that gives every
 // warp two tasks (a single dense record of 19,000 genes: 38 tasks of 8 words).  Then the
-// members found, a warp each.
+// members found, a warp each; or (one) of each record its best leaf of score tau, see
+// EmitList, and the record's |y| beside it.
 template <bool kBig>
 __device__ void window_eval(const Cohort &c, const Solve &s, const LevelOut &o, LevelSh<kBig> &sh, Batch &b, const u64 *Ush,
-                            int nw, int L, u64 tau)
+                            int nw, int L, u64 tau, bool one = false)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     int cg = 1;
@@ -489,7 +513,9 @@ __device__ void window_eval(const Cohort &c, const Solve &s, const LevelOut &o, 
     const int inc0 = warp_incl_scan(i0, lane);
     const int inc1 = __shfl_sync(kFull, inc0, 31) + warp_incl_scan(i1, lane);
     const int T = __shfl_sync(kFull, inc1, 31);
-    EmitList el{sh.em, &sh.ec, LevelSh<kBig>::kEm, 0};
+    u32 *least = one ? reinterpret_cast<u32 *>(sh.em) : nullptr;
+    EmitList el{sh.em, &sh.ec, LevelSh<kBig>::kEm, 0, least};
+    static_assert(LevelSh<kBig>::kEm >= LevelSh<kBig>::kWin, "two words per record of the window");
     for (int x = warp; x < T; x += nwarps) {
         // its record: the number of records whose tasks end at or before x
         const int j = __popc(__ballot_sync(kFull, lane < nw && inc0 <= x)) +
@@ -505,6 +531,7 @@ __device__ void window_eval(const Cohort &c, const Solve &s, const LevelOut &o, 
             unsigned by, bn;
             int kn;
             const int k = dense_words(c, Ush, r.p, L, b, by, bn, kn, lane);
+            if (one && lane == 0) least[2 * j + 1] = (u32)k;
             const int wi = (lo >> 6) + (x - first) * dw + (lane & (dw - 1));
             dense_item_level(c, s, o, el, b, r.p, by, bn, k, kn, L, lo, wi, cg, tau, nb, emitted);
             __syncwarp();
@@ -518,6 +545,7 @@ __device__ void window_eval(const Cohort &c, const Solve &s, const LevelOut &o, 
         if (lane == 0 && em) sh.emit[j] = 1;
     }
     __syncthreads();
+    if (one) return;
     const int ne = sh.ec < LevelSh<kBig>::kEm ? sh.ec : LevelSh<kBig>::kEm;
     for (int e = warp; e < ne; e += nwarps) {
         const u64 m = sh.em[e];
@@ -588,11 +616,11 @@ __device__ void level_first(const Cohort &c, const Solve &s, const Frontiers &f,
             u64 nb = 0;
             bool em = false;
             for (int w0 = lo >> 6; w0 <= (c.G - 1) >> 6; w0 += 32)
-                dense_item_level(c, s, LevelOut{nullptr, nullptr, 0u}, EmitList{nullptr, nullptr, 0, 0}, b, p, by, bn, ky, kn,
-                                 l, lo, w0 + lane, 1, ~0ull, nb, em);
+                dense_item_level(c, s, LevelOut{}, EmitList{}, b, p, by, bn, ky, kn, l, lo, w0 + lane, 1, ~0ull, nb, em);
             nb = warp_max_u64(nb);
             if (lane == j) {
                 ub[i] = nb;
+                f.lb[l][i].s = 0;
                 best = nb > best ? nb : best;
             }
             __syncwarp();
@@ -612,11 +640,12 @@ __device__ void level_first(const Cohort &c, const Solve &s, const Frontiers &f,
             window_tasks<kBig>(c, sh, j, sh.rec[j].p, l, true);
         }
         __syncthreads();
-        window_eval<kBig>(c, s, LevelOut{nullptr, nullptr, 0u}, sh, b, Ush, nw, l, ~0ull);
+        window_eval<kBig>(c, s, LevelOut{}, sh, b, Ush, nw, l, ~0ull);
         __syncthreads();
         if (j < nw) {
             const u64 v = sh.nb[j];
             ub[sh.ri[j] & ~kDenseBit] = v;
+            f.lb[l][sh.ri[j] & ~kDenseBit].s = 0;
             best = v > best ? v : best;
         }
         __syncthreads();
@@ -679,25 +708,37 @@ __device__ void level_tally(const Solve &s, const Frontiers &f, LevelSh<kBig> &s
     if (threadIdx.x < kTally && sh.tally[threadIdx.x]) atomicAdd(&s.lev->tally[step & 3][threadIdx.x], sh.tally[threadIdx.x]);
 }
 
+// The step after the next starts from zero (rank 0).
+__device__ __forceinline__ void level_clear(const Solve &s, const Team &t, int step)
+{
+    if (t.rank != 0) return;
+    if (threadIdx.x == 0) {
+        s.lev->lmax[(step + 2) & 3] = 0;
+        s.lev->mcnt[(step + 2) & 3] = 0;
+    }
+    if (threadIdx.x < kTally) s.lev->tally[(step + 2) & 3][threadIdx.x] = 0;
+}
+
 // The band of step `step`, scores + 1 from tau to Lk: the block's share of the leaf parents
-// and champions whose scores reach tau leaves its members, and the largest bound below it
-// counts for the next band.  Every thread of the block calls it; a grid barrier follows.
+// and champions whose scores reach tau leaves its members (counted up to `limit`), and the
+// largest bound below it counts for the next band.  Every thread of the block calls it; a grid
+// barrier follows.
 template <bool kBig>
 __device__ void level_search(const Cohort &c, const Solve &s, const Frontiers &f, LevelSh<kBig> &sh, Batch &b, const Team &t,
-                             const FrontTab &ft, const u64 *Ush, u64 Lk, u64 tau, int step)
+                             const FrontTab &ft, const u64 *Ush, u64 Lk, u64 tau, int step, u32 limit)
 {
     constexpr int kIlpS = LevelSh<kBig>::kIlp, kWin = LevelSh<kBig>::kWin, kQ = LevelSh<kBig>::kQ;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int l = s.h - 1;
     u64 *ub = f.ub[l];
-    if (t.rank == 0) {  // the step after the next starts from zero
-        if (threadIdx.x == 0) {
-            s.lev->lmax[(step + 2) & 3] = 0;
-            s.lev->mcnt[(step + 2) & 3] = 0;
-        }
-        if (threadIdx.x < kTally) s.lev->tally[(step + 2) & 3][threadIdx.x] = 0;
+    level_clear(s, t, step);
+    const LevelOut o{s.mem + (size_t)(step & 1) * s.mcap, &s.lev->mcnt[step & 3], s.mcap, limit, &sh.full};
+    if (threadIdx.x == 0) {
+        sh.full = 0;
+        sh.qn = sh.en = sh.ec = sh.nd = sh.more = 0;
     }
-    const LevelOut o{s.mem + (size_t)(step & 1) * s.mcap, &s.lev->mcnt[step & 3], s.mcap};
+    if (threadIdx.x < kTally) sh.tally[threadIdx.x] = 0;
+    __syncthreads();
     const u64 top = s.a_den * (u64)c.Nn + 1, unit = s.a_num < s.a_den ? s.a_num : s.a_den;
     u64 next = 0;
     // with a_num = 0 a score does not depend on TP: a champion is the best of all the
@@ -730,13 +771,14 @@ __device__ void level_search(const Cohort &c, const Solve &s, const Frontiers &f
     }
     const Share sr((u32)ft.n[l], (u32)t.size, (u32)nwarps, (u32)t.rank);
     const u32 steps = flat ? 0u : sr.steps();
-    if (threadIdx.x < kTally) sh.tally[threadIdx.x] = 0;
     Tally ty;
     for (int pass = 0; steps > 0; ++pass) {
         // the block's bounds; those that reach tau are queued (what does not fit is found by
         // another scan after the queue is done: its bounds still reach tau)
-        if (threadIdx.x == 0) sh.qn = sh.en = sh.ec = sh.nd = sh.more = 0;
-        __syncthreads();
+        if (pass > 0) {
+            if (threadIdx.x == 0) sh.qn = sh.en = sh.ec = sh.nd = sh.more = 0;
+            __syncthreads();
+        }
         for (u32 k0 = 0; k0 < steps; k0 += kIlpS) {
             u64 v[kIlpS];
 #pragma unroll
@@ -817,7 +859,7 @@ __device__ void level_search(const Cohort &c, const Solve &s, const Frontiers &f
                 if (bound < tau) {
                     lowered(i, bound);
                 } else if (!dense && k == k0y && bound - unit < tau && __ldcg(&f.lb[l][i].s) == bound) {
-                    Key kc;
+                    Key kc;  // (of all the record's tumors: no count in t2)
                     kc.t0 = __ldcg(&f.lb[l][i].t0);
                     kc.t1 = __ldcg(&f.lb[l][i].t1);
                     kc.t2 = __ldcg(&f.lb[l][i].t2);
@@ -889,11 +931,200 @@ __device__ void level_search(const Cohort &c, const Solve &s, const Frontiers &f
         atomicAdd(&s.lev->tally[(step + 1) & 3][threadIdx.x], sh.tally[threadIdx.x]);
 }
 
-// The picks of a band from its n members, by every block on the same input.  U of the block
-// is brought up to date; the lead block (rank 0) records the picks from position K on.
-// Returns their number; fallen: the largest score + 1 that a member left over still has (a
-// listed record's cached leaf takes all its tumors at FP = 0, so that score bounds the
-// record).  Every thread of the block calls it.
+// The most members of level Lk that are worth a list, with `left` tumors uncovered: every
+// pick covers at least tp of them (more normals take more tumors to the same score), so
+// there are at most left / tp picks to come.  A list costs every block some passes over it,
+// 0.02 us a member (0.8 us with more tumors than it lists, their rows are read), a pick
+// without a list one step of about 15 us: 700 or 20 members a pick.
+__device__ __forceinline__ u32 members_worth(u32 left, u32 tp, bool big)
+{
+    const u32 picks = max(left / max(tp, 1u), 1u);
+    return big ? max(20u * picks, 64u) : max(700u * picks, 4096u);
+}
+__device__ __forceinline__ u32 level_worth(const Cohort &c, const Solve &s, u64 Lk, u32 left)
+{
+    const u64 base = s.a_den * (u64)c.Nn + 1;
+    u64 tp = Lk > base && s.a_num ? (Lk - base + s.a_num - 1) / s.a_num : 1ull;
+    tp = tp < 2048 ? tp : 2048;
+    return min(s.mlimit, members_worth(left, (u32)tp, tp > kMemIds));
+}
+
+// A step of a level with more members than are worth a list: the best member of the block's
+// share (score Lk, the smallest tuple) goes to the block's slot.  A record's best leaf is kept in lb with the number of the record's tumors in U, and
+// is valid while that many are left (U only shrinks), so a step evaluates only the
+// records that the last picks touched; the others are read from lb.  Every thread of the block
+// calls it; a grid barrier follows.
+template <bool kBig>
+__device__ __noinline__ void level_search_one(const Cohort &c, const Solve &s, const Rec *F, u32 cap, u64 *ub, Key *lb,
+                                              LevelSh<kBig> &sh, Batch &b, const Team &t, const FrontTab &ft,
+                                              const u64 *Ush, u64 Lk, int step)
+{
+    constexpr int kWin = LevelSh<kBig>::kWin, kQ = LevelSh<kBig>::kQ;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int l = s.h - 1;
+    level_clear(s, t, step);
+    const u64 top = s.a_den * (u64)c.Nn + 1;
+    u64 next = 0;
+    u32 *least = reinterpret_cast<u32 *>(sh.em);
+    Key *wb = warp_keys();  // the warp's best member so far
+    if (lane == 0) wb[warp] = key_empty();
+    __syncwarp();
+    auto offer = [&](Key k) {  // by the whole warp; an empty key: none
+        if (!__any_sync(kFull, k.s != 0)) return;
+        k.t2 &= ~0xffffffffull;
+        k = warp_max_key(k);
+        if (lane == 0 && key_better(k, wb[warp])) wb[warp] = k;
+    };
+    auto load_key = [](const Key *p) {
+        Key k;
+        k.s = __ldcg(&p->s);
+        k.t0 = __ldcg(&p->t0);
+        k.t1 = __ldcg(&p->t1);
+        k.t2 = __ldcg(&p->t2);
+        return k;
+    };
+    for (int s0 = t.rank * (int)blockDim.x; s0 < c.Nt; s0 += t.size * (int)blockDim.x) {
+        const int smp = s0 + (int)threadIdx.x;
+        Key k = key_empty();
+        if (smp < c.Nt && in_mask(Ush, smp)) {
+            const u64 v = __ldcg(&s.champ[smp].s);
+            if (v == Lk) k = load_key(s.champ + smp);
+            else if (v < Lk && v > next) next = v;
+        }
+        offer(k);
+    }
+    const Share sr((u32)ft.n[l], (u32)t.size, (u32)nwarps, (u32)t.rank);
+    const u32 steps = sr.steps();
+    auto lowered = [&](u32 i, u64 v) {
+        ub[i] = v;
+        next = v > next ? v : next;
+    };
+    for (int pass = 0; steps > 0; ++pass) {  // as in level_search: what does not fit the queue is found by another scan
+        if (threadIdx.x == 0) sh.qn = sh.en = sh.more = 0;
+        __syncthreads();
+        for (u32 k0 = 0; k0 < steps; ++k0) {
+            const u32 i = sr.at(k0, (u32)warp, (u32)lane);
+            u64 w = i < sr.n ? __ldcg(ub + i) : 0ull;
+            if (w & kEmitted) {
+                if (pass > 0) continue;  // done in this step
+                w &= ~kEmitted;
+                ub[i] = w;
+            }
+            if (w >= Lk) {
+                const int p = atomicAdd(&sh.qn, 1);
+                if (p < kQ) sh.q[p] = i;
+                else sh.more = 1;
+            } else if (w && pass == 0) {
+                next = w > next ? w : next;
+            }
+        }
+        __syncthreads();
+        const int nq = sh.qn < kQ ? sh.qn : kQ;
+        const bool more = sh.more != 0;
+        for (int q0 = 0; q0 < nq; q0 += (int)blockDim.x) {
+            const int qi = q0 + lane * nwarps + warp;
+            const bool act = qi < nq;
+            const u32 i = act ? sh.q[qi] : 0u;
+            __syncthreads();  // entries of this pass are read before the records to evaluate overwrite them
+            Rec &r = b.r[lane];
+            bool dense = false;
+            int k = 0, k0y = 0;
+            if (act) {
+                load_rec_tumors(&r, F + front_slot(cap, ft.soff[l], i));
+                dense = is_dense(r.ky, r.kn);
+                k0y = r.ky;
+                if (!dense)
+                    for (int q = 0; q < k0y; ++q) k += in_mask(Ush, r.ids[q]) ? 1 : 0;
+            }
+            __syncwarp();
+            unsigned dm = __ballot_sync(kFull, dense);
+            while (dm) {
+                const int j = __ffs(dm) - 1;
+                dm &= dm - 1;
+                u64 y = 0;
+                if (lane < c.Wt) {
+                    y = Ush[lane];
+#pragma unroll
+                    for (int q = 0; q < kMaxH - 1; ++q)
+                        if (q < l) y &= __ldg(c.T + (size_t)prefix_gene(b.r[j].p, q) * c.WTp + lane);
+                }
+                const int ky = (int)__reduce_add_sync(kFull, (unsigned)__popcll(y));
+                if (lane == j) k = ky;
+            }
+            Key best = key_empty();
+            if (act) {
+                const u64 bound = k >= 2 ? s.a_num * (u64)k + top : 0ull;
+                if (bound < Lk) {
+                    lowered(i, bound);
+                } else {
+                    const Key kb = load_key(lb + i);
+                    const int of = (int)(kb.t2 & 0xffffull);
+                    if (kb.s && kb.s <= Lk && (of ? of : k0y) == k) {
+                        if (kb.s == Lk) {
+                            best = kb;
+                            ub[i] = Lk | kEmitted;
+                        } else {
+                            lowered(i, kb.s);
+                        }
+                    } else {
+                        sh.q[atomicAdd(&sh.en, 1)] = i;  // at most the entries read so far
+                    }
+                }
+            }
+            offer(best);
+            __syncthreads();
+        }
+        const int ne = sh.en;
+        for (int w0 = 0; w0 < ne; w0 += kWin) {
+            const int nw = ne - w0 < kWin ? ne - w0 : kWin;
+            const int j = (int)threadIdx.x;
+            if (threadIdx.x == 0) sh.nd = sh.ec = 0;
+            __syncthreads();
+            if (j < nw) {
+                const u32 i = sh.q[w0 + j];
+                Rec &r = sh.rec[j];
+                load_rec(&r, F + front_slot(cap, ft.soff[l], i));
+                const bool dense = is_dense(r.ky, r.kn);
+                int k = 0;
+                if (!dense) {
+                    for (int q = 0; q < (int)r.ky; ++q) {
+                        const int smp = r.ids[q];
+                        if (in_mask(Ush, smp)) r.ids[k++] = (u16)smp;
+                    }
+                    r.ky = (u16)k;
+                }
+                sh.ri[j] = i | (dense ? kDenseBit : 0u);
+                least[2 * j] = ~0u;
+                least[2 * j + 1] = (u32)k;
+                window_tasks<kBig>(c, sh, j, r.p, l, dense);
+            }
+            __syncthreads();
+            window_eval<kBig>(c, s, LevelOut{}, sh, b, Ush, nw, l, Lk, true);
+            Key best = key_empty();
+            if (j < nw) {
+                const u32 i = sh.ri[j] & ~kDenseBit;
+                if (sh.emit[j]) {
+                    int po[kMaxH - 1];
+                    prefix_po(c, sh.rec[j].p, l, po);
+                    best = leaf_key(Lk, po, l, (int)least[2 * j]);
+                    lb[i] = Key{Lk, best.t0, best.t1, best.t2 | (u64)least[2 * j + 1]};
+                    ub[i] = Lk | kEmitted;
+                    next = sh.nb[j] > next ? sh.nb[j] : next;
+                } else {
+                    lowered(i, sh.nb[j]);
+                }
+            }
+            offer(best);
+            __syncthreads();
+        }
+        if (!more) break;
+    }
+    block_level_max(next, sh.wmax, &s.lev->lmax[(step + 1) & 3]);
+    if (warp == 0) {
+        const Key k = warp_max_key(lane < nwarps ? wb[lane] : key_empty());
+        if (lane == 0) s.slots[(size_t)(step & 1) * s.nslots + t.rank] = k;
+    }
+}
 
 // Row words of the tumors that carry all genes of k, lane w: word w.
 __device__ __forceinline__ u64 key_rows(const Cohort &c, const Key &k, int h, int lane)
@@ -925,18 +1156,12 @@ __device__ __forceinline__ void record_pick(const Solve &s, const Key &k, u64 sc
     s.sel[pos] = Key{score, k.t0, k.t1, (k.t2 & kTupleBits) | (u64)tp};
 }
 
-// a_num = 0: one pick, the best member, with every uncovered tumor it covers.
+// One pick: the best of the threads' keys k (score Lk or empty), with every uncovered tumor
+// it covers.  sh.k is the number of picks.
 template <bool kBig>
-__device__ int select_flat(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, u64 *Ush, const Member *mem, int n, u64 Lk,
-                           int K, bool lead)
+__device__ int pick_best(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, u64 *Ush, Key k, u64 Lk, int K, bool lead)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    Key k = key_empty();
-    for (int i = (int)threadIdx.x; i < n; i += (int)blockDim.x) {
-        Key m = member_key(mem + i);
-        m.s = Lk;
-        if (key_better(m, k)) k = m;
-    }
     Key *wk = warp_keys();
     k = warp_max_key(k);
     if (lane == 0) wk[warp] = k;
@@ -957,6 +1182,42 @@ __device__ int select_flat(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, u
     }
     __syncthreads();
     return sh.k;
+}
+
+// a_num = 0: one pick of the members.
+template <bool kBig>
+__device__ int select_flat(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, u64 *Ush, const Member *mem, int n, u64 Lk,
+                           int K, bool lead)
+{
+    Key k = key_empty();
+    for (int i = (int)threadIdx.x; i < n; i += (int)blockDim.x) {
+        Key m = member_key(mem + i);
+        m.s = Lk;
+        if (key_better(m, k)) k = m;
+    }
+    return pick_best<kBig>(c, s, sh, Ush, k, Lk, K, lead);
+}
+
+// One pick from the blocks' slots of level_search_one.
+template <bool kBig>
+__device__ int select_one(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, u64 *Ush, int step, int blocks, u64 Lk, int K,
+                          bool lead)
+{
+    const Key *slots = s.slots + (size_t)(step & 1) * s.nslots;
+    Key k = key_empty();
+    for (int i = (int)threadIdx.x; i < blocks; i += (int)blockDim.x) {
+        Key m;
+        m.s = __ldcg(&slots[i].s);
+        m.t0 = __ldcg(&slots[i].t0);
+        m.t1 = __ldcg(&slots[i].t1);
+        m.t2 = __ldcg(&slots[i].t2);
+        if (key_better(m, k)) k = m;
+    }
+    if (threadIdx.x == 0) sh.k = 0;
+    const int got = pick_best<kBig>(c, s, sh, Ush, k, Lk, K, lead);
+    if (lead && (int)threadIdx.x < c.WTp) s.U[threadIdx.x] = Ush[threadIdx.x];
+    __syncthreads();  // sh.k is free again
+    return got;
 }
 
 // A pool of members (list: their indexes): their tumors as row words on chip (word-major, so
@@ -1379,9 +1640,15 @@ __device__ int select_any(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, Be
     return K1;
 }
 
+// The picks of a band from its n members, by every block on the same input.  U of the block
+// is brought up to date; the lead block (rank 0) records the picks from position K on.
+// Returns their number, or -1 (nothing done) when the top level alone has more than a pool
+// takes and the list is not worth its passes (open: uncovered tumors); fallen: the largest score + 1 that a member
+// left over still has (a listed record's cached leaf takes all its tumors at FP = 0, so that
+// score bounds the record).  Every thread of the block calls it.
 template <bool kBig>
 __device__ int level_select(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, Batch *scratch, u64 *Ush, int n, u64 Lk,
-                            u64 tau, int step, int K, bool lead, u64 &fallen)
+                            u64 tau, int step, int K, bool lead, u64 &fallen, u32 open)
 {
     const Member *mem = s.mem + (size_t)(step & 1) * s.mcap;
     fallen = 0;
@@ -1444,13 +1711,33 @@ __device__ int level_select(const Cohort &c, const Solve &s, LevelSh<kBig> &sh, 
         if (take <= pool && (tau < Lk || take <= 32)) {
             got = take ? select_pool<kBig>(c, s, sh, ps, Ush, mem, take, tau, K, lead, fallen) : 0;
         } else {  // the top level alone (if there are others, their records are looked at again)
-            bool small = kBig && s.h <= 4 && n <= kMany;
-            if (small) {  // the same answer in every block
-                bool ok = true;
-                for (int i = (int)threadIdx.x; i < n; i += T) ok = ok && __ldcg(&mem[i].k) <= 4;
-                small = __syncthreads_and(ok) != 0;
+            // the fewest and the most tumors of a member: the same answers in every block
+            u32 *few = reinterpret_cast<u32 *>(sh.wmax), *most = few + 1;
+            u32 kmin = ~0u, kmax = 0;
+            if (threadIdx.x == 0) {
+                *few = ~0u;
+                *most = 0;
             }
-            if (small) got = select_many<kBig>(c, s, sh, *reinterpret_cast<ManySh *>(scratch), Ush, mem, n, Lk, K, lead, fallen);
+            __syncthreads();
+            for (int i = (int)threadIdx.x; i < n; i += T) {
+                const u32 k = __ldcg(&mem[i].k);
+                kmin = min(kmin, k);
+                kmax = max(kmax, k);
+            }
+            kmin = __reduce_min_sync(kFull, kmin);
+            kmax = __reduce_max_sync(kFull, kmax);
+            if ((threadIdx.x & 31) == 0) {
+                atomicMin(few, kmin);
+                atomicMax(most, kmax);
+            }
+            __syncthreads();
+            kmin = *few;
+            kmax = *most;
+            if ((u32)n > min(s.mlimit, members_worth(open, kmin, kmax > (u32)kMemIds))) {
+                __syncthreads();
+                return -1;
+            }
+            if (kBig && s.h <= 4 && n <= kMany && kmax <= 4) got = select_many<kBig>(c, s, sh, *reinterpret_cast<ManySh *>(scratch), Ush, mem, n, Lk, K, lead, fallen);
             else got = select_any<kBig>(c, s, sh, *reinterpret_cast<BestSh *>(scratch), Ush, mem, n, Lk, K, lead, fallen);
         }
     }

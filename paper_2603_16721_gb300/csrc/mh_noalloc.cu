@@ -15,10 +15,9 @@
 //
 // Every GPU that loads this library keeps the array (kScratchBytes) until the
 // process exits.  The solve is the persistent one (by score levels, as mh_solve's), in the
-// fixed pieces; where one of them is too small for it -- more than kNaLists mutations, a band
-// of more than kNaMembers members, a frontier of shared nodes beyond its region, no room for
-// the cooperative launch -- the rounds run one kernel per phase instead, which needs none of
-// these pieces.  Every call shares the array: calls whose work overlaps on the GPU
+// fixed pieces; where one of them is too small for it -- more than kNaLists mutations, a
+// frontier of shared nodes beyond its region, no room for the cooperative launch -- the rounds
+// run one kernel per phase instead, which needs none of these pieces.  Every call shares the array: calls whose work overlaps on the GPU
 // (different streams, different host threads) race on it and must be
 // serialised by the caller.  What must start at zero is cleared by each call.
 #include <cstdarg>
@@ -46,7 +45,7 @@ constexpr int kNaGW = kNaMaxG / 64;    // 128 words
 constexpr int kNaRounds = kNaMaxNt + 2;
 
 constexpr size_t kNaLists = 1u << 20;        // tumor mutations listed (SL, SLo)
-constexpr u32 kNaMembers = 1u << 16;         // members of a band of score levels
+constexpr u32 kNaMembers = 1u << 16;         // members listed of a band of score levels
 
 constexpr size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -303,7 +302,7 @@ extern "C" MH_API int mh_solve_noalloc(const uint64_t *d_bitmaps, int32_t G, int
     s.ssum = nullptr;
     s.lev = nullptr;
     s.mem = nullptr;
-    s.mcap = 0;
+    s.mcap = s.mlimit = 0;
     s.sel = nullptr;
     s.covsel = nullptr;
     s.cr = nullptr;
@@ -337,7 +336,7 @@ extern "C" MH_API int mh_solve_noalloc(const uint64_t *d_bitmaps, int32_t G, int
     sl.ssum = (u64 *)(base + kOffSsum);
     sl.lev = (Level *)(base + kOffLevel);
     sl.mem = (Member *)(base + kOffMem);
-    sl.mcap = kNaMembers;
+    sl.mcap = sl.mlimit = kNaMembers;  // a level of more is picked one by one
     sl.sel = (Key *)(base + kOffSel);
     sl.covsel = (int *)(base + kOffCovsel);
     sl.cr = (u16 *)(base + kOffCr);

@@ -267,7 +267,8 @@ MH_API int mh_cancel(mh_server *server, uint64_t ticket);
  * the error paths.  spec: "alloc_fail=N" -- the N-th next device allocation of the
  * library fails (MH_ENOMEM); "timeout_after=N" -- the N-th next persistent solve
  * reports MH_ETIMEOUT as if a bounded device wait had expired (after its kernel has
- * run normally); "none" or NULL clears both.  The environment variable MH_FAULT
+ * run normally); "result_fail=N" -- the host memory of the N-th next result cannot be
+ * had (MH_ENOMEM, after its solve); "none" or NULL clears all.  The environment variable MH_FAULT
  * takes the same specs and is read at the first allocation or solve.  Nothing is
  * injected on the device.  Errors: MH_EINVAL (unknown spec). */
 MH_API int mh_set_fault(const char *spec);

@@ -102,9 +102,10 @@ size_t frontier_budget(int dev = -1)
 
 // n elements from the device's pool, ordered on stream st.
 // Host-side fault injection (mh_set_fault, or MH_FAULT in the environment at the
-// first call): the n-th next device allocation fails, or the n-th next solve
-// reports that a bounded device wait expired.  Nothing is injected on the device.
-std::atomic<int> g_fault_alloc{0}, g_fault_timeout{0};
+// first call): the n-th next device allocation fails, the n-th next solve reports
+// that a bounded device wait expired, or the host memory of the n-th next result
+// cannot be had.  Nothing is injected on the device.
+std::atomic<int> g_fault_alloc{0}, g_fault_timeout{0}, g_fault_result{0};
 std::atomic<int> g_fault_env_read{0};
 
 int parse_fault(const char *spec)
@@ -112,6 +113,7 @@ int parse_fault(const char *spec)
     if (!spec || !*spec || !strcmp(spec, "none")) {
         g_fault_alloc = 0;
         g_fault_timeout = 0;
+        g_fault_result = 0;
         return MH_OK;
     }
     int n = 0;
@@ -123,7 +125,11 @@ int parse_fault(const char *spec)
         g_fault_timeout = n;
         return MH_OK;
     }
-    return fail(MH_EINVAL, "fault spec '%s': expected none, alloc_fail=N or timeout_after=N (N >= 1)", spec);
+    if (sscanf(spec, "result_fail=%d", &n) == 1 && n > 0) {
+        g_fault_result = n;
+        return MH_OK;
+    }
+    return fail(MH_EINVAL, "fault spec '%s': expected none, alloc_fail=N, timeout_after=N or result_fail=N (N >= 1)", spec);
 }
 
 // Counts an armed fault down; true when it fires.
@@ -791,7 +797,7 @@ int collect_result(mh_handle *H, int h, bool persistent, double solve_ms, const 
     const int k = hs[0];
     const int rounds = hs[4];
     if (k < 0 || rounds < 0 || rounds > cap || k > cap) return fail(MH_ECUDA, "inconsistent solve state (k=%d, rounds=%d)", k, rounds);
-    mh_result *R = (mh_result *)calloc(1, sizeof(mh_result));
+    mh_result *R = fault_fires(g_fault_result) ? nullptr : (mh_result *)calloc(1, sizeof(mh_result));
     if (!R) return fail(MH_ENOMEM, "host allocation of the result failed");
     R->h = h;
     R->k = k;
@@ -1660,18 +1666,19 @@ extern "C" MH_API int mh_solve_batch(mh_handle *const *handles, const mh_solve_o
         }
     }
     if (rc) return rc;
-    for (int i = 0; i < n; ++i)  // all the copies queued, each on its handle's stream, then the waits
-        if ((rc = queue_result(handles[i]))) {
-            for (int j = 0; j < i; ++j) cudaStreamSynchronize(handles[j]->stream);  // nothing left in flight
-            return rc;
-        }
+    // all the copies are queued, each on its handle's stream, and all are waited for before the
+    // first result is made: whatever fails, no copy is in flight when the call returns (a
+    // handle's pinned buffer goes back to the pool without a wait)
+    int queued = 0;
+    while (queued < n && (rc = queue_result(handles[queued])) == MH_OK) ++queued;
+    for (int i = 0; i < queued; ++i) {
+        if (i > 0 && handles[i]->stream == handles[i - 1]->stream) continue;
+        const cudaError_t e = cudaStreamSynchronize(handles[i]->stream);
+        if (e != cudaSuccess && rc == MH_OK) rc = fail(MH_ECUDA, "reading the result back failed: %s", cudaGetErrorString(e));
+    }
+    if (rc) return rc;
     for (int i = 0; i < n; ++i) {
-        const cudaError_t e = i == 0 || handles[i]->stream != handles[i - 1]->stream
-                                  ? cudaStreamSynchronize(handles[i]->stream)
-                                  : cudaSuccess;
-        rc = e == cudaSuccess
-                 ? collect_result(handles[i], opts[i].h, true, ms, nullptr, 1, 0, &out[i], ms, true)
-                 : fail(MH_ECUDA, "reading the result back failed: %s", cudaGetErrorString(e));
+        rc = collect_result(handles[i], opts[i].h, true, ms, nullptr, 1, 0, &out[i], ms, true);
         if (rc == MH_OK) {
             out[i]->diag[6] = (uint64_t)smm;
             out[i]->diag[7] = (uint64_t)graphed;

@@ -206,7 +206,7 @@ def mh_evaluate(handle: "Handle", genes) -> dict:
 
 
 def mh_set_fault(spec) -> None:
-    """Host-side fault injection: "alloc_fail=N", "timeout_after=N" or None / "none"."""
+    """Host-side fault injection: "alloc_fail=N", "timeout_after=N", "result_fail=N" or None / "none"."""
     lib = load()
     lib.mh_set_fault.restype = ctypes.c_int
     lib.mh_set_fault.argtypes = [ctypes.c_char_p]

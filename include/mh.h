@@ -297,7 +297,8 @@ MH_API void mh_server_destroy(mh_server *server);
  *   stream    : cudaStream_t (NULL = legacy default stream); the call is synchronous.
  * Limits: G <= 8192, Nt <= 1024, Nn <= 1024, 1 <= h <= 4, and at most 2^17
  * prefixes per intermediate depth of the search; larger inputs return MH_EINVAL,
- * a larger frontier MH_ENOMEM, each with a message naming the limit.  Every call
+ * a larger frontier MH_ENOMEM, each with a message naming the limit; a wait of the
+ * solve that ran out returns MH_ETIMEOUT.  Every call
  * looks up the array's device address on the current device (cudaGetSymbolAddress,
  * so calls may span a device reset); the first call on a device also loads the
  * library's device code there, so make it before any CUDA stream capture.  All calls share the array and

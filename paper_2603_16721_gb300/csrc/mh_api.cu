@@ -231,6 +231,12 @@ void pinned_res_put(void *p, size_t bytes)
 
 namespace mh {
 void set_error_text(const char *text) { g_last_error = text; }
+bool injected_timeout() { return fault_fires(g_fault_timeout); }
+int solve_error(int word, const char *timeout_text)
+{
+    if (word == kErrTimeout) return fail(MH_ETIMEOUT, "%s", timeout_text);
+    return fail(MH_ECUDA, "internal error %d: a step of the solve made no progress", word);
+}
 }  // namespace mh
 
 struct mh_handle {
@@ -1010,8 +1016,7 @@ MH_API int mh_solve_ex(mh_handle *H, const mh_solve_opts *opts, mh_result **out)
             kernel_ms += kx;
             if (fault_fires(g_fault_timeout))
                 return fail(MH_ETIMEOUT, "injected timeout (mh_set_fault) after round %d", rounds_done);
-            if (hs[2])
-                return fail(MH_ETIMEOUT, "a grid barrier of the persistent solve timed out in round %d", rounds_done);
+            if (hs[2]) return solve_error(hs[2], "a grid barrier of the persistent solve timed out");
             if (hs[3] == kOverMembers) {  // the band is searched again
                 if ((rc = grow_members(H, &s, st))) return rc;
                 continue;
@@ -1430,7 +1435,7 @@ int run_batch(mh_handle *const *hs, const mh_solve_opts *opts, int n, const std:
         for (int i : act) {
             mh_handle *H = hs[i];
             MH_CUDA(cudaMemcpy(H->hState, H->dState, sizeof(int) * kStateWords, cudaMemcpyDeviceToHost));
-            if (H->hState[2]) return fail(MH_ETIMEOUT, "a team barrier of the batched solve timed out");
+            if (H->hState[2]) return solve_error(H->hState[2], "a team barrier of the batched solve timed out");
             if (H->hState[3] == kOverMembers) {
                 const int rc = grow_members(H, &ss[i], st);
                 if (rc) return rc;
@@ -1495,7 +1500,7 @@ int run_in_turn(mh_handle *const *hs, const mh_solve_opts *opts, int n, double *
     for (int i = 0; i < n; ++i) {
         mh_handle *H = hs[i];
         MH_CUDA(cudaMemcpy(H->hState, H->dState, sizeof(int) * kStateWords, cudaMemcpyDeviceToHost));
-        if (H->hState[2]) return fail(MH_ETIMEOUT, "a grid barrier of the batched solve timed out");
+        if (H->hState[2]) return solve_error(H->hState[2], "a grid barrier of the batched solve timed out");
         if (H->hState[3]) {  // overflowed: grown and solved again from the start
             const int r = H->hState[4];
             int rc = MH_OK;
@@ -1914,7 +1919,7 @@ struct mh_server {
                 cv.notify_all();
                 continue;
             }
-            if (st8[2]) rc = fail(MH_ETIMEOUT, "a team barrier of the served solve timed out");
+            if (st8[2]) rc = solve_error(st8[2], "a team barrier of the served solve timed out");
             if (rc == MH_OK && st8[3] == kOverMembers) {
                 rc = grow_members(H, &r->s, st);
                 if (rc == MH_OK) {

@@ -19,6 +19,7 @@ constexpr int kMaxGenes = 65535;   // gene indices are 16-bit in prefixes and ke
 constexpr int kWarpsPerBlock = 8;
 constexpr int kMaxWarpsPerBlock = 32;
 constexpr int kErrTimeout = 4;     // same value as MH_ETIMEOUT
+constexpr int kErrNoProgress = 8;  // a step of a solve neither picked nor went down: a defect
 constexpr int kThreads = kWarpsPerBlock * 32;
 constexpr int kCountStride = 16;   // u32 slots per counter array (>= kMaxH + 1)
 // Frontier appends are spread over kShards counters, each in its own 128-byte
@@ -313,5 +314,10 @@ cudaError_t launch_barrier_probe(GridSync *g, int *state, cudaStream_t st);
 
 // Message returned by mh_last_error() on the calling thread.
 void set_error_text(const char *text);
+// Whether an injected timeout report (mh_set_fault) is due for the solve at hand.
+bool injected_timeout();
+// The error that a solve left in its state (word 2, not 0), with its message set: MH_ETIMEOUT
+// for a wait that passed its bound, MH_ECUDA for a defect.
+int solve_error(int word, const char *timeout_text);
 
 }  // namespace mh

@@ -2376,7 +2376,7 @@ __device__ __forceinline__ void solve_levels(const Cohort &c, const Solve &s, co
             K += got;
             if (lead && threadIdx.x == 0) s.state[kStK] = K;
             if (got == 0 && Lnext >= Lk) {  // cannot be: a step picks or goes down (no endless loop in any case)
-                if (lead && threadIdx.x == 0) s.state[kStError] = kErrTimeout;
+                if (lead && threadIdx.x == 0) s.state[kStError] = kErrNoProgress;
                 return;
             }
             Lk = Lnext;

@@ -17,7 +17,8 @@
 // process exits.  The solve is the persistent one (by score levels, as mh_solve's), in the
 // fixed pieces; where one of them is too small for it -- more than kNaLists mutations, a
 // frontier of shared nodes beyond its region, no room for the cooperative launch -- the rounds
-// run one kernel per phase instead, which needs none of these pieces.  Every call shares the array: calls whose work overlaps on the GPU
+// run one kernel per phase instead, which needs none of these pieces.  Any other error of the
+// persistent solve is returned.  Every call shares the array: calls whose work overlaps on the GPU
 // (different streams, different host threads) race on it and must be
 // serialised by the caller.  What must start at zero is cleared by each call.
 #include <cstdarg>
@@ -394,18 +395,24 @@ extern "C" MH_API int mh_solve_noalloc(const uint64_t *d_bitmaps, int32_t G, int
     const int pgrid = persistent_grid(num_sms, false);
     if (!done && pgrid > 0 && pgrid <= s.nslots && (size_t)hp[kPrepMutations] <= kNaLists) {
         launch_solve_init(cl, sl, Nt + 2, Nt + 1, counts, kCountSets, st, gsync);
-        if (launch_solve_persistent(cl, sl, fl, gsync, counts, pgrid, false, st) == cudaSuccess) {
+        const cudaError_t le = launch_solve_persistent(cl, sl, fl, gsync, counts, pgrid, false, st);
+        if (le == cudaSuccess) {
             k_na_unpack<<<4, 256, 0, st>>>(s.res, s.state, h, capacity, d_genes, d_tp, d_fp, true);
             NA_CUDA(cudaGetLastError());
             NA_CUDA(cudaMemcpyAsync(st8, s.state, sizeof st8, cudaMemcpyDeviceToHost, st));
             NA_CUDA(cudaStreamSynchronize(st));
-            if (st8[1] && !st8[2] && !st8[3]) {
+            if (injected_timeout()) return na_fail(MH_ETIMEOUT, "injected timeout (mh_set_fault)");
+            if (st8[2]) return solve_error(st8[2], "mh_solve_noalloc: a grid barrier timed out");
+            if (st8[1] && !st8[3]) {
                 *k_out = st8[0];
                 if (rounds_out) *rounds_out = st8[4];
                 return MH_OK;
             }
-        } else {
+        } else if (le == cudaErrorCooperativeLaunchTooLarge || le == cudaErrorLaunchOutOfResources ||
+                   le == cudaErrorMemoryAllocation) {
             cudaGetLastError();  // no room for the grid: one kernel per phase
+        } else {
+            return na_fail(MH_ECUDA, "mh_solve_noalloc: the launch of the solve failed: %s", cudaGetErrorString(le));
         }
     }
     // (over: what ran so far left its state and counts)

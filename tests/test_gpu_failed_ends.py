@@ -1,6 +1,7 @@
 """What a call that fails at its end leaves behind, the failures made on the host: a batch
 that cannot make one of its results leaves no copy in flight into the handles' buffers
-(each handle on a stream of its own), which later handles get again."""
+(each handle on a stream of its own), which later handles get again; the allocation-free
+solve returns the error of its persistent kernel."""
 import numpy as np
 import pytest
 
@@ -48,3 +49,25 @@ def test_batch_without_memory_for_a_result(mh, monkeypatch, at):
             assert got.records() == r.records() and np.array_equal(got.visited, r.visited)
         for H in handles:
             H.close()
+
+
+def test_noalloc_reports_a_timeout(mh):
+    """A bounded wait that ran out is an error here too, not a silent second solve."""
+    import torch
+
+    (bm, G, Nt, Nn), h = _cohorts(1)[0], 3
+    ref = oracle.pdfs(bm, G, Nt, Nn, h)
+    d = torch.from_numpy(bm.view(np.int64)).to("cuda")
+
+    def solve():
+        out = [torch.full((n,), -1, dtype=torch.int32, device="cuda") for n in (Nt * h, Nt, Nt)]
+        k, _ = mh.mh_solve_noalloc(d.data_ptr(), G, Nt, Nn, h, (1, 10), torch.cuda.current_stream().cuda_stream,
+                                   *(x.data_ptr() for x in out), Nt)
+        g, tp, fp = (x.cpu().numpy() for x in out)
+        return [(tuple(g[i * h:(i + 1) * h].tolist()), int(tp[i]), int(fp[i])) for i in range(k)]
+
+    mh.mh_set_fault("timeout_after=1")
+    with pytest.raises(mh.MHError) as e:
+        solve()
+    assert e.value.code == mh.MH_ETIMEOUT
+    assert solve() == ref.records()

@@ -493,7 +493,8 @@ __device__ __forceinline__ void window_tasks(const Cohort &c, LevelSh<kBig> &sh,
 
 // The block's window of nw records spread over its warps: listed records in tasks of 32
 // column words, dense ones in tasks of 32 / cg words, cg the smallest that gives every
-// warp two tasks (a single dense record of 19,000 genes: 38 tasks of 8 words).  Then the
+// warp two tasks (a single dense record of 19,000 genes: 38 tasks of 8 words), and no more
+// words than there are (300 genes: 5 of them, and the samples of a word shared by 4 lanes).  Then the
 // members found, a warp each; or (one) of each record its best leaf of score tau, see
 // EmitList, and the record's |y| beside it.
 template <bool kBig>
@@ -501,8 +502,9 @@ __device__ void window_eval(const Cohort &c, const Solve &s, const LevelOut &o, 
                             int nw, int L, u64 tau, bool one = false)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int words = ((c.G - 1) >> 6) + 1;
     int cg = 1;
-    while (cg < 16 && sh.nd * ((((c.G - 1) >> 6) + 32 / cg) / (32 / cg)) < 2 * nwarps) cg *= 2;
+    while (cg < 16 && (16 / cg >= words || sh.nd * ((((c.G - 1) >> 6) + 32 / cg) / (32 / cg)) < 2 * nwarps)) cg *= 2;
     const int dw = 32 / cg;
     auto ntasks = [&](int j) {
         const int per = sh.ri[j] & kDenseBit ? dw : 32;
@@ -1802,8 +1804,37 @@ struct CountOut {
     }
 };
 
+// Calls add(round, times) for the tumors of y (lane w: word w) but the last-covered one, each at
+// its cover round, equal rounds of a step together (with few rounds most tumors share one: a
+// lane each on one counter is served one after another).  Returns the last cover round (-1: y
+// is empty).
+template <class F>
+__device__ __forceinline__ int cover_rounds(const u16 *cr, u64 y, int lane, F &&add)
+{
+    int mx = -1;
+    auto put = [&](int v) {
+        const unsigned peers = __match_any_sync(kFull, v);
+        if (v >= 0 && lane == __ffs(peers) - 1) add(v, (u32)__popc(peers));
+    };
+    for (u64 x = y; __any_sync(kFull, x != 0); x &= x - 1) {
+        int v = -1;
+        if (x) {
+            const int q = cr[lane * 64 + __ffsll((long long)x) - 1];
+            if (mx >= 0) v = q < mx ? q : mx;
+            mx = q > mx ? q : mx;
+        }
+        put(v);
+    }
+    const int top = (int)__reduce_max_sync(kFull, (unsigned)(mx + 1)) - 1;
+    const int last = __ffs(__ballot_sync(kFull, mx == top)) - 1;
+    put(lane == last ? -1 : mx);
+    return top;
+}
+
 // Chunk `ch` (32 column words) of a dense leaf parent's leaves: its tumors' columns in
-// cover order (ord), 16 loads in flight, the sums of 16 tumors added by 16 lanes together.
+// cover order (ord), 16 loads in flight; the sum of a tumor is added by its lane, or one sum of
+// 16 tumors when they share a round.  The tumors are listed first, 32 places of the order at a
+// time (1536 fit the warp's records; the rest of a longer list follows).
 __device__ __noinline__ void dense_counts(const Cohort &c, const CountOut &out, const u16 *cr, const u16 *ord, Batch &b,
                                           const Prefix &p, int l, int ch)
 {
@@ -1814,45 +1845,57 @@ __device__ __noinline__ void dense_counts(const Cohort &c, const CountOut &out, 
 #pragma unroll
     for (int q = 0; q < kMaxH - 1; ++q)
         if (q < l && lane < c.Wt) y &= __ldg(c.T + (size_t)prefix_gene(p, q) * c.WTp + lane);
+    u16 *ids = reinterpret_cast<u16 *>(b.r);
+    constexpr int kIds = (int)(sizeof(b.r) / sizeof(u16)) & ~15;
     __syncwarp();
     b.ys[lane] = y;
     __syncwarp();
     const bool on = wi <= (c.G - 1) >> 6 && wi >= (lo >> 6);
     const u64 rw = on ? range_word(wi, lo, c.G - 1) : 0ull;
     u64 m = 0;
-    int id = 0, n = 0;  // lane q < n: the q-th tumor waiting
-    auto batch = [&](int k) {  // the first k <= 16 of them
-        u64 x[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            const int smp = __shfl_sync(kFull, id, q);
-            x[q] = on && q < k ? __ldg(c.CT + (size_t)smp * c.GW + wi) & rw : 0ull;
+    int n = 0;  // tumors listed
+    for (int q0 = 0; q0 < c.Nt;) {
+        for (; q0 < c.Nt && n <= kIds - 32; q0 += 32) {
+            const int smp = q0 + lane < c.Nt ? (int)ord[q0 + lane] : -1;
+            const bool in = smp >= 0 && in_mask(b.ys, smp);
+            const unsigned hit = __ballot_sync(kFull, in);
+            if (in) ids[n + __popc(hit & ((1u << lane) - 1u))] = (u16)smp;
+            n += __popc(hit);
         }
-        u32 mine = 0;
+        __syncwarp();
+        const int end = q0 < c.Nt ? n & ~15 : n;  // whole groups of 16 while more are to come
+        for (int i0 = 0; i0 < end; i0 += 16) {
+            const int k = end - i0 < 16 ? end - i0 : 16;
+            u64 x[16];
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            const u32 v = __reduce_add_sync(kFull, (u32)__popcll(x[q] & m));
-            m |= x[q];
-            if (lane == q) mine = v;
+            for (int q = 0; q < 16; ++q) x[q] = on && q < k ? __ldg(c.CT + (size_t)ids[i0 + q] * c.GW + wi) & rw : 0ull;
+            const int first = cr[ids[i0]], last = cr[ids[i0 + k - 1]];
+            if (first == last) {
+                u32 sum = 0;
+#pragma unroll
+                for (int q = 0; q < 16; ++q) {
+                    sum += (u32)__popcll(x[q] & m);
+                    m |= x[q];
+                }
+                sum = __reduce_add_sync(kFull, sum);
+                if (lane == 0 && sum) out.add(first, 2 * l + 1, sum);
+            } else {
+                u32 mine = 0;
+#pragma unroll
+                for (int q = 0; q < 16; ++q) {
+                    const u32 v = __reduce_add_sync(kFull, (u32)__popcll(x[q] & m));
+                    m |= x[q];
+                    if (lane == q) mine = v;
+                }
+                if (lane < k && mine) out.add(cr[ids[i0 + lane]], 2 * l + 1, mine);
+            }
         }
-        if (lane < k && mine) out.add(cr[id], 2 * l + 1, mine);
-        id = __shfl_sync(kFull, id, (lane + k) & 31);
-        n -= k;
-    };
-    for (int q0 = 0; q0 < c.Nt; q0 += 16) {  // the next 16 candidates: lanes 16 .. 31 hold them
-        const int s0 = lane >= 16 && q0 + lane - 16 < c.Nt ? (int)ord[q0 + lane - 16] : -1;
-        const unsigned hit = __ballot_sync(kFull, s0 >= 0 && in_mask(b.ys, s0 < 0 ? 0 : s0));
-        const int k = __popc(hit);
-        if (!k) continue;
-        // append: lane n + i takes the i-th hit
-        const int want = lane - n;
-        const int src = want >= 0 && want < k ? (int)__fns(hit, 0, want + 1) : lane;
-        const int v = __shfl_sync(kFull, s0, src & 31);
-        if (want >= 0 && want < k) id = v;
-        n += k;
-        if (n >= 16) batch(16);
+        __syncwarp();
+        const u16 rest = end + lane < n ? ids[end + lane] : (u16)0;  // fewer than 16
+        __syncwarp();
+        if (end + lane < n) ids[lane] = rest;
+        n -= end;
     }
-    if (n) batch(n);
 }
 
 // The counters of all R rounds from cr: see the head of this file.  Every block adds its
@@ -1889,9 +1932,11 @@ __device__ void level_counts(const Cohort &c, const Solve &s, const Frontiers &f
     // hi(2) - g each in depth 2's correction
     {
         const int last1 = c.G - h, hi2 = c.G - h + 1;
-        for (int g0 = (t.rank * nwarps + warp) * 32; g0 <= last1; g0 += t.size * nwarps * 32) {
-            const int g = g0 + lane;
-            const int k = g <= last1 ? (int)__ldg(&c.GR[g].ky) : 0;
+        const Share sg((u32)(last1 < 0 ? 0 : last1 + 1), (u32)t.size, (u32)nwarps, (u32)t.rank);
+        for (u32 k0 = 0; k0 < sg.steps(); ++k0) {
+            const u32 gi = sg.at(k0, (u32)warp, (u32)lane);
+            const int g = gi < sg.n ? (int)gi : 0;
+            const int k = gi < sg.n ? (int)__ldg(&c.GR[g].ky) : 0;
             if (k >= 1 && k <= kListT) {
                 int mx = -1;
                 for (int q = 0; q < k; ++q) {
@@ -1903,19 +1948,11 @@ __device__ void level_counts(const Cohort &c, const Solve &s, const Frontiers &f
             }
             unsigned many = __ballot_sync(kFull, k > kListT);
             while (many) {
-                const int gd = g0 + __ffs(many) - 1;
+                const int gd = __shfl_sync(kFull, g, __ffs(many) - 1);
                 many &= many - 1;
                 const u64 y = lane < c.Wt ? __ldg(c.T + (size_t)gd * c.WTp + lane) : 0ull;
-                int mx = -1;
-                for (u64 x = y; x; x &= x - 1) {
-                    const int r = cr[lane * 64 + __ffsll((long long)x) - 1];
-                    if (mx >= 0) out.add(r < mx ? r : mx, 2, (u32)(hi2 - gd));
-                    mx = r > mx ? r : mx;
-                }
-                const int top = (int)__reduce_max_sync(kFull, (unsigned)(mx + 1)) - 1;
-                const int lead = __ffs(__ballot_sync(kFull, mx == top)) - 1;
-                if (lane == lead) out.add(top, 1, 1u);
-                else if (mx >= 0) out.add(mx, 2, (u32)(hi2 - gd));
+                const int top = cover_rounds(cr, y, lane, [&](int r, u32 times) { out.add(r, 2, times * (u32)(hi2 - gd)); });
+                if (lane == 0) out.add(top, 1, 1u);
             }
         }
     }
@@ -1962,19 +1999,10 @@ __device__ void level_counts(const Cohort &c, const Solve &s, const Frontiers &f
 #pragma unroll
                     for (int q = 0; q < kMaxH - 1; ++q)
                         if (q < l && lane < c.Wt) y &= __ldg(c.T + (size_t)prefix_gene(p, q) * c.WTp + lane);
-                    int mx = -1;
-                    auto put = [&](int x) {
-                        out.add(x, 2 * (l - 1) + 1, 1u);
-                        out.add(x, 2 * l, wt);
-                    };
-                    for (u64 x = y; x; x &= x - 1) {
-                        const int q = cr[lane * 64 + __ffsll((long long)x) - 1];
-                        if (mx >= 0) put(q < mx ? q : mx);
-                        mx = q > mx ? q : mx;
-                    }
-                    const int top = (int)__reduce_max_sync(kFull, (unsigned)(mx + 1)) - 1;
-                    const int lead = __ffs(__ballot_sync(kFull, mx == top)) - 1;
-                    if (lane != lead && mx >= 0) put(mx);
+                    cover_rounds(cr, y, lane, [&](int r, u32 times) {
+                        out.add(r, 2 * (l - 1) + 1, times);
+                        out.add(r, 2 * l, times * wt);
+                    });
                 }
             if (leafp && dense) {
                 const int p = atomicAdd(&sh.qn, 1);

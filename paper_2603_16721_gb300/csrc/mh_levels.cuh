@@ -1833,7 +1833,7 @@ __device__ __forceinline__ int cover_rounds(const u16 *cr, u64 y, int lane, F &&
 
 // Chunk `ch` (32 column words) of a dense leaf parent's leaves: its tumors' columns in
 // cover order (ord), 16 loads in flight; the sum of a tumor is added by its lane, or one sum of
-// 16 tumors when they share a round.  The tumors are listed first, 32 places of the order at a
+// 16 tumors when they share a round.  The tumors are listed first, 128 places of the order at a
 // time (1536 fit the warp's records; the rest of a longer list follows).
 __device__ __noinline__ void dense_counts(const Cohort &c, const CountOut &out, const u16 *cr, const u16 *ord, Batch &b,
                                           const Prefix &p, int l, int ch)
@@ -1852,23 +1852,36 @@ __device__ __noinline__ void dense_counts(const Cohort &c, const CountOut &out, 
     __syncwarp();
     const bool on = wi <= (c.G - 1) >> 6 && wi >= (lo >> 6);
     const u64 rw = on ? range_word(wi, lo, c.G - 1) : 0ull;
+    // (loads without conditions: a lane beyond the words reads the last one and drops it)
+    const u64 *col = c.CT + min(wi, (c.G - 1) >> 6);
+    const int GW = c.GW;
     u64 m = 0;
     int n = 0;  // tumors listed
-    for (int q0 = 0; q0 < c.Nt;) {
-        for (; q0 < c.Nt && n <= kIds - 32; q0 += 32) {
-            const int smp = q0 + lane < c.Nt ? (int)ord[q0 + lane] : -1;
-            const bool in = smp >= 0 && in_mask(b.ys, smp);
-            const unsigned hit = __ballot_sync(kFull, in);
-            if (in) ids[n + __popc(hit & ((1u << lane) - 1u))] = (u16)smp;
-            n += __popc(hit);
+    const int Nt = c.Nt;
+    for (int q0 = 0; q0 < Nt;) {
+        for (; q0 < Nt && n <= kIds - 128; q0 += 128) {
+            int smp[4];
+            bool in[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) smp[u] = ord[min(q0 + 32 * u + lane, Nt - 1)];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) in[u] = q0 + 32 * u + lane < Nt && in_mask(b.ys, smp[u]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const unsigned hit = __ballot_sync(kFull, in[u]);
+                if (in[u]) ids[n + __popc(hit & ((1u << lane) - 1u))] = (u16)smp[u];
+                n += __popc(hit);
+            }
         }
         __syncwarp();
-        const int end = q0 < c.Nt ? n & ~15 : n;  // whole groups of 16 while more are to come
+        const int end = q0 < Nt ? n & ~15 : n;  // whole groups of 16 while more are to come
         for (int i0 = 0; i0 < end; i0 += 16) {
             const int k = end - i0 < 16 ? end - i0 : 16;
             u64 x[16];
 #pragma unroll
-            for (int q = 0; q < 16; ++q) x[q] = on && q < k ? __ldg(c.CT + (size_t)ids[i0 + q] * c.GW + wi) & rw : 0ull;
+            for (int q = 0; q < 16; ++q) x[q] = __ldg(col + (size_t)ids[i0 + (q < k ? q : 0)] * GW);
+#pragma unroll
+            for (int q = 0; q < 16; ++q) x[q] &= q < k ? rw : 0ull;
             const int first = cr[ids[i0]], last = cr[ids[i0 + k - 1]];
             if (first == last) {
                 u32 sum = 0;
@@ -2103,15 +2116,26 @@ __device__ void level_counts(const Cohort &c, const Solve &s, const Frontiers &f
     __syncthreads();
     const int nq = sh.qn;
     if (nq > 0) {
-        for (int i = (int)threadIdx.x; i < c.Nt; i += (int)blockDim.x) {
-            const int x = cr[i];
-            int pos = 0;
-            for (int j = 0; j < c.Nt; ++j) {
-                const int y = cr[j];
-                pos += (y > x || (y == x && j < i)) ? 1 : 0;
+        // (a counting sort; the order within a round does not matter.  Counting the tumors before
+        // each one took 160 us for 2000.)
+        u32 *bin = reinterpret_cast<u32 *>(&b - warp);  // rounds, in the block's scratch
+        static_assert((kMaxSamples + 1) * sizeof(u32) <= kWarpsPerBlock * sizeof(Batch), "a word per round");
+        for (int r = (int)threadIdx.x; r < R; r += (int)blockDim.x) bin[r] = 0;
+        __syncthreads();
+        for (int i = (int)threadIdx.x; i < c.Nt; i += (int)blockDim.x) atomicAdd(&bin[cr[i]], 1u);
+        __syncthreads();
+        if (warp == 0) {
+            u32 later = 0;  // tumors of the later rounds
+            for (int top = R; top > 0; top -= 32) {
+                const int r = top - 1 - lane;
+                const u32 x = r >= 0 ? bin[r] : 0u;
+                const u32 inc = (u32)warp_incl_scan((int)x, lane);
+                if (r >= 0) bin[r] = later + inc - x;
+                later += __shfl_sync(kFull, inc, 31);
             }
-            sh.ord[pos] = (u16)i;
         }
+        __syncthreads();
+        for (int i = (int)threadIdx.x; i < c.Nt; i += (int)blockDim.x) sh.ord[atomicAdd(&bin[cr[i]], 1u)] = (u16)i;
         __syncthreads();
         const int l = h - 1, nchunk = (((c.G - 1) >> 6) + 1 + 31) >> 5;
         if (nq <= LevelSh<kBig>::kQ) {

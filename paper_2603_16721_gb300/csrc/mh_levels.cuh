@@ -702,7 +702,8 @@ __device__ void level_tally(const Solve &s, const Frontiers &f, LevelSh<kBig> &s
     Tally ty;
     for (u32 k = 0; k < sr.steps(); ++k) {
         const u32 i = sr.at(k, (u32)warp, (u32)lane);
-        if (i < sr.n) ty.add(Lk, s.a_num, __ldcg(ub + i));
+        const u64 v = i < sr.n ? __ldcg(ub + i) : 0ull;
+        if (v) ty.add(Lk, s.a_num, v);  // (0: no leaf left)
         if ((k & 63u) == 63u) ty.flush(sh.tally);
     }
     ty.flush(sh.tally);

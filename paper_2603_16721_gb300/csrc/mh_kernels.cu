@@ -1066,10 +1066,14 @@ __device__ bool phase_expand(const Cohort &c, const Solve &s, int round, int lev
     u64 leaf_vis = 0, leaf_alive = 0;  // closed-form leaves of single-sample children (level = h - 1)
     u64 *deep = acc + kAccDeep;
     const int h = s.h;
-    // With pruning off and fewer records than the warps' batches hold, a task is 32 children of
-    // a record, from the rows: at G = 300 the 298 depth-1 records kept 298 of 2432 warps busy
-    // with up to 298 children each (32 us per round; 9 us spread over all of them).
-    const bool by_children = all_children && (u64)count < (u64)kBatch * nw;
+    // With pruning off a task is 32 children of a record, from the rows, where whole records
+    // keep few warps busy: at G = 300 the 298 depth-1 records kept 298 of 2432 warps busy with
+    // up to 298 children each (34 us per round; 11 us spread over all of them).  The line: depth-1
+    // parents up to as many as the warps' batches hold (by records / by children, us per
+    // round, three hits: G = 1200 114 / 55, 5000 658 / 492), deeper ones, whose children come
+    // cheaper from the lists, when there are fewer than warps (all depths by children / as
+    // here: four hits G = 300 310 / 225, five hits G = 60 85 / 54).
+    const bool by_children = all_children && (u64)count < (level == 2 ? (u64)kBatch * nw : nw);
     if (by_children) {
         const u32 nch = (u32)(c.G + 31) / 32;
         for (u64 x = gw; x < (u64)count * nch; x += nw) {

@@ -370,7 +370,7 @@ int build_store(mh_handle *H, const uint64_t *bm, bool sync = true)
     const size_t oCC = piece((size_t)Nt * (c.GW + 1) * sizeof(u16)), oSL = piece(nSL * sizeof(u16));
     const size_t oSLo = piece(nSL * sizeof(u16)), oSO = piece(SO.size() * sizeof(u32));
     const size_t oOrig = piece((size_t)G * sizeof(u16)), oInv = piece((size_t)G * sizeof(u32));
-    const size_t oGR = piece((size_t)G * sizeof(Rec)), oGS = piece((size_t)G * sizeof(u64));
+    const size_t oGR = piece((size_t)G * sizeof(Rec));
     const size_t oTO = piece(rowsT * sizeof(u64)), oNO = piece(rowsN * sizeof(u64));
     // scratch for the build: the rows as given, the permutation, the original-order
     // sample-major copy (freed in stream order after the build)
@@ -408,7 +408,6 @@ int build_store(mh_handle *H, const uint64_t *bm, bool sync = true)
     c.SO = H->dSO;
     c.SLo = H->dSLo;
     c.GR = (const Rec *)(H->dStore + oGR);
-    c.GS = (const u64 *)(H->dStore + oGS);
     c.TO = (const u64 *)(H->dStore + oTO);
     c.NO = (const u64 *)(H->dStore + oNO);
     StoreBuild b;
@@ -423,7 +422,6 @@ int build_store(mh_handle *H, const uint64_t *bm, bool sync = true)
     b.CTo = (u64 *)(scratch + tCTo);
     b.CC = H->dCC; b.SL = H->dSL; b.SLo = H->dSLo; b.orig = H->dOrig; b.inv = H->dInv;
     b.GR = (Rec *)(H->dStore + oGR);
-    b.GS = (u64 *)(H->dStore + oGS);
     MH_CUDA(launch_store_build(b, st));
     dfree(scratch, st);
     if (sync) MH_CUDA(cudaStreamSynchronize(st));  // build errors surface here

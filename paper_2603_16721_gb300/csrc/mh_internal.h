@@ -60,8 +60,6 @@ struct Cohort {
     // samples listed when few (see Rec).  A round filters the listed tumors by U.
     // nullptr: depth-1 records are built from the rows.
     const Rec *GR;
-    // G static tumor signatures: OR of 1 << (s & 63) over the tumors of each gene.
-    const u64 *GS;
     // The rows again in the caller's (original) gene order, G x WTp and G x WNp: a
     // key's genes read without the search-position lookup.  nullptr: use inv.
     const u64 *TO, *NO;
@@ -105,7 +103,6 @@ struct StoreBuild {
     u16 *CC, *SL, *SLo, *orig;
     u32 *inv;
     Rec *GR;
-    u64 *GS;
 };
 
 // A combination of the band being resolved: its tuple (as in Key; FP and TP in the low

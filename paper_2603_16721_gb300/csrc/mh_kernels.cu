@@ -55,9 +55,8 @@ __device__ __forceinline__ Team grid_team() { return Team{(int)blockIdx.x, (int)
 // rows and the block's copy of U (Ush), bests stored into the round's slot array,
 // the round's threshold word, diagnostics by round parity.
 // fm: the solve by score levels (see "Counting by per-sample sums" below and
-// mh_levels.cuh): only nodes shared by two or more tumors are built; build: the
-// expansion builds the kept frontiers and adds no counters (they follow from the kept
-// nodes after the last level).
+// mh_levels.cuh): the expansion builds the kept frontiers, only nodes shared by two or
+// more tumors, and adds no counters (they follow from the kept nodes after the last level).
 struct RoundIO {
     const u64 *Ush;
     Key *slots;
@@ -65,12 +64,11 @@ struct RoundIO {
     u64 *hint;
     int par;
     bool fm;
-    bool build;
     const u64 *thr;  // score-bound mode: the block's own lower bound on the round's best score
 };
 __device__ __forceinline__ RoundIO launch_io(const Solve &s)
 {
-    return RoundIO{nullptr, s.slots, false, s.best_hint, 0, false, false, nullptr};
+    return RoundIO{nullptr, s.slots, false, s.best_hint, 0, false, nullptr};
 }
 
 __device__ __forceinline__ int prefix_gene(const Prefix &p, int i)
@@ -605,25 +603,12 @@ __device__ __forceinline__ int batch_prepare(const Cohort &c, const RoundIO &io,
     }
     if (valid && fm) {
         // counting by per-sample sums: a node shared by fewer than two uncovered
-        // tumors is accounted for by those sums (nothing to search below it); a
-        // shared one adds (|y| - 1) x (its children) to the depth's correction
+        // tumors is accounted for by those sums (nothing to build below it)
         lo = prefix_gene(b.r[lane].p, L - 1) + 1;
         hi = hi_bound;
         ky = b.r[lane].ky;
         kn = b.r[lane].kn;
         if (ky < 2) hi = lo - 1;
-        else if (hi >= lo) visited += (u64)(ky - 1) * (u64)(hi - lo + 1);
-        if (orig && hi >= lo) {  // ascending original indices of the prefix genes (leaf keys)
-            for (int q = 0; q < L; ++q) {
-                const u16 v = orig[prefix_gene(b.r[lane].p, q)];
-                int k = q - 1;
-                while (k >= 0 && b.po[lane][k] > v) {
-                    b.po[lane][k + 1] = b.po[lane][k];
-                    --k;
-                }
-                b.po[lane][k + 1] = v;
-            }
-        }
     } else if (valid) {
         lo = prefix_gene(b.r[lane].p, L - 1) + 1;
         hi = hi_bound;
@@ -726,18 +711,13 @@ __device__ __forceinline__ void sibling_items(const Cohort &c, const Batch &b, i
     for (int u = 0; u < kIlp; ++u) m[u] &= rw[u];
 }
 
-// The same sibling test counting how many samples have each sibling: m = the
-// siblings of at least one sample (non-empty children), m2 = of at least two
-// (children shared by two or more uncovered tumors); with SUM, sum[u] = the
-// number of (sample, sibling) pairs in the range word (the children's sizes
-// summed).
-template <bool SUM>
+// The same sibling test for the siblings of at least two samples (m2: the children
+// shared by two or more uncovered tumors).
 __device__ __forceinline__ void sibling_items2(const Cohort &c, const Batch &b, int t0, int total, int &j,
-                                               int (&jj)[kIlp], int (&wi)[kIlp], int (&ky)[kIlp], u64 (&m)[kIlp],
-                                               u64 (&m2)[kIlp], int (&sum)[kIlp])
+                                               int (&jj)[kIlp], int (&wi)[kIlp], int (&ky)[kIlp], u64 (&m2)[kIlp])
 {
     int kmax = 0;
-    u64 rw[kIlp];
+    u64 rw[kIlp], m[kIlp];
 #pragma unroll
     for (int u = 0; u < kIlp; ++u) {
         const int t = t0 + 32 * u;
@@ -746,7 +726,6 @@ __device__ __forceinline__ void sibling_items2(const Cohort &c, const Batch &b, 
         rw[u] = 0;
         m[u] = 0;
         m2[u] = 0;
-        sum[u] = 0;
         if (t < total) {
             while (t >= b.off[j + 1]) ++j;
             wi[u] = (b.lo[j] >> 6) + (t - b.off[j]);
@@ -768,7 +747,6 @@ __device__ __forceinline__ void sibling_items2(const Cohort &c, const Batch &b, 
             const u64 a = x0[u] & rw[u], e = x1[u] & rw[u];
             m2[u] |= (m[u] & (a | e)) | (a & e);
             m[u] |= a | e;
-            if (SUM) sum[u] += __popcll(a) + __popcll(e);
         }
     }
 }
@@ -1132,9 +1110,7 @@ __device__ bool phase_expand(const Cohort &c, const Solve &s, int round, int lev
             u64 m[kIlp], rw[kIlp];
             if (fm) {
                 // children shared by two or more uncovered tumors only
-                u64 m1[kIlp];
-                int sum[kIlp];
-                sibling_items2<false>(c, b, tb + lane, total, j, jj, wi, ky, m1, m, sum);
+                sibling_items2(c, b, tb + lane, total, j, jj, wi, ky, m);
             } else {
                 sibling_items(c, b, tb + lane, total, j, jj, wi, ky, m, rw);
 #pragma unroll
@@ -1174,7 +1150,6 @@ __device__ bool phase_expand(const Cohort &c, const Solve &s, int round, int lev
                         child.pad[0] = child.pad[1] = child.pad[2] = 0;
                         child_tumors(c, parent, L, (int)(u32)jw, g & 63, child);
                         emit = true;
-                        if (fm) alive += (u64)(child.ky - 1);  // the depth's correction
                         // a child of a listed parent is listed: one sample -> closed form
                         if (single && child.ky == 1 && single_sample_closed(single, s.champ_ok, child.ids[0])) {
                             single_sample_count(c, h, level, g, child.ids[0], leaf_vis, leaf_alive, deep);
@@ -1213,7 +1188,6 @@ __device__ bool phase_expand(const Cohort &c, const Solve &s, int round, int lev
                 bool closed = false;
                 if (fm) {
                     closed = kyc < 2;  // single-sample children: in the per-sample sums
-                    if (!closed) alive += (u64)(kyc - 1);
                 } else {
                     alive += (u64)(kyc > 0);
                     if (single && kyc == 1 && g <= hi && single_sample_closed(single, s.champ_ok, smp)) {
@@ -1242,9 +1216,8 @@ __device__ bool phase_expand(const Cohort &c, const Solve &s, int round, int lev
     d1.visited = warp_sum_u64(d1.visited);
     d1.pruned = warp_sum_u64(d1.pruned);
     if (lane == 0) {
-        // fm: the depth's corrections (visited, surviving), finished at the end of the round
         acc_add(acc, 0, visited);
-        acc_add(acc, 1, fm ? alive : visited - alive);
+        acc_add(acc, 1, visited - alive);
         acc_add(acc, 8, d1.visited);
         acc_add(acc, 9, d1.pruned);
         acc_add(deep, 2 * h, leaf_vis);
@@ -1252,7 +1225,7 @@ __device__ bool phase_expand(const Cohort &c, const Solve &s, int round, int lev
     }
     warp_cycles(acc, t0, lane);
     __syncthreads();
-    if (!io.build) {
+    if (!fm) {
         if (threadIdx.x < 2 && acc[threadIdx.x])
             atomicAdd(s.cnt + ((size_t)round * s.h + (level - 1)) * 2 + threadIdx.x, acc[threadIdx.x]);
         if (threadIdx.x >= 8 && threadIdx.x < 10 && acc[threadIdx.x])
@@ -2226,17 +2199,6 @@ __device__ bool end_of_round(const Cohort &c, const Solve &s, int round, const K
     return done;
 }
 
-// The greedy loop of one cohort run by a team of co-resident blocks.  Where every
-// tumor's champion is known the solve goes by score levels (solve_levels); otherwise a
-// round is the depth-2 .. h-1 expansions (depth 1 built on the fly from the gene rows),
-// the leaves, a barrier, and the end of round computed redundantly by every block, so
-// rounds are separated by h - 1 barriers.  Data indexed by round parity: the slots the
-// blocks' bests go to, the frontier counters and the threshold word; rank 0 clears the
-// next round's set at the start of a round (all reads of it ended before the previous
-// round's last barrier).  Returns when the solve is done, a frontier overflowed, a
-// barrier timed out (recorded in the cohort's state) or, in a batch, the barrier that
-// ended a round carried a yield request.
-
 // The time since `tm` goes to a phase's total (block 0, thread 0).
 struct PhaseTimer {
     bool on;
@@ -2252,7 +2214,7 @@ struct PhaseTimer {
 };
 
 // The solve by score levels (mh_levels.cuh): the kept frontiers are built and every leaf
-// parent is evaluated once; then one grid barrier per level, the members of the level
+// parent is evaluated once; then one grid barrier per band, the members of the band
 // gathered before it and its picks made after it by every block alike; then the rounds
 // and their counters.  A launch may end between two levels (a yield request, or members
 // that outgrew their buffer, the level then being searched again): s.state holds the
@@ -2281,7 +2243,7 @@ __device__ __forceinline__ void solve_levels(const Cohort &c, const Solve &s, co
     const int step0 = *(volatile int *)&s.state[kStStep] & ~kOneStep;
     bool one = (*(volatile int *)&s.state[kStStep] & kOneStep) != 0;
     if (step0 == 0) {
-        const RoundIO io{Ush, s.slots, true, s.best_hint, 0, true, true, nullptr};
+        const RoundIO io{Ush, s.slots, true, s.best_hint, 0, true, nullptr};
         if (h == 2) {
             phase_build1(c, s, f, counts, b, t, Ush);
             if (!grid_sync(gsync, s.state, t.size)) return;
@@ -2413,6 +2375,16 @@ __device__ __forceinline__ void solve_levels(const Cohort &c, const Solve &s, co
     pt.lap(s, 3);
 }
 
+// The greedy loop of one cohort run by a team of co-resident blocks.  Where every
+// tumor's champion is known the solve goes by score levels (solve_levels); otherwise a
+// round is the depth-2 .. h-1 expansions (depth 1 built on the fly from the gene rows),
+// the leaves, a barrier, and the end of round computed redundantly by every block, so
+// rounds are separated by h - 1 barriers.  Data indexed by round parity: the slots the
+// blocks' bests go to, the frontier counters and the threshold word; rank 0 clears the
+// next round's set at the start of a round (all reads of it ended before the previous
+// round's last barrier).  Returns when the solve is done, a frontier overflowed, a
+// barrier timed out (recorded in the cohort's state) or, in a batch, the barrier that
+// ended a round carried a yield request.
 // (Forced in line, and solve_levels with it: when the kernel grew past the compiler's limit and
 // solve_team became a function, its arguments, kernel parameters before, were read through
 // pointers: 5000 genes, 500 + 300 samples, three hits 537 us to 605, with the score bound
@@ -2472,7 +2444,7 @@ __device__ __forceinline__ void solve_team(const Cohort &c, const Solve &s, cons
     for (;;) {
         const int par = round & 1;
         u32 *counts = counts_base + (size_t)par * kCountWords;
-        const RoundIO io{Ush, s.slots + (size_t)par * s.nslots, true, s.best_hint + par, par, false, false,
+        const RoundIO io{Ush, s.slots + (size_t)par * s.nslots, true, s.best_hint + par, par, false,
                          bound ? &thr_sh : nullptr};
         if (t.rank == 0) {  // the next round's counters and threshold start from zero
             u32 *cn = counts_base + (size_t)(par ^ 1) * kCountWords;
@@ -2752,13 +2724,13 @@ int batch_blocks_per_sm(int build)
     static std::atomic<int> cache[3][kMaxDev];
     return blocks_per_sm(cache[build == 1 ? 0 : (build == 3 ? 1 : 2)], [&] {
         int per_sm = 0;
-    const cudaError_t e =
-        build == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_batch<1, kSmallWarps>,
-                                                                   kSmallWarps * 32, 0)
-        : build == 3 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_batch<3, kWarpsPerBlock>,
-                                                                     kThreads, 0)
-                     : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_batch<4, kWarpsPerBlock>,
-                                                                     kThreads, 0);
+        const cudaError_t e =
+            build == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_batch<1, kSmallWarps>,
+                                                                       kSmallWarps * 32, 0)
+            : build == 3 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_batch<3, kWarpsPerBlock>,
+                                                                         kThreads, 0)
+                         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_batch<4, kWarpsPerBlock>,
+                                                                         kThreads, 0);
         if (e != cudaSuccess) return 0;
         return build == 1 ? (per_sm >= 1 ? 1 : 0) : per_sm;
     });

@@ -63,8 +63,7 @@ constexpr size_t kOffSL = kOffCC + align256(sizeof(u16) * kNaMaxNt * (kNaGW + 1)
 constexpr size_t kOffSLo = kOffSL + align256(sizeof(u16) * kNaLists);
 constexpr size_t kOffSO = kOffSLo + align256(sizeof(u16) * kNaLists);
 constexpr size_t kOffGR = kOffSO + align256(sizeof(u32) * (kNaMaxNt + 1));
-constexpr size_t kOffGS = kOffGR + align256(sizeof(Rec) * kNaMaxG);
-constexpr size_t kOffOrig = kOffGS + align256(sizeof(u64) * kNaMaxG);
+constexpr size_t kOffOrig = kOffGR + align256(sizeof(Rec) * kNaMaxG);
 constexpr size_t kOffInv = kOffOrig + align256(sizeof(u16) * kNaMaxG);
 constexpr size_t kOffKeys = kOffInv + align256(sizeof(u32) * kNaMaxG);
 constexpr size_t kOffOrder = kOffKeys + align256(sizeof(u32) * kNaMaxG);
@@ -271,19 +270,17 @@ extern "C" MH_API int mh_solve_noalloc(const uint64_t *d_bitmaps, int32_t G, int
     u16 *orig = (u16 *)(base + kOffOrig);
     u32 *inv = (u32 *)(base + kOffInv);
     Rec *GR = (Rec *)(base + kOffGR);
-    u64 *GS = (u64 *)(base + kOffGS);
     c.T = T; c.N = N; c.CT = CT; c.CN = CN; c.orig = orig; c.inv = inv;
     c.CC = nullptr;  // one kernel per phase: no running-count table, every subtree is searched
     c.SL = nullptr;
     c.SO = nullptr;
     c.SLo = nullptr;
     c.GR = nullptr;
-    c.GS = nullptr;
     c.TO = nullptr;
     c.NO = nullptr;
     Cohort cl = c;  // by levels: the whole store
     cl.CC = Nt ? CC : nullptr;
-    cl.SL = SL; cl.SO = SO; cl.SLo = SLo; cl.GR = GR; cl.GS = GS; cl.TO = TO; cl.NO = NO;
+    cl.SL = SL; cl.SO = SO; cl.SLo = SLo; cl.GR = GR; cl.TO = TO; cl.NO = NO;
 
     Solve s;
     s.h = h;
@@ -363,7 +360,7 @@ extern "C" MH_API int mh_solve_noalloc(const uint64_t *d_bitmaps, int32_t G, int
     sb.T = T; sb.N = N; sb.TO = TO; sb.NO = NO; sb.CT = CT; sb.CN = CN;
     sb.CTo = (u64 *)(base + kOffCTo);
     sb.CC = CC; sb.SL = SL; sb.SLo = SLo; sb.orig = orig; sb.inv = inv;
-    sb.GR = GR; sb.GS = GS;
+    sb.GR = GR;
     NA_CUDA(launch_store_build(sb, st));
     // the first round's frontiers decide whether the solve fits (U only shrinks: later
     // ones are smaller)

@@ -80,8 +80,8 @@ __global__ void k_store_lists(const u64 *CT, const u64 *CTo, int Nt, int GW, con
 }
 
 // Static depth-1 record of every gene (search order): all its tumors and normals,
-// listed when few, and its tumor signature.  One thread per gene.
-__global__ void k_store_records(const u64 *T, const u64 *N, int G, int Wt, int Wn, int WTp, int WNp, Rec *GR, u64 *GS)
+// listed when few.  One thread per gene.
+__global__ void k_store_records(const u64 *T, const u64 *N, int G, int Wt, int Wn, int WTp, int WNp, Rec *GR)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= G) return;
@@ -92,11 +92,7 @@ __global__ void k_store_records(const u64 *T, const u64 *N, int G, int Wt, int W
     r.pad[0] = r.pad[1] = r.pad[2] = 0;
     const u64 *trow = T + (size_t)i * WTp, *nrow = N + (size_t)i * WNp;
     int ky = 0, kn = 0;
-    u64 sig = 0;
-    for (int w = 0; w < Wt; ++w) {
-        ky += __popcll(trow[w]);
-        sig |= trow[w];
-    }
+    for (int w = 0; w < Wt; ++w) ky += __popcll(trow[w]);
     for (int w = 0; w < Wn; ++w) kn += __popcll(nrow[w]);
     r.ky = (u16)(ky < 0xffff ? ky : 0xffff);
     r.kn = (u16)(kn < 0xffff ? kn : 0xffff);
@@ -111,7 +107,6 @@ __global__ void k_store_records(const u64 *T, const u64 *N, int G, int Wt, int W
             for (u64 y = nrow[w]; y; y &= y - 1) r.ids[k++] = (u16)(w * 64 + __ffsll((long long)y) - 1);
     }
     GR[i] = r;
-    GS[i] = sig;
 }
 
 }  // namespace
@@ -131,7 +126,7 @@ cudaError_t launch_store_build(const StoreBuild &b, cudaStream_t st)
     if (c.Nn > 0) launch_transpose(c, b.N, c.WNp, c.Nn, b.CN, st);
     if (c.Nt > 0)
         k_store_lists<<<(c.Nt + 3) / 4, 128, 0, st>>>(b.CT, b.CTo, c.Nt, c.GW, b.SO, b.CC, b.SL, b.SLo);
-    if (c.G > 0) k_store_records<<<(c.G + 127) / 128, 128, 0, st>>>(b.T, b.N, c.G, c.Wt, c.Wn, c.WTp, c.WNp, b.GR, b.GS);
+    if (c.G > 0) k_store_records<<<(c.G + 127) / 128, 128, 0, st>>>(b.T, b.N, c.G, c.Wt, c.Wn, c.WTp, c.WNp, b.GR);
     return cudaGetLastError();
 }
 

@@ -138,14 +138,22 @@ def algorithmic_ops(r, Nt, Nn):
     return visited_all * (wt + 1) + scored * per_scored, visited_leaf * (wt + 1) + scored * per_scored
 
 
+def kernel_source_sha256():
+    """Of the files that the solve kernel is made of, one after another."""
+    import hashlib
+    sha = hashlib.sha256()
+    for name in ("mh_kernels.cu", "mh_levels.cuh", "mh_barrier.h", "mh_internal.h"):
+        with open(os.path.join(ROOT, "paper_2603_16721_gb300", "csrc", name), "rb") as f:
+            sha.update(f.read())
+    return sha.hexdigest()
+
+
 def _profiled_fields(kernel_file="k_solve_c2.md"):
     """Fields of the committed ncu summary of the solve kernel ("- `key`: `value`"
     lines), if that summary was taken from the kernel source as it is now (else {})."""
-    import hashlib
-    src = os.path.join(ROOT, "paper_2603_16721_gb300", "csrc", "mh_kernels.cu")
     try:
         text = open(os.path.join(ROOT, "profiles", kernel_file)).read()
-        sha = hashlib.sha256(open(src, "rb").read()).hexdigest()
+        sha = kernel_source_sha256()
     except OSError:
         return {}
     fields = {k: v.strip("`") for k, v in (ln.strip("- `").split(": ", 1) for ln in text.splitlines()

@@ -8,13 +8,14 @@
 // best member by key is picked, the members' scores follow from their tumors still in U,
 // and so on until the best is below tau, which is where the next band starts.  A band is one
 // pass over the kept leaf parents whose bound reaches tau and one grid barrier; its picks are
-// made by every block alike.  A solve has 7 to 20 bands where it has 50 to 700 rounds, and
-// each of these used to cost a chain of about 10 us (scan, re-evaluation, grid barrier, slot
-// reduction, winner rows).  tau is chosen so that the bounds that reach it are few (about
-// one record per block to evaluate); where a single level already has more (the last ones:
+// made by every block alike.  A solve has 1 to 12 bands where it has 12 to 740 rounds (15 to
+// 23 bands with rows too dense to list), and each round used to cost a chain of about 10 us
+// (scan, re-evaluation, grid barrier, slot reduction, winner rows).  tau is chosen so that at
+// most 64 bounds per block reach it; where a single level already has more (the last ones:
 // thousands of combinations of two or three tumors), the band is that level.  Its rounds are
 // then the lexicographically first set of pairwise disjoint intersections among the members,
-// since a member that meets a pick has fallen below the level for good.
+// since a member that meets a pick has fallen below the level for good.  A level with more
+// members than are worth a list (see members_worth) is picked one member a step.
 //
 // The counters of every round (visited and pruned nodes per depth) do not depend on
 // how the winners were found, only on the round cr(s) in which each tumor is covered:
@@ -952,11 +953,16 @@ __device__ __forceinline__ u32 level_worth(const Cohort &c, const Solve &s, u64 
     return min(s.mlimit, members_worth(left, (u32)tp, tp > kMemIds));
 }
 
+// (Both sides, ms of a solve, by lists of any length / as here: 60 groups of 14 tumors that
+// share 100 genes, three hits, 9.7 million members 204 / 5.1; 20 groups of 30 tumors, 3.2 million
+// of unlisted tumors 1666 / 4.7; 60 genes in all of 64 tumors, four hits, 0.5 million 403 / 2.4;
+// 95 pairs sharing 200 genes, two hits 24 / 1.9, 17 us a pick.)
+
 // A step of a level with more members than are worth a list: the best member of the block's
-// share (score Lk, the smallest tuple) goes to the block's slot.  A record's best leaf is kept in lb with the number of the record's tumors in U, and
-// is valid while that many are left (U only shrinks), so a step evaluates only the
-// records that the last picks touched; the others are read from lb.  Every thread of the block
-// calls it; a grid barrier follows.
+// share (score Lk, the smallest tuple) goes to the block's slot.  A record's best leaf is kept
+// in lb with the number of the record's tumors in U, and is valid while that many are left (U
+// only shrinks), so a step evaluates only the records that the last picks touched; the others
+// are read from lb.  Every thread of the block calls it; a grid barrier follows.
 template <bool kBig>
 __device__ __noinline__ void level_search_one(const Cohort &c, const Solve &s, const Rec *F, u32 cap, u64 *ub, Key *lb,
                                               LevelSh<kBig> &sh, Batch &b, const Team &t, const FrontTab &ft,
@@ -1835,7 +1841,11 @@ __device__ __forceinline__ int cover_rounds(const u16 *cr, u64 y, int lane, F &&
 // Chunk `ch` (32 column words) of a dense leaf parent's leaves: its tumors' columns in
 // cover order (ord), 16 loads in flight; the sum of a tumor is added by its lane, or one sum of
 // 16 tumors when they share a round.  The tumors are listed first, 128 places of the order at a
-// time (1536 fit the warp's records; the rest of a longer list follows).
+// time (1536 fit the warp's records; the rest of a longer list follows).  Bound by latency: a
+// warp takes 1.4 us a group of 16 (the column words from L2) and 0.7 us to list 128 places.  All
+// counters of 1000 genes, 500 tumors at 0.1, two hits, one round: 282 us with tumors shifted
+// into place 16 at a time, depth 1 by 32 genes a warp and the order by counting predecessors, 58
+// now; 200 genes, 2000 tumors at 0.2, three hits 927 -> 376.
 __device__ __noinline__ void dense_counts(const Cohort &c, const CountOut &out, const u16 *cr, const u16 *ord, Batch &b,
                                           const Prefix &p, int l, int ch)
 {
